@@ -45,6 +45,10 @@ def main():
              f"#define OG_SR_POLY_INV_HALF {1.0 / HALF!r}",
              "__constant__ float og_sr_poly[OG_SR_POLY_DEG + 1] = {"]
     lines += [f"    {float(np.float32(v))!r}f," for v in c]
+    lines += ["};",
+              "// each coefficient twice, for packed (two-lane) evaluation",
+              "__constant__ float2 og_sr_poly2[OG_SR_POLY_DEG + 1] = {"]
+    lines += [f"    {{{float(np.float32(v))!r}f, {float(np.float32(v))!r}f}}," for v in c]
     lines += ["};", ""]
     with open(os.path.join(here, "short_range_poly.inc"), "w") as f:
         f.write("\n".join(lines))

@@ -12,18 +12,26 @@
 // exactly the terms of its own per-particle walk (the rules are listed in
 // og.h), while node data is read once per warp.
 //
-// Evaluation.  Queued entries are expanded into source slots; a source
-// beyond r_cut of the group box is dropped and the others are staged in a
-// ring of two 32-slot batches.  For a batch, a cheap conservative test
-// (|x_i|^2 + |x_j|^2 - 2 x_i.x_j against r_cut^2, with a per-slot rounding
-// margin) marks the (target, source) pairs that can lie inside the cut; the
-// marked pairs are compacted into a target-major list by a warp prefix sum,
-// and each warp iteration evaluates 32 listed pairs.  A segmented scan over
-// the lanes sums each target's run in a fixed order, so the result does not
-// depend on scheduling.  In the adjoint, the lane that owns a slot sums that
-// source's terms over the iteration's lanes in lane order (their lanes are
-// found through a shared-memory bit mask per slot).  The FP64 variant shares
-// all of this with FP64 decisions and pair arithmetic.
+// Evaluation.  Queued entries are expanded into source slots, 32 at a time
+// (fetched by cp.async while the previous ones are evaluated); a source
+// beyond r_cut of the group box is dropped and the others are staged, up to
+// 64 for a batch.  In the FP32 walks a batch is evaluated by tiles of 8
+// targets x 8 sources: each of the group's four sub-groups of 8 lists the
+// pairs of adjacent slots within r_cut of its box, and a warp iteration takes
+// four listed pairs against its 8 targets, two sources per lane in packed
+// (f32x2) arithmetic, with the exact cut taken per pair.  A target's sum stays
+// in registers over its sub-group's list, in a fixed order, so the result
+// does not depend on scheduling; in the adjoint the sources' sums over the 8
+// targets are exchanged by shuffles.  The FP64 variant lists the pairs inside
+// a conservative cut filter (|x_i|^2 + |x_j|^2 - 2 x_i.x_j against r_cut^2)
+// target by target, evaluates 32 listed pairs per iteration and sums each
+// target's run by a segmented scan.
+//
+// The kernel is bound by instruction issue and by the instruction cache: its
+// warps are at different places of a loop nest of about 2000 instructions, and
+// an adjoint build with 20 % more code runs 40 % slower on the clustered set
+// and no slower with one warp per SM.  Hence the loops that are not unrolled,
+// and the softened and cut-band pairs evaluated after their list.
 //
 // FP32 path.  Positions are split floats in box units (hi a multiple of 2^-23,
 // lo the rest), so hi_i - hi_j is exact and every displacement
@@ -33,7 +41,7 @@
 // reference, so decisions agree with an FP64 walk.  Interactions use the
 // special-function unit (rsqrt, ex2) and a polynomial for
 // erfcx(u) + 2u/sqrt(pi); per-target sums are Kahan-compensated after every
-// batch of 32 staged sources (at most 32 terms per target).
+// batch (at most 64 terms per target, 8 per lane and slot parity).
 #include <type_traits>
 
 #include "og_internal.cuh"
@@ -43,7 +51,7 @@ namespace og {
 
 constexpr int kWarpsPerBlock = 2;
 
-enum : int { DEC_DISCARD = 0, DEC_OPEN = 1, DEC_ACCEPT = 2, DEC_ACCEPT_OUT = 3, DEC_UNSURE = 4 };
+enum : int { DEC_DISCARD = 0, DEC_OPEN = 1, DEC_ACCEPT = 2, DEC_ACCEPT_OUT = 3 };
 
 
 // ------------------------------------------------------------------ helpers
@@ -58,14 +66,17 @@ __device__ __forceinline__ float ex2_approx(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // Minimum image of a box-unit difference t (|t| < 1.5): t - rint(t), with
 // rint by the 1.5 * 2^23 rounding constant (round to nearest even, so
 // +-0.5 stay), equal bit for bit to t - 1 / t + 1 / t on t > 0.5 / t < -0.5 /
 // otherwise.
-__device__ __forceinline__ float mi1(float t) {
-  const float r = __fadd_rn(__fadd_rn(t, 12582912.0f), -12582912.0f);
-  return __fadd_rn(t, -r);
-}
+__device__ __forceinline__ float round1(float t) { return __fadd_rn(__fadd_rn(t, 12582912.0f), -12582912.0f); }
+__device__ __forceinline__ float mi1(float t) { return __fadd_rn(t, -round1(t)); }
 
 __device__ __forceinline__ float sr_poly(float t) {
   float p = og_sr_poly[OG_SR_POLY_DEG];
@@ -195,17 +206,16 @@ constexpr int kStack = 276;
 constexpr int kStackNeed = 32;   // pushes of one step
 constexpr int kDeep = 64;
 static_assert(kDeep + 31 + 7 * 20 + 8 <= kStack - kStackNeed, "stack bound");
+constexpr int kSub = 4;          // sub-groups of 8 Hilbert-consecutive targets
 constexpr int kQueue = 128;      // queued leaves / accepted nodes per warp
 constexpr int kQueueNeed = 64;   // a step queues at most 2 entries per node
-constexpr int kSlots = 32;       // sources per evaluation batch
-constexpr int kRing = 2 * kSlots; // staged sources: two batches
-constexpr int kList = 512;       // (node or slot, target) list entries
+constexpr int kSlots = 32;       // sources fetched at a time
+constexpr int kStage = 2 * kSlots; // staged sources: one batch
+constexpr int kList = 512;       // FP64 variant: listed pairs; the FP32 walk lists at most kSub * kGroup entries
 
 // Stack entry: (first node | node count << 28, lane mask); node indices stay
 // below 2^28 (checked on the host).  Queue entry: (first particle or node,
-// particle count or -1 for an accepted node, lane mask, image flags).
-// Image flags bit 0: one shift puts the whole entry at the minimum image of
-// every target of the group (bits 1-6: the shift per axis, 0 / +1 / -1).
+// particle count or -1 for an accepted node, lane mask, unused).
 struct WarpBufs {
   int2* stack;
   int4* queue;
@@ -219,10 +229,7 @@ struct MixedScratch {
   float4 C[kGroup], A[kGroup], B[kGroup];  // C, A image-shifted when the node has a common image
   int node[kGroup], fl[kGroup];
   uint32_t mask[kGroup], acc[kGroup], open[kGroup];
-  uint32_t dmask[kGroup];  // lanes whose sub-group box leaves the node undecided
 };
-
-constexpr int kSub = 4;  // sub-groups of 8 Hilbert-consecutive targets
 
 enum : int { CL_NONE = -1, CL_DROP = 0, CL_OPEN = 1, CL_ACCEPT = 2, CL_MIXED = 3 };
 
@@ -260,24 +267,17 @@ __device__ __forceinline__ int classify(const WalkArgs& A, const GroupInfo& G, c
   return CL_MIXED;
 }
 
-// Image shift that puts every (target, source) pair of an entry that can lie
+// Image shift that puts every (target, source) pair of a node that can lie
 // inside rcut at its minimum image, if one exists for the whole cube.
-__device__ __forceinline__ int image_flags(const WalkArgs& A, const GroupInfo& G, const float4& NC) {
+__device__ __forceinline__ bool node_image(const WalkArgs& A, const GroupInfo& G, const float4& NC, float& nx, float& ny,
+                                           float& nz) {
   const float hs = 0.5f * NC.w;
   const float dx = NC.x - G.cx, dy = NC.y - G.cy, dz = NC.z - G.cz;
-  const float nx = rintf(dx), ny = rintf(dy), nz = rintf(dz);
-  const bool uni = fabsf(dx - nx) + G.ex + hs < A.uni_lim && fabsf(dy - ny) + G.ey + hs < A.uni_lim &&
-                   fabsf(dz - nz) + G.ez + hs < A.uni_lim;
-  if (!uni) return 0;
-  const int cx = nx > 0.5f ? 1 : (nx < -0.5f ? 2 : 0);
-  const int cy = ny > 0.5f ? 1 : (ny < -0.5f ? 2 : 0);
-  const int cz = nz > 0.5f ? 1 : (nz < -0.5f ? 2 : 0);
-  return 1 | (cx << 1) | (cy << 3) | (cz << 5);
-}
-
-__device__ __forceinline__ float shift_of(int flags, int axis) {
-  const int c = (flags >> (1 + 2 * axis)) & 3;
-  return c == 1 ? 1.0f : (c == 2 ? -1.0f : 0.0f);
+  nx = round1(dx);
+  ny = round1(dy);
+  nz = round1(dz);
+  return fabsf(dx - nx) + G.ex + hs < A.uni_lim && fabsf(dy - ny) + G.ey + hs < A.uni_lim &&
+         fabsf(dz - nz) + G.ez + hs < A.uni_lim;
 }
 
 // Validates the queue and writes the slot offsets; returns the slot count or
@@ -285,6 +285,7 @@ __device__ __forceinline__ float shift_of(int flags, int axis) {
 __device__ __forceinline__ int queue_offsets(const WalkArgs& A, const WarpBufs& W, int nq, int lane) {
   int run = 0;
   bool badq = false;
+#pragma unroll 1
   for (int b0 = 0; b0 < nq; b0 += 32) {
     const int e = b0 + lane;
     int c = 0;
@@ -315,11 +316,14 @@ __device__ __forceinline__ int queue_offsets(const WalkArgs& A, const WarpBufs& 
 
 // 32 x 32 bit-matrix transpose across the warp: lane r holds row r (bit c =
 // column c) and receives column r.  Five stages swap the off-diagonal blocks
-// of side 16, 8, 4, 2, 1 between partner lanes.
+// of side 16, 8, 4, 2, 1 between partner lanes.  (Unrolled, the forward walk
+// needs 110 registers instead of 96 and loses a resident block; the adjoint
+// is 2-5 % faster with it.)
+template <int kUnroll>
 __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
   const uint32_t keep[5] = {0x0000ffffu, 0x00ff00ffu, 0x0f0f0f0fu, 0x33333333u, 0x55555555u};
   int j = 16;
-#pragma unroll
+#pragma unroll kUnroll
   for (int st = 0; st < 5; ++st, j >>= 1) {
     const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
     x = (lane & j) == 0 ? ((x & keep[st]) | ((y & keep[st]) << j)) : ((x & ~keep[st]) | ((y & ~keep[st]) >> j));
@@ -343,92 +347,102 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
   return d;
 }
 
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float lo2(unsigned long long a) { return __uint_as_float((uint32_t)a); }
+__device__ __forceinline__ float hi2(unsigned long long a) { return __uint_as_float((uint32_t)(a >> 32)); }
+// sr_poly of both halves; the doubled coefficients sit in constant memory
+// (a 64-bit operand cannot be an immediate).
+__device__ __forceinline__ unsigned long long sr_poly2(unsigned long long t) {
+  const unsigned long long* c = reinterpret_cast<const unsigned long long*>(og_sr_poly2);
+  unsigned long long p = c[OG_SR_POLY_DEG];
+#pragma unroll
+  for (int k = OG_SR_POLY_DEG - 1; k >= 0; --k) p = fma2(p, t, c[k]);
+  return p;
+}
+__device__ __forceinline__ uint32_t low_bits(int n) { return n >= 32 ? 0xffffffffu : ((1u << n) - 1u); }
+
 // Exact per-target decision for a node (FP32 with an FP64 re-check in the
 // band), target given by its split position.  With uni, NC and NA are
 // already shifted to the image that is the minimum image for every target
-// of the group, so no per-target minimum image is taken.
+// of the group, so no per-target minimum image is taken.  A node beyond
+// rcut is opened rather than discarded: none of its descendants gives this
+// target a term, and the test is saved.  A node whose farthest corner is
+// inside the cut has its centre of mass inside it.
 __device__ __forceinline__ float mi1_if(bool per_target, float t) { return per_target ? mi1(t) : t; }
 
 __device__ __forceinline__ int decide_f32(const WalkArgs& A, int64_t k, const float4& th, const float4& tl, int node,
-                                          const int4& ND, const float4& NC, const float4& NA, const float4& NB,
+                                          int level, const float4& NC, const float4& NA, const float4& NB,
                                           bool uni) {
   const float s = NC.w, hs = 0.5f * s;
   // hi differences are exact: the minimum image is taken before the lo parts are added
   const float ax = fabsf(mi1_if(!uni, NC.x - th.x) - tl.x);
   const float ay = fabsf(mi1_if(!uni, NC.y - th.y) - tl.y);
   const float az = fabsf(mi1_if(!uni, NC.z - th.z) - tl.z);
-  const float ex = fmaxf(ax - hs, 0.f), ey = fmaxf(ay - hs, 0.f), ez = fmaxf(az - hs, 0.f);
-  const float e2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-  if (e2 > A.rc2_hi) return DEC_DISCARD;
   const float d0 = mi1_if(!uni, th.x - NA.x) + (tl.x - NB.x);
   const float d1 = mi1_if(!uni, th.y - NA.y) + (tl.y - NB.y);
   const float dz = mi1_if(!uni, th.z - NA.z) + (tl.z - NB.z);
   const float d2 = fmaf(d0, d0, fmaf(d1, d1, dz * dz));
-  int dec;
-  if (e2 >= A.rc2_lo) {
-    dec = DEC_UNSURE;
-  } else {
-    const float fx = ax + hs, fy = ay + hs, fz = az + hs;
-    const float far2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
-    const float lhs = s * s;
-    const float cmax = fmaxf(ax, fmaxf(ay, az));
-    const int a1 = lhs < A.th2_lo * d2 ? 1 : (lhs > A.th2_hi * d2 ? 0 : 2);
-    const int a2 = cmax > A.lim_hi * s ? 1 : (cmax < A.lim_lo * s ? 0 : 2);
-    const int a3 = far2 < A.rc2_lo ? 1 : (far2 > A.rc2_hi ? 0 : 2);
-    if (a1 == 0 || a2 == 0 || a3 == 0) dec = DEC_OPEN;
-    else if (a1 == 2 || a2 == 2 || a3 == 2) dec = DEC_UNSURE;
-    else dec = d2 < A.rc2_lo ? DEC_ACCEPT : (d2 > A.rc2_hi ? DEC_ACCEPT_OUT : DEC_UNSURE);
-  }
-  if (dec == DEC_UNSURE) dec = decide_exact(A, k, node, meta_level(ND.w));
-  return dec;
+  const float fx = ax + hs, fy = ay + hs, fz = az + hs;
+  const float far2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+  const float lhs = s * s;
+  const float cmax = fmaxf(ax, fmaxf(ay, az));
+  if (lhs > A.th2_hi * d2 || cmax < A.lim_lo * s || far2 > A.rc2_hi) return DEC_OPEN;
+  if (lhs < A.th2_lo * d2 && cmax > A.lim_hi * s && far2 < A.rc2_lo) return DEC_ACCEPT;
+  return decide_exact(A, k, node, level);
 }
 
-// One pair's result on the target side: FP32 (with the hit flag in w) or
-// FP64 (hit flag separate).
-template <bool F64> struct Term { float x, y, z, w; };
-template <> struct Term<true> { double x, y, z; float w; };
+// One pair's result in the FP64 variant and whether it lies inside the cut.
+struct Term64 {
+  double x, y, z;
+  bool in;
+};
 
 // Lane of the walk: FP32 + Kahan forward (ADJ = false) or adjoint
-// (ADJ = true), or the all-FP64 forward comparison variant (F64 = true:
-// FP64 decisions, FP64 pair arithmetic with CUDA's erfc / exp, plain double
-// sums).  All share the traversal, the box test, the FP32 cut filter (a
-// conservative superset of the pairs inside the cut) and the compaction.
+// (ADJ = true), or the all-FP64 forward variant (F64 = true: FP64 pair
+// arithmetic, plain double sums).  All share the traversal, its decisions
+// (which agree with FP64) and the box test.
 // FUSED (with ADJ): the adjoint walk that also writes the forward
 // accelerations, each pair's force factor serving both (one traversal for a
 // loss whose weights are known before the walk).
 template <bool ADJ, bool F64, bool FUSED = false>
 struct LaneFP {
   static_assert(!FUSED || (ADJ && !F64), "the fused walk is the FP32 adjoint plus the forward sums");
+  static constexpr int kListSize = F64 ? kList : kSub * kGroup;
   // per-warp data that lives through the whole walk
   struct Smem {
     float4 tA[kGroup];    // targets: hi part, h^2
     float4 tB[kGroup];    // targets: lo part
     float4 tW[ADJ ? kGroup : 1];   // adjoint: dL/da of each target
-    float4 SG[ADJ ? kGroup : 1];     // adjoint: source-side term (G, S) of each lane's listed pair
-    uint32_t smask[ADJ ? kSlots : 1];  // adjoint: the lanes whose listed pair has this slot
+    float4 SG[ADJ ? kStage : 1];   // adjoint: source-side sums (G, S) of each staged slot over the batch
     int self[kGroup];     // staged slot holding the target itself, or -1
-    typename std::conditional<F64, double3, float4>::type Ps[kGroup];  // each target's sum over the batch
-    float4 Pf[FUSED ? kGroup : 1];  // fused: each target's forward sum over the batch
-    int fneg[kGroup];     // listed pairs of the batch found outside the exact cut
+    double3 Ps[F64 ? kGroup : 1];  // FP64 variant: each target's sum over the batch
+    int fneg[F64 ? kGroup : 1];  // FP64 variant: listed pairs of the batch outside the exact cut
   };
   // per-batch staging (dead between evaluations; shares memory with the
   // traversal's scratch)
-  // Staged sources live in a ring of two batches: survivors of the box test
-  // are appended at the tail, and a batch is evaluated once 32 are pending.
+  // Survivors of the box test are appended; a batch is evaluated once the
+  // next 32 might not fit.  The FP32 walk keeps the two sources of adjacent
+  // slots 2k, 2k + 1 component by component, so that one 16-byte load gives
+  // two register pairs of a packed (f32x2) operand.
   struct Stage {
-    float4 sa[kRing];     // staged source: hi part (image-shifted), mass
-    float4 sb[kRing];     // lo part, h^2
-    int2 sc[kRing];       // id (particle, or -2 - node), per-pair image flag
-    uint32_t sq[kRing];   // lane mask of the source's queue entry
-    float fX[kRing], fY[kRing], fZ[kRing], fW[kRing];  // filter form (see put)
+    float4 s0[F64 ? 1 : kStage / 2];  // -hi.x of both, -hi.y of both (image-shifted)
+    float4 s1[F64 ? 1 : kStage / 2];  // -hi.z, -mass
+    float4 s2[F64 ? 1 : kStage / 2];  // -lo.x, -lo.y
+    float4 s3[F64 ? 1 : kStage / 2];  // -lo.z, h^2
+    float4 ra[F64 ? 1 : kSlots], rb[F64 ? 1 : kSlots];  // the next 32 sources as they arrive from the tree
+    int id[kStage];       // particle, or -2 - node
+    uint32_t sq[kStage];  // lane mask of the source's queue entry
+    float fX[F64 ? kStage : 1], fY[F64 ? kStage : 1], fZ[F64 ? kStage : 1], fW[F64 ? kStage : 1];  // filter form (see put)
   };
-  // a slot's source as read from the tree, hi part image-shifted when its
-  // entry has a common image (uni)
+  // a slot's source as read from the tree
   struct Fetch {
     float4 a, b;
-    int id;
+    int id;  // particle, or -2 - node
     uint32_t q;
-    bool node, uni;
   };
 
   int64_t k;          // sorted index of this lane's target
@@ -439,7 +453,6 @@ struct LaneFP {
   float Pf[3], Sf[3], Cf[3];  // fused: the forward sums likewise
   double a64[3];      // FP64 variant: plain double sums
   int nint;
-  float4 gs;          // adjoint: this lane's slot, source-side sums (G, S) over the batch
 
   __device__ void init(const WalkArgs& A, Smem& M, int64_t kk, bool v, int lane, const GroupInfo& G) {
     k = kk;
@@ -450,17 +463,15 @@ struct LaneFP {
     M.tA[lane] = make_float4(a.x, a.y, a.z, b.w);
     M.tB[lane] = make_float4(b.x, b.y, b.z, 0.f);
     if constexpr (F64) M.Ps[lane] = make_double3(0.0, 0.0, 0.0);
-    else M.Ps[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
     a64[0] = a64[1] = a64[2] = 0.0;
-    M.fneg[lane] = 0;
-    if (ADJ) { gs = make_float4(0.f, 0.f, 0.f, 0.f); M.smask[lane] = 0u; }
+    if constexpr (F64) M.fneg[lane] = 0;
+    if constexpr (ADJ) M.SG[lane] = M.SG[lane + 32] = make_float4(0.f, 0.f, 0.f, 0.f);
     xr[0] = (a.x - G.cx) + b.x;
     xr[1] = (a.y - G.cy) + b.y;
     xr[2] = (a.z - G.cz) + b.z;
     sr = fmaf(xr[0], xr[0], fmaf(xr[1], xr[1], xr[2] * xr[2]));
 #pragma unroll
     for (int c = 0; c < 3; ++c) { P[c] = 0.f; S[c] = 0.f; C[c] = 0.f; Pf[c] = 0.f; Sf[c] = 0.f; Cf[c] = 0.f; }
-    if constexpr (FUSED) M.Pf[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (ADJ) {
       float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
       if (v) {
@@ -472,19 +483,12 @@ struct LaneFP {
     nint = 0;
   }
 
-  __device__ __forceinline__ int decide_for(const WalkArgs& A, const Smem& M, int t, int64_t kt, int node,
-                                            const int4& ND, const float4& NC, const float4& NA, const float4& NB,
-                                            bool uni) const {
-    if constexpr (F64) return decide_exact(A, kt, node, meta_level(ND.w));
-    else return decide_f32(A, kt, M.tA[t], M.tB[t], node, ND, NC, NA, NB, uni);
-  }
-
   // FP64 variant: target gbase + i against staged slot s, read from the
   // FP64 tree arrays; the cut is taken on the FP64 distance (accepted nodes
   // are inside by decision).
-  __device__ __forceinline__ Term<true> pair_eval64(const WalkArgs& A, const Stage& St, int i, int s,
+  __device__ __forceinline__ Term64 pair_eval64(const WalkArgs& A, const Stage& St, int i, int s,
                                                     int64_t gbase) const {
-    const int id = St.sc[s].x;
+    const int id = St.id[s];
     const int64_t kt = gbase + i;
     const double* x = A.T.x64;
     double sp[3], m, h;
@@ -504,9 +508,7 @@ struct LaneFP {
 #pragma unroll
     for (int c = 0; c < 3; ++c) dv[c] = mi64(__dsub_rn(x[3 * kt + c], sp[c]), A.box);
     const double r2 = norm2_64(dv[0], dv[1], dv[2]);
-    Term<true> t;
-    t.x = t.y = t.z = 0.0;
-    t.w = 0.f;
+    Term64 t = {0.0, 0.0, 0.0, false};
     if (id >= 0 && !(r2 < A.rc2_64)) return t;
     const double r = sqrt(r2);
     const double hh = fmax(A.T.h64[kt], h);
@@ -525,76 +527,99 @@ struct LaneFP {
     t.x = sc * dv[0];
     t.y = sc * dv[1];
     t.z = sc * dv[2];
-    t.w = 1.f;
+    t.in = true;
     return t;
   }
 
-  // Fetch slot s of queue entry e.
-  __device__ __forceinline__ Fetch fetch(const WalkArgs& A, const WarpBufs& W, int e, int s) const {
-    Fetch f;
+  // Start fetching slot s of queue entry e: its two 16-byte records go to
+  // this lane's place in the staging buffer, asynchronously in the FP32 walk.
+  __device__ __forceinline__ void fetch(const WalkArgs& A, const WarpBufs& W, Stage& St, int e, int s, int lane,
+                                        Fetch& f) const {
     const int4 Q = W.queue[e];
-    f.node = Q.y < 0;
-    if (f.node) {
-      f.a = A.T.nA[Q.x];
-      f.b = A.T.nB[Q.x];
-      f.id = -2 - Q.x;
-    } else {
-      const int j = Q.x + (s - W.qoff[e]);
-      f.a = A.T.pA[j];
-      f.b = A.T.pB[j];
-      f.id = j;
-    }
-    f.uni = (Q.w & 1) != 0;
-    if (f.uni) {
-      f.a.x -= shift_of(Q.w, 0);
-      f.a.y -= shift_of(Q.w, 1);
-      f.a.z -= shift_of(Q.w, 2);
-    }
+    const bool node = Q.y < 0;
+    const int j = node ? Q.x : Q.x + (s - W.qoff[e]);
+    const float4* pa = (node ? A.T.nA : A.T.pA) + j;
+    const float4* pb = (node ? A.T.nB : A.T.pB) + j;
+    f.id = node ? -2 - j : j;
     f.q = (uint32_t)Q.z;
-    return f;
+    if constexpr (F64) {
+      f.a = *pa;
+      f.b = *pb;
+    } else {
+      cp_async16(&St.ra[lane], pa);
+      cp_async16(&St.rb[lane], pb);
+    }
   }
 
-  // Position of a fetched source relative to the group centre, and whether
-  // it can have a pair inside the cut with some target of the group (its
-  // distance to the padded group box within the conservative group
-  // threshold).  Accepted nodes and entries without a common image are
-  // always kept.
-  __device__ __forceinline__ bool keep(const WalkArgs& A, const Fetch& f, const GroupInfo& G, float& x0, float& x1,
-                                       float& x2) const {
-    x0 = (f.a.x - G.cx) + f.b.x;
-    x1 = (f.a.y - G.cy) + f.b.y;
-    x2 = (f.a.z - G.cz) + f.b.z;
-    if (f.node || !f.uni) return true;
-    const float g0 = fmaxf(fabsf(x0) - G.ex, 0.f), g1 = fmaxf(fabsf(x1) - G.ey, 0.f), g2 = fmaxf(fabsf(x2) - G.ez, 0.f);
+  // The fetched source, once arrived: shifted to its image nearest to the
+  // group centre (x: its position relative to that centre), and whether it
+  // can have a pair inside the cut with some target of the group (its
+  // distance to the padded group box within the conservative threshold).
+  // uni: that image is the minimum image of every target of the group that
+  // it can have such a pair with.
+  __device__ __forceinline__ bool arrive(const WalkArgs& A, const Stage& St, int lane, const GroupInfo& G, Fetch& f,
+                                         float (&x)[3], bool& uni) const {
+    if constexpr (!F64) {
+      cp_async_wait();
+      f.a = St.ra[lane];
+      f.b = St.rb[lane];
+    }
+    x[0] = f.a.x - G.cx;
+    x[1] = f.a.y - G.cy;
+    x[2] = f.a.z - G.cz;
+    const float n0 = round1(x[0]), n1 = round1(x[1]), n2 = round1(x[2]);
+    f.a.x -= n0;
+    f.a.y -= n1;
+    f.a.z -= n2;
+    x[0] = (x[0] - n0) + f.b.x;
+    x[1] = (x[1] - n1) + f.b.y;
+    x[2] = (x[2] - n2) + f.b.z;
+    const float a0 = fabsf(x[0]), a1 = fabsf(x[1]), a2 = fabsf(x[2]);
+    uni = fmaxf(a0 + G.ex, fmaxf(a1 + G.ey, a2 + G.ez)) < A.uni_lim;
+    const float g0 = fmaxf(a0 - G.ex, 0.f), g1 = fmaxf(a1 - G.ey, 0.f), g2 = fmaxf(a2 - G.ez, 0.f);
     return fmaf(g0, g0, fmaf(g1, g1, g2 * g2)) <= A.grp_rc2;
   }
 
-  // Stage a fetched source at ring position pos.
-  // Filter form: (-2 x, -2 y, -2 z, |x|^2 - r_cut^2 - margin) relative to the
-  // group centre, so |x_i - x_j|^2 - r_cut^2 - margin evaluates as
-  // fW + |x_i|^2 + fX x_i + fY y_i + fZ z_i.  The FP32 evaluation of that
-  // chain is within 18 u (|x_i| + |x_j|)^2 + 18 u r_cut^2 of the exact value
-  // (u = 2^-24); the margin is 64 u times that bound's bracket, so every pair
-  // inside the cut gives a negative value.
-  __device__ __forceinline__ void put(const WalkArgs& A, Stage& S, Smem& M, const Fetch& f, int pos, float x0,
-                                      float x1, float x2, int64_t gbase, float Rg) const {
-    float fx = 0.f, fy = 0.f, fz = 0.f, fw = -1e30f;  // accepted node or per-pair image: always a candidate
-    if (f.uni && !f.node) {
-      const float sj = fmaf(x0, x0, fmaf(x1, x1, x2 * x2));
-      const float rr = sqrtf(sj) + Rg;
-      fx = -2.f * x0;
-      fy = -2.f * x1;
-      fz = -2.f * x2;
-      fw = (sj - A.rc2_hi) - 3.814697265625e-06f * fmaf(rr, rr, A.rc2_hi);
+  // Stage a fetched source in slot pos.
+  // FP64 variant, filter form: (-2 x, -2 y, -2 z, |x|^2 - r_cut^2 - margin)
+  // relative to the group centre, so |x_i - x_j|^2 - r_cut^2 - margin
+  // evaluates as fW + |x_i|^2 + fX x_i + fY y_i + fZ z_i.  The FP32 evaluation
+  // of that chain is within 18 u (|x_i| + |x_j|)^2 + 18 u r_cut^2 of the exact
+  // value (u = 2^-24); the margin is 64 u times that bound's bracket, so every
+  // pair inside the cut gives a negative value.
+  __device__ __forceinline__ void put(const WalkArgs& A, Stage& S, Smem& M, const Fetch& f, int pos,
+                                      const float (&x)[3], bool uni, int64_t gbase, float Rg) const {
+    if constexpr (!F64) {
+      const int e = 4 * (pos >> 1) + (pos & 1);  // this slot's first word of its pair's 16 bytes
+      float* p0 = &S.s0[0].x + e;
+      float* p1 = &S.s1[0].x + e;
+      float* p2 = &S.s2[0].x + e;
+      float* p3 = &S.s3[0].x + e;
+      p0[0] = -f.a.x;
+      p0[2] = -f.a.y;
+      p1[0] = -f.a.z;
+      p1[2] = -f.a.w;
+      p2[0] = -f.b.x;
+      p2[2] = -f.b.y;
+      p3[0] = -f.b.z;
+      p3[2] = f.b.w;
+    } else {
+      float fx = 0.f, fy = 0.f, fz = 0.f, fw = -1e30f;  // accepted node or per-pair image: always a candidate
+      if (uni && f.id >= 0) {
+        const float sj = fmaf(x[0], x[0], fmaf(x[1], x[1], x[2] * x[2]));
+        const float rr = sqrtf(sj) + Rg;
+        fx = -2.f * x[0];
+        fy = -2.f * x[1];
+        fz = -2.f * x[2];
+        fw = (sj - A.rc2_hi) - 3.814697265625e-06f * fmaf(rr, rr, A.rc2_hi);
+      }
+      S.fX[pos] = fx;
+      S.fY[pos] = fy;
+      S.fZ[pos] = fz;
+      S.fW[pos] = fw;
     }
-    S.sa[pos] = f.a;
-    S.sb[pos] = f.b;
-    S.sc[pos] = make_int2(f.id, f.uni ? 0 : 1);
+    S.id[pos] = f.id;
     S.sq[pos] = f.q;
-    S.fX[pos] = fx;
-    S.fY[pos] = fy;
-    S.fZ[pos] = fz;
-    S.fW[pos] = fw;
     if (f.id >= gbase && f.id < gbase + kGroup) M.self[f.id - gbase] = pos;
   }
 
@@ -610,55 +635,9 @@ struct LaneFP {
     }
   }
 
-  // Target i of the group against staged slot s: the exact cut decision, and
-  // the interaction (target-side term, hit flag).  In the adjoint the
-  // source-side terms go to sg.
-  __device__ __forceinline__ float4 pair_eval(const WalkArgs& A, const Stage& St, const Smem& M, int i, int s,
-                                              int64_t gbase, float4& sg, float3& fw) const {
-    fw = make_float3(0.f, 0.f, 0.f);
-    const float4 ta = M.tA[i], tb = M.tB[i];
-    const float4 a = St.sa[s], b = St.sb[s];
-    const int2 c = St.sc[s];
-    float dh0 = ta.x - a.x, dh1 = ta.y - a.y, dh2 = ta.z - a.z;
-    if (c.y) {
-      dh0 = mi1(dh0);
-      dh1 = mi1(dh1);
-      dh2 = mi1(dh2);
-    }
-    float dv[3];
-    dv[0] = dh0 + (tb.x - b.x);
-    dv[1] = dh1 + (tb.y - b.y);
-    dv[2] = dh2 + (tb.z - b.z);
-    const float r2 = fmaf(dv[0], dv[0], fmaf(dv[1], dv[1], dv[2] * dv[2]));
-    // accepted node (id < 0): inside by decision; particle: cut band, then FP64
-    bool in = c.x < 0 || r2 < A.pp_lo;
-    if (!in) in = r2 <= A.pp_hi && pair_inside_exact(A, gbase + i, c.x);
-    sg = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!in) return make_float4(0.f, 0.f, 0.f, 0.f);
-    float F, Fr;
-    force_f32<ADJ>(A, r2, fmaxf(ta.w, b.w), F, Fr);
-    if (!ADJ) {
-      const float sc = -a.w * F;
-      return make_float4(sc * dv[0], sc * dv[1], sc * dv[2], 1.f);
-    } else {
-      const float4 w = M.tW[i];
-      const float dw = fmaf(dv[0], w.x, fmaf(dv[1], w.y, dv[2] * w.z));
-      const float qq = Fr * dw;
-      const float j0 = -fmaf(F, w.x, qq * dv[0]);
-      const float j1 = -fmaf(F, w.y, qq * dv[1]);
-      const float j2 = -fmaf(F, w.z, qq * dv[2]);
-      sg = make_float4(j0, j1, j2, -F * dw);
-      if constexpr (FUSED) {
-        const float sc = -a.w * F;
-        fw = make_float3(sc * dv[0], sc * dv[1], sc * dv[2]);
-      }
-      return make_float4(a.w * j0, a.w * j1, a.w * j2, 1.f);
-    }
-  }
-
   // Evaluate the queued entries (see the header comment).
   __device__ void evaluate(const WalkArgs& A, const WarpBufs& W, Stage& St, Smem& M, int nq, int lane,
-                           const GroupInfo& G, int64_t gbase, uint32_t vmask, float Rg) {
+                           const GroupInfo& G, const float4* SGB, int64_t gbase, uint32_t vmask, float Rg) {
     const int total = queue_offsets(A, W, nq, lane);
     if (total < 0) {
       if (lane == 0) set_status(A.wsb, ST_TREELINK);
@@ -667,75 +646,402 @@ struct LaneFP {
     const uint32_t lt = (1u << lane) - 1u;
     M.self[lane] = -1;
     __syncwarp();
-    // raw slots are fetched 32 at a time and the survivors of the box test
-    // are appended to the ring; pending slots occupy positions
-    // [32 half, 32 half + pend) mod 64
+    // slots are fetched 32 at a time and the survivors of the box test are
+    // appended to the staged ones
     // Each window of 32 slots finds its slots' entries without a search:
     // ecur holds the window's first slot, the entries starting inside the
     // window set bit (start - rb) of one OR-reduced mask (an entry holds at
     // least one slot, so at most 31 start inside it), and slot rb + l lies
     // in entry ecur + (number of starts at or before bit l).
-    int pend = 0, tail = 0, half = 0;
+    // The next window is fetched while the current one is staged and evaluated.
+    int pend = 0;
+    bool mi = false;  // some staged source has no image common to the whole group
     int ecur = 0;
-    for (int rb = 0; rb < total; rb += 32) {
+    Fetch cur = {};
+    auto window = [&](int rb, Fetch& f) {
       const int ek = ecur + 1 + lane;
       const int sk = ek < nq ? W.qoff[ek] - rb : 32;
       const uint32_t starts = __reduce_or_sync(0xffffffffu, (sk > 0 && sk < 32) ? (1u << sk) : 0u);
-      Fetch cur = {};
-      bool kp = false;
-      float x0 = 0.f, x1 = 0.f, x2 = 0.f;
-      if (rb + lane < total) {
-        cur = fetch(A, W, ecur + __popc(starts & ((2u << lane) - 1u)), rb + lane);
-        kp = keep(A, cur, G, x0, x1, x2);
-      }
+      if (rb + lane < total) fetch(A, W, St, ecur + __popc(starts & ((2u << lane) - 1u)), rb + lane, lane, f);
+      // the entry holding the following window's first slot
+      const int en = ecur + __popc(starts);
+      ecur = en + (en + 1 < nq && W.qoff[en + 1] == rb + 32 ? 1 : 0);
+    };
+    window(0, cur);
+#pragma unroll 1
+    for (int rb = 0; rb < total; rb += 32) {
+      bool uni = true;
+      float x[3] = {0.f, 0.f, 0.f};
+      const bool kp = rb + lane < total && arrive(A, St, lane, G, cur, x, uni);
       const uint32_t km = __ballot_sync(0xffffffffu, kp);
-      if (kp) put(A, St, M, cur, (tail + __popc(km & lt)) & (kRing - 1), x0, x1, x2, gbase, Rg);
-      tail = (tail + __popc(km)) & (kRing - 1);
+      if (kp) put(A, St, M, cur, pend + __popc(km & lt), x, uni, gbase, Rg);
+      mi = mi || __any_sync(0xffffffffu, kp && !uni);
       pend += __popc(km);
+      if (rb + 32 < total) window(rb + 32, cur);
       __syncwarp();
-      const bool last = rb + 32 >= total;
-      while (pend >= kSlots || (last && pend > 0)) {
-        const int cnt = min(pend, kSlots);
-        batch(A, W, St, M, half * kSlots, cnt, lane, gbase, vmask);
-        pend -= cnt;
-        half ^= 1;
+      if (pend > 0 && (pend > kStage - 32 || rb + 32 >= total)) {
+        if constexpr (F64) {
+#pragma unroll 1
+          for (int hb = 0; hb < pend; hb += 32) batch_list(A, W, St, M, hb, min(pend - hb, 32), lane, gbase, vmask);
+        } else {
+          batch_tiles(A, W, St, M, SGB, pend, lane, gbase, vmask, mi);
+        }
+        pend = 0;
+        mi = false;
       }
-      // the entry holding the next window's first slot
-      int en = ecur + __popc(starts);
-      if (en + 1 < nq && W.qoff[en + 1] == rb + 32) ++en;
-      ecur = en;
     }
   }
 
-  // One batch: the cnt staged sources at ring positions [hb, hb + cnt).
-  __device__ void batch(const WalkArgs& A, const WarpBufs& W, Stage& St, Smem& M, int hb, int cnt, int lane,
-                        int64_t gbase, uint32_t vmask) {
-    const unsigned long long X2 = pack2(xr[0], xr[0]), Y2 = pack2(xr[1], xr[1]), Z2 = pack2(xr[2], xr[2]);
-    const unsigned long long S2 = pack2(sr, sr);
-    // bit s of msk: slot s is in this lane's part of its entry's lane mask
-    const bool has = lane < cnt;
-    const uint32_t q = has ? St.sq[hb + lane] : 0u;
-    const uint32_t cm = cnt == 32 ? 0xffffffffu : ((1u << cnt) - 1u);
-    uint32_t msk;
-    if (__any_sync(0xffffffffu, has && q != vmask)) msk = transpose32(q, lane);
-    else msk = valid ? cm : 0u;
-    // conservative cut test for all 32 slots, two per instruction; the sign
-    // bit of each result is shifted into acc (slot 0 ends up at bit 31)
-    uint32_t acc = 0;
-#pragma unroll
-    for (int s = 0; s < kSlots; s += 4) {
-      const float4 fx = *reinterpret_cast<const float4*>(St.fX + hb + s);
-      const float4 fy = *reinterpret_cast<const float4*>(St.fY + hb + s);
-      const float4 fz = *reinterpret_cast<const float4*>(St.fZ + hb + s);
-      const float4 fw = *reinterpret_cast<const float4*>(St.fW + hb + s);
-      unsigned long long r01 = add2(pack2(fw.x, fw.y), S2);
-      unsigned long long r23 = add2(pack2(fw.z, fw.w), S2);
+  // Conservative cut test of this lane's target against the slots s and
+  // s + 1 .. s + 3 of the filter arrays, two per instruction; a result's sign
+  // bit is set where the pair can lie inside the cut.
+  struct Filter {
+    unsigned long long X2, Y2, Z2, S2;
+    __device__ __forceinline__ void four(const Stage& St, int s, unsigned long long& r01,
+                                         unsigned long long& r23) const {
+      const float4 fx = *reinterpret_cast<const float4*>(St.fX + s);
+      const float4 fy = *reinterpret_cast<const float4*>(St.fY + s);
+      const float4 fz = *reinterpret_cast<const float4*>(St.fZ + s);
+      const float4 fw = *reinterpret_cast<const float4*>(St.fW + s);
+      r01 = add2(pack2(fw.x, fw.y), S2);
+      r23 = add2(pack2(fw.z, fw.w), S2);
       r01 = fma2(pack2(fz.x, fz.y), Z2, r01);
       r23 = fma2(pack2(fz.z, fz.w), Z2, r23);
       r01 = fma2(pack2(fy.x, fy.y), Y2, r01);
       r23 = fma2(pack2(fy.z, fy.w), Y2, r23);
       r01 = fma2(pack2(fx.x, fx.y), X2, r01);
       r23 = fma2(pack2(fx.z, fx.w), X2, r23);
+    }
+  };
+  __device__ __forceinline__ Filter filter() const {
+    return {pack2(xr[0], xr[0]), pack2(xr[1], xr[1]), pack2(xr[2], xr[2]), pack2(sr, sr)};
+  }
+
+  // One target against one slot pair: displacements, squared distances and
+  // -mass, packed over the pair's two slots.
+  struct Pair {
+    unsigned long long dx, dy, dz, r2, nm;
+    float h20, h21;  // softening: max of the target's and the source's h^2
+  };
+  // A sub-group's target as this lane holds it, each component twice.
+  struct Target {
+    unsigned long long x, y, z, u, v, w;  // hi and lo parts
+    unsigned long long wx, wy, wz;        // adjoint: dL/da
+    float h2;
+  };
+  // Packed sums of this lane's pairs with its target, even and odd slots.
+  struct Sums {
+    unsigned long long ax, ay, az;  // target side: the force, or m J w in the adjoint
+    unsigned long long bx, by, bz;  // fused: the force
+  };
+
+  __device__ __forceinline__ Pair load_pair(const Stage& St, const Target& T, int k, bool mi) const {
+    const float4 v0 = St.s0[k], v1 = St.s1[k], v2 = St.s2[k], v3 = St.s3[k];
+    Pair p;
+    p.dx = add2(T.x, pack2(v0.x, v0.y));
+    p.dy = add2(T.y, pack2(v0.z, v0.w));
+    p.dz = add2(T.z, pack2(v1.x, v1.y));
+    if (mi) {
+      p.dx = pack2(mi1(lo2(p.dx)), mi1(hi2(p.dx)));
+      p.dy = pack2(mi1(lo2(p.dy)), mi1(hi2(p.dy)));
+      p.dz = pack2(mi1(lo2(p.dz)), mi1(hi2(p.dz)));
+    }
+    p.dx = add2(p.dx, add2(T.u, pack2(v2.x, v2.y)));
+    p.dy = add2(p.dy, add2(T.v, pack2(v2.z, v2.w)));
+    p.dz = add2(p.dz, add2(T.w, pack2(v3.x, v3.y)));
+    p.r2 = fma2(p.dx, p.dx, fma2(p.dy, p.dy, mul2(p.dz, p.dz)));
+    p.nm = pack2(v1.z, v1.w);
+    p.h20 = fmaxf(T.h2, v3.z);
+    p.h21 = fmaxf(T.h2, v3.w);
+    return p;
+  }
+
+  // Adds a pair with force factors F (zero for a slot that is no hit) to the
+  // lane's sums and, in the adjoint, to the slots' sums.  own: this lane's
+  // slot pair is its own (lanes past the end of the list repeat the last one).
+  __device__ __forceinline__ void add_pair(Smem& M, const Target& T, const Pair& p, unsigned long long F,
+                                           unsigned long long Fr, int k, bool own, int lane, Sums& S) const {
+    if constexpr (!ADJ) {
+      const unsigned long long sc = mul2(p.nm, F);
+      S.ax = fma2(sc, p.dx, S.ax);
+      S.ay = fma2(sc, p.dy, S.ay);
+      S.az = fma2(sc, p.dz, S.az);
+    } else {
+      const unsigned long long dw = fma2(p.dx, T.wx, fma2(p.dy, T.wy, mul2(p.dz, T.wz)));
+      const unsigned long long qq = mul2(Fr, dw);
+      // J w and F d.w; the source side takes their negatives
+      const unsigned long long j0 = fma2(F, T.wx, mul2(qq, p.dx));
+      const unsigned long long j1 = fma2(F, T.wy, mul2(qq, p.dy));
+      const unsigned long long j2 = fma2(F, T.wz, mul2(qq, p.dz));
+      const unsigned long long js = mul2(F, dw);
+      S.ax = fma2(p.nm, j0, S.ax);
+      S.ay = fma2(p.nm, j1, S.ay);
+      S.az = fma2(p.nm, j2, S.az);
+      if constexpr (FUSED) {
+        const unsigned long long sc = mul2(p.nm, F);
+        S.bx = fma2(sc, p.dx, S.bx);
+        S.by = fma2(sc, p.dy, S.by);
+        S.bz = fma2(sc, p.dz, S.bz);
+      }
+      // sum over the 8 targets: each step exchanges half of the values with
+      // the partner lane, so that lane (k, t) ends with one of the eight sums
+      // (slot 2k + bit 2 of t, component t & 3)
+      const bool s2 = lane & 4, s1 = lane & 2, s0 = lane & 1;
+      float c0 = s2 ? hi2(j0) : lo2(j0), c1 = s2 ? hi2(j1) : lo2(j1);
+      float c2 = s2 ? hi2(j2) : lo2(j2), c3 = s2 ? hi2(js) : lo2(js);
+      c0 += __shfl_xor_sync(0xffffffffu, s2 ? lo2(j0) : hi2(j0), 4);
+      c1 += __shfl_xor_sync(0xffffffffu, s2 ? lo2(j1) : hi2(j1), 4);
+      c2 += __shfl_xor_sync(0xffffffffu, s2 ? lo2(j2) : hi2(j2), 4);
+      c3 += __shfl_xor_sync(0xffffffffu, s2 ? lo2(js) : hi2(js), 4);
+      float d0 = s1 ? c2 : c0, d1 = s1 ? c3 : c1;
+      d0 += __shfl_xor_sync(0xffffffffu, s1 ? c0 : c2, 2);
+      d1 += __shfl_xor_sync(0xffffffffu, s1 ? c1 : c3, 2);
+      float v = s0 ? d1 : d0;
+      v += __shfl_xor_sync(0xffffffffu, s0 ? d0 : d1, 1);
+      if (own) (&M.SG[0].x)[8 * k + (lane & 7)] -= v;
+    }
+  }
+
+  // Outside the softening length and below the cut band: the packed form holds.
+  __device__ __forceinline__ bool plain(const WalkArgs& A, float r2, float h2) const {
+    return r2 < A.pp_lo && r2 >= h2;
+  }
+
+  // The packed force factors of both slots, zero where h0 / h1 is false.
+  __device__ __forceinline__ void force_pair(const WalkArgs& A, const Pair& p, bool h0, bool h1,
+                                             unsigned long long& F, unsigned long long& Fr) const {
+    const unsigned long long ri = pack2(rsqrt_approx(lo2(p.r2)), rsqrt_approx(hi2(p.r2)));
+    const unsigned long long r = mul2(p.r2, ri);
+    const unsigned long long ri2 = mul2(ri, ri);
+    const unsigned long long K = mul2(ri2, ri);
+    const unsigned long long ea = mul2(p.r2, pack2(A.ex2c, A.ex2c));
+    const unsigned long long ex = pack2(ex2_approx(lo2(ea)), ex2_approx(hi2(ea)));
+    const unsigned long long f = mul2(sr_poly2(fma2(r, pack2(A.t_scale, A.t_scale), pack2(-1.0f, -1.0f))), ex);
+    F = mul2(K, f);
+    F = pack2(h0 ? lo2(F) : 0.f, h1 ? hi2(F) : 0.f);
+    if constexpr (ADJ) {
+      // F'/r = (K'/r) f + K f'/r, K'/r = -3 K / r^2, f'(r)/r = fp_c r exp(-u^2)
+      Fr = fma2(mul2(mul2(pack2(-3.0f, -3.0f), K), ri2), f, mul2(K, mul2(mul2(pack2(A.fp_c, A.fp_c), ex), r)));
+      Fr = pack2(h0 ? lo2(Fr) : 0.f, h1 ? hi2(Fr) : 0.f);
+    }
+  }
+
+  // A pair the packed form does not cover: the exact cut (an accepted node is
+  // inside by decision, a particle in the band is decided in FP64), then the
+  // force with the softened kernel.  False if outside the cut.
+  __device__ __forceinline__ bool force_rare(const WalkArgs& A, const Stage& St, int64_t i, int s, float r2, float h2,
+                                             float& F, float& Fr) const {
+    if (!(r2 < A.pp_lo)) {
+      const int id = St.id[s];
+      if (id >= 0 && !pair_inside_exact(A, i, id)) return false;
+    }
+    force_f32<ADJ>(A, r2, h2, F, Fr);
+    return true;
+  }
+
+  // One FP32 batch: the cnt staged sources, as pairs of adjacent slots.
+  //
+  // Tile: a warp iteration takes the 8 targets of one sub-group against 4
+  // slot pairs (8 sources), lane = (pair of the four, target of the eight),
+  // each lane both sources of its pair in packed arithmetic.  A sub-group
+  // lists the slot pairs with a source inside the cut of its box.  The 8
+  // targets lie close together and adjacent slots come from one leaf, so
+  // about half of the 64 (target, source) pairs of an iteration are hits
+  // (a third of a whole group's would be).  A target's sum stays in
+  // registers over the sub-group's iterations and is reduced over its four
+  // lanes once per batch.  Measured against listing the pairs one by one,
+  // 32 per iteration, with a segmented scan for the sums (full lanes, but the
+  // list, the gathered operands and the scan cost two thirds of the pair
+  // work): forward 3.17 -> 2.68 ms on the 128^3 lattice, 23.2 -> 19.2 ms on the
+  // 128^3 clustered set, 0.66 -> 0.36 ms on 4096 particles (one group per SM);
+  // adjoint 4.61 -> 3.73 and 33.3 -> 25.0 ms.  Loading the next iteration's pair
+  // before the current one is evaluated is a fifth of that on 4096 particles.
+  __device__ void batch_tiles(const WalkArgs& A, const WarpBufs& W, Stage& St, Smem& M, const float4* SGB,
+                              int cnt, int lane, int64_t gbase, uint32_t vmask, bool mi) {
+    // an odd count leaves the last pair's second slot empty: its data must be finite
+    if ((cnt & 1) && lane < 8) {
+      float4* p = lane < 2 ? &St.s0[cnt >> 1] : lane < 4 ? &St.s1[cnt >> 1] : lane < 6 ? &St.s2[cnt >> 1] : &St.s3[cnt >> 1];
+      (&p->x)[2 * (lane & 1) + 1] = 0.f;
+    }
+    const uint2 qq = *reinterpret_cast<const uint2*>(St.sq + 2 * lane);
+    const bool has0 = 2 * lane < cnt, has1 = 2 * lane + 1 < cnt;
+    const uint32_t q0 = has0 ? qq.x : 0u, q1 = has1 ? qq.y : 0u;
+    // lane = slot pair: the sub-groups within reach of either slot's source
+    // (the source's distance to the padded box; the exact cut is taken per
+    // pair), listed per sub-group
+    unsigned char* list = reinterpret_cast<unsigned char*>(W.list);
+    const uint32_t lt = (1u << lane) - 1u;
+    const float reach2 = mi ? 8.0f : A.grp_rc2;  // without a common image every pair is listed
+    uint32_t U = 0;  // slot pairs listed for this lane's sub-group
+    {
+      const float4 v0 = St.s0[lane], v1 = St.s1[lane];
+#pragma unroll
+      for (int g = 0; g < kSub; ++g) {
+        const float4 c4 = SGB[2 * g], e4 = SGB[2 * g + 1];
+        const unsigned long long x = add2(pack2(c4.x, c4.x), pack2(v0.x, v0.y));
+        const unsigned long long y = add2(pack2(c4.y, c4.y), pack2(v0.z, v0.w));
+        const unsigned long long z = add2(pack2(c4.z, c4.z), pack2(v1.x, v1.y));
+        const unsigned long long gx = pack2(fmaxf(fabsf(lo2(x)) - e4.x, 0.f), fmaxf(fabsf(hi2(x)) - e4.x, 0.f));
+        const unsigned long long gy = pack2(fmaxf(fabsf(lo2(y)) - e4.y, 0.f), fmaxf(fabsf(hi2(y)) - e4.y, 0.f));
+        const unsigned long long gz = pack2(fmaxf(fabsf(lo2(z)) - e4.z, 0.f), fmaxf(fabsf(hi2(z)) - e4.z, 0.f));
+        const unsigned long long g2 = fma2(gx, gx, fma2(gy, gy, mul2(gz, gz)));
+        const uint32_t gm = 0xffu << (8 * g);
+        const bool in0 = (q0 & gm) != 0u && lo2(g2) <= reach2;
+        const bool in1 = (q1 & gm) != 0u && hi2(g2) <= reach2;
+        const uint32_t um = __ballot_sync(0xffffffffu, in0 || in1);
+        if ((um >> lane) & 1u) list[32 * g + __popc(um & lt)] = (unsigned char)lane;
+        if ((lane >> 3) == g) U = um;
+      }
+    }
+    // bit k of m0 / m1: slot 2k / 2k + 1 holds a source of this lane's target
+    uint32_t m0, m1;
+    if (__any_sync(0xffffffffu, (has0 && q0 != vmask) || (has1 && q1 != vmask))) {
+      m0 = transpose32<ADJ ? 5 : 1>(q0, lane);
+      m1 = transpose32<ADJ ? 5 : 1>(q1, lane);
+    } else {
+      m0 = valid ? low_bits((cnt + 1) >> 1) : 0u;
+      m1 = valid ? low_bits(cnt >> 1) : 0u;
+    }
+    const int so = M.self[lane];
+    if (so >= 0) {
+      const uint32_t others = ~(1u << (so >> 1));
+      if (so & 1) m1 &= others;
+      else m0 &= others;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int g = 0; g < kSub; ++g) {
+      const int n = __popc(__shfl_sync(0xffffffffu, U, 8 * g));
+      if (n == 0) continue;
+      const int t = 8 * g + (lane & 7);
+      const uint32_t q0m = __shfl_sync(0xffffffffu, m0, t), q1m = __shfl_sync(0xffffffffu, m1, t);
+      int hits = 0;
+      Target T;
+      {
+        const float4 ta = M.tA[t], tb = M.tB[t];
+        T.x = pack2(ta.x, ta.x); T.y = pack2(ta.y, ta.y); T.z = pack2(ta.z, ta.z);
+        T.u = pack2(tb.x, tb.x); T.v = pack2(tb.y, tb.y); T.w = pack2(tb.z, tb.z);
+        T.h2 = ta.w;
+        if constexpr (ADJ) {
+          const float4 w = M.tW[t];
+          T.wx = pack2(w.x, w.x); T.wy = pack2(w.y, w.y); T.wz = pack2(w.z, w.z);
+        }
+      }
+      Sums S = {0, 0, 0, 0, 0, 0};
+      uint32_t rare = 0u;  // bit i: iteration i of the list holds a pair the packed form does not cover
+      // the next iteration's pair is loaded, up to its squared distances,
+      // before the current one is evaluated
+      int kn = list[32 * g + min(lane >> 3, n - 1)];
+      Pair pn = load_pair(St, T, kn, mi);
+#pragma unroll 1
+      for (int e0 = 0; e0 < n; e0 += 4) {
+        const int e = e0 + (lane >> 3);
+        const int k = kn;
+        const Pair p = pn;
+        kn = list[32 * g + min(e + 4, n - 1)];
+        pn = load_pair(St, T, kn, mi);
+        const bool h0 = e < n && ((q0m >> k) & 1u) && lo2(p.r2) <= A.pp_hi;
+        const bool h1 = e < n && ((q1m >> k) & 1u) && hi2(p.r2) <= A.pp_hi;
+        const bool p0 = h0 && plain(A, lo2(p.r2), p.h20), p1 = h1 && plain(A, hi2(p.r2), p.h21);
+        if (h0 != p0 || h1 != p1) rare |= 1u << (e0 >> 2);
+        hits += (p0 ? 1 : 0) + (p1 ? 1 : 0);
+        unsigned long long F, Fr = 0;
+        force_pair(A, p, p0, p1, F, Fr);
+        add_pair(M, T, p, F, Fr, k, e < n, lane, S);
+      }
+      rare = __reduce_or_sync(0xffffffffu, rare);
+#pragma unroll 1
+      while (rare) {
+        const int e0 = 4 * (__ffs(rare) - 1);
+        rare &= rare - 1u;
+        const int e = e0 + (lane >> 3);
+        const int k = list[32 * g + min(e, n - 1)];
+        const Pair p = load_pair(St, T, k, mi);
+        float F[2] = {0.f, 0.f}, Fr[2] = {0.f, 0.f};
+#pragma unroll 1
+        for (int c = 0; c < 2; ++c) {
+          const float r2 = c ? hi2(p.r2) : lo2(p.r2), h2 = c ? p.h21 : p.h20;
+          const bool h = e < n && (((c ? q1m : q0m) >> k) & 1u) && r2 <= A.pp_hi;
+          float f = 0.f, fr = 0.f;
+          if (h && !plain(A, r2, h2) && force_rare(A, St, gbase + t, 2 * k + c, r2, h2, f, fr)) ++hits;
+          if (c) { F[1] = f; Fr[1] = fr; }
+          else { F[0] = f; Fr[0] = fr; }
+        }
+        add_pair(M, T, p, pack2(F[0], F[1]), pack2(Fr[0], Fr[1]), k, e < n, lane, S);
+      }
+      // the target's sum over its four lanes (even and odd slots first)
+      float p0 = lo2(S.ax) + hi2(S.ax), p1 = lo2(S.ay) + hi2(S.ay), p2 = lo2(S.az) + hi2(S.az);
+      p0 += __shfl_xor_sync(0xffffffffu, p0, 8);
+      p1 += __shfl_xor_sync(0xffffffffu, p1, 8);
+      p2 += __shfl_xor_sync(0xffffffffu, p2, 8);
+      p0 += __shfl_xor_sync(0xffffffffu, p0, 16);
+      p1 += __shfl_xor_sync(0xffffffffu, p1, 16);
+      p2 += __shfl_xor_sync(0xffffffffu, p2, 16);
+      hits += __shfl_xor_sync(0xffffffffu, hits, 8);
+      hits += __shfl_xor_sync(0xffffffffu, hits, 16);
+      if ((lane >> 3) == g) {
+        nint += hits;
+        P[0] = p0;
+        P[1] = p1;
+        P[2] = p2;
+      }
+      if constexpr (FUSED) {
+        float f0 = lo2(S.bx) + hi2(S.bx), f1 = lo2(S.by) + hi2(S.by), f2 = lo2(S.bz) + hi2(S.bz);
+        f0 += __shfl_xor_sync(0xffffffffu, f0, 8);
+        f1 += __shfl_xor_sync(0xffffffffu, f1, 8);
+        f2 += __shfl_xor_sync(0xffffffffu, f2, 8);
+        f0 += __shfl_xor_sync(0xffffffffu, f0, 16);
+        f1 += __shfl_xor_sync(0xffffffffu, f1, 16);
+        f2 += __shfl_xor_sync(0xffffffffu, f2, 16);
+        if ((lane >> 3) == g) {
+          Pf[0] = f0;
+          Pf[1] = f1;
+          Pf[2] = f2;
+        }
+      }
+      __syncwarp();  // the slots' sums of this sub-group before the next one's
+    }
+    M.self[lane] = -1;
+    fold();
+    if constexpr (ADJ) {
+#pragma unroll 1
+      for (int u = 0; u < 2; ++u) {
+        const int s = lane + 32 * u;
+        const float4 g = M.SG[s];
+        if (s < cnt && (g.x != 0.f || g.y != 0.f || g.z != 0.f || g.w != 0.f)) {
+          const int id = St.id[s];
+          double* Gd = id >= 0 ? A.Gp + 3 * (int64_t)id : A.Gn + 3 * (int64_t)(-2 - id);
+          double* Sd = id >= 0 ? A.Sp + id : A.Sn + (-2 - id);
+          atomicAdd(Gd, f2d_exact(g.x));
+          atomicAdd(Gd + 1, f2d_exact(g.y));
+          atomicAdd(Gd + 2, f2d_exact(g.z));
+          atomicAdd(Sd, f2d_exact(g.w));
+        }
+        M.SG[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+    __syncwarp();
+  }
+
+  // One FP64 batch: the cnt staged sources at slots [hb, hb + cnt).  The FP64
+  // pipe runs a warp instruction at the same cost however few lanes are
+  // active, so the hit pairs are listed and each iteration evaluates 32.
+  __device__ void batch_list(const WalkArgs& A, const WarpBufs& W, Stage& St, Smem& M, int hb, int cnt, int lane,
+                             int64_t gbase, uint32_t vmask) {
+    // bit s of msk: slot s is in this lane's part of its entry's lane mask
+    const bool has = lane < cnt;
+    const uint32_t q = has ? St.sq[hb + lane] : 0u;
+    uint32_t msk;
+    if (__any_sync(0xffffffffu, has && q != vmask)) msk = transpose32<1>(q, lane);
+    else msk = valid ? low_bits(cnt) : 0u;
+    // conservative cut test for all 32 slots; the sign bit of each result is
+    // shifted into acc (slot 0 ends up at bit 31)
+    uint32_t acc = 0;
+    const Filter f = filter();
+#pragma unroll
+    for (int s = 0; s < kSlots; s += 4) {
+      unsigned long long r01, r23;
+      f.four(St, hb + s, r01, r23);
       acc = __funnelshift_l((uint32_t)r01, acc, 1);
       acc = __funnelshift_l((uint32_t)(r01 >> 32), acc, 1);
       acc = __funnelshift_l((uint32_t)r23, acc, 1);
@@ -749,6 +1055,7 @@ struct LaneFP {
     // a batch with more pairs than the list holds is processed in two
     // halves of its slots (at most 32 x 16 pairs each)
     const bool split = nhit > kList;
+#pragma unroll 1
     for (int part = 0; part < (split ? 2 : 1); ++part) {
       const uint32_t hp = split ? (hit & (part == 0 ? 0x0000ffffu : 0xffff0000u)) : hit;
       // compaction: target-major pair list
@@ -772,148 +1079,57 @@ struct LaneFP {
       }
       nint += c;  // listed pairs; those outside the exact cut are subtracted below
       __syncwarp();
-      {
-        const int we = T;
-        for (int p0 = 0; p0 < we; p0 += 32) {
-          const int p = p0 + lane;
-          const bool hv = p < we;
-          int i = 0, slot = 0;
-          Term<F64> r;
-          r.x = r.y = r.z = 0;
-          r.w = 0.f;
-          float4 sg = make_float4(0.f, 0.f, 0.f, 0.f);
-          float3 fw = make_float3(0.f, 0.f, 0.f);
-          if (hv) {
-            const int e = W.list[p];
-            i = e >> 5;
-            slot = e & 31;
-            if constexpr (F64) {
-              r = pair_eval64(A, St, i, hb + slot, gbase);
-            } else {
-              const float4 rr = pair_eval(A, St, M, i, hb + slot, gbase, sg, fw);
-              r.x = rr.x;
-              r.y = rr.y;
-              r.z = rr.z;
-              r.w = rr.w;
-            }
-            if (r.w == 0.f) atomicAdd(&M.fneg[i], 1);
-          }
-          // segmented inclusive scan over the lanes: the pairs of one target
-          // are consecutive, so each target's run is summed in a fixed tree
-          // order and its last lane adds the sum to the target's batch total
-          const int oi = __shfl_sync(0xffffffffu, off, i);
-          const int ci = __shfl_sync(0xffffffffu, c, i);
-          const int first = max(oi - p0, 0);
-          // the longest run reaching back into this iteration: steps beyond
-          // it add nothing (warp-uniform, so skipping them changes no sum)
-          const int span = (int)__reduce_max_sync(0xffffffffu, (unsigned)(hv ? lane - first : 0));
+#pragma unroll 1
+      for (int p0 = 0; p0 < T; p0 += 32) {
+        const int p = p0 + lane;
+        const bool hv = p < T;
+        int i = 0;
+        Term64 r = {0.0, 0.0, 0.0, false};
+        if (hv) {
+          const int e = W.list[p];
+          i = e >> 5;
+          r = pair_eval64(A, St, i, hb + (e & 31), gbase);
+          if (!r.in) atomicAdd(&M.fneg[i], 1);
+        }
+        // segmented inclusive scan over the lanes: the pairs of one target
+        // are consecutive, so each target's run is summed in a fixed tree
+        // order and its last lane adds the sum to the target's batch total
+        const int oi = __shfl_sync(0xffffffffu, off, i);
+        const int ci = __shfl_sync(0xffffffffu, c, i);
+        const int first = max(oi - p0, 0);
+        // the longest run reaching back into this iteration: steps beyond
+        // it add nothing (warp-uniform, so skipping them changes no sum)
+        const int span = (int)__reduce_max_sync(0xffffffffu, (unsigned)(hv ? lane - first : 0));
 #pragma unroll
-          for (int d = 1; d < 32; d <<= 1) {
-            if (d > 4 && span < d) break;
-            const auto y0 = __shfl_up_sync(0xffffffffu, r.x, d);
-            const auto y1 = __shfl_up_sync(0xffffffffu, r.y, d);
-            const auto y2 = __shfl_up_sync(0xffffffffu, r.z, d);
-            if (lane - d >= first) {
-              r.x += y0;
-              r.y += y1;
-              r.z += y2;
-            }
-            if constexpr (FUSED) {
-              const float f0 = __shfl_up_sync(0xffffffffu, fw.x, d);
-              const float f1 = __shfl_up_sync(0xffffffffu, fw.y, d);
-              const float f2 = __shfl_up_sync(0xffffffffu, fw.z, d);
-              if (lane - d >= first) {
-                fw.x += f0;
-                fw.y += f1;
-                fw.z += f2;
-              }
-            }
+        for (int d = 1; d < 32; d <<= 1) {
+          if (d > 4 && span < d) break;
+          const double y0 = __shfl_up_sync(0xffffffffu, r.x, d);
+          const double y1 = __shfl_up_sync(0xffffffffu, r.y, d);
+          const double y2 = __shfl_up_sync(0xffffffffu, r.z, d);
+          if (lane - d >= first) {
+            r.x += y0;
+            r.y += y1;
+            r.z += y2;
           }
-          if (hv && p == min(min(oi + ci, we), p0 + 32) - 1) {
-            auto a = M.Ps[i];
-            a.x += r.x;
-            a.y += r.y;
-            a.z += r.z;
-            M.Ps[i] = a;
-            if constexpr (FUSED) {
-              float4 b = M.Pf[i];
-              b.x += fw.x;
-              b.y += fw.y;
-              b.z += fw.z;
-              M.Pf[i] = b;
-            }
-          }
-          if (ADJ) {
-            // source-side terms: each listed pair's term goes to shared
-            // memory with its lane bit in its slot's mask; the lane that owns
-            // the slot sums them in lane order and adds the sum to its batch
-            // total, kept in registers
-            M.SG[lane] = sg;
-            if (hv) atomicOr(&M.smask[slot], 1u << lane);
-            __syncwarp();
-            uint32_t mk = M.smask[lane];
-            if (mk) {
-              M.smask[lane] = 0u;
-              float4 acc = M.SG[__ffs(mk) - 1];
-              mk &= mk - 1u;
-              while (mk) {
-                const float4 v = M.SG[__ffs(mk) - 1];
-                acc.x += v.x;
-                acc.y += v.y;
-                acc.z += v.z;
-                acc.w += v.w;
-                mk &= mk - 1u;
-              }
-              gs.x += acc.x;
-              gs.y += acc.y;
-              gs.z += acc.z;
-              gs.w += acc.w;
-            }
-          }
-          __syncwarp();
+        }
+        if (hv && p == min(min(oi + ci, T), p0 + 32) - 1) {
+          double3 a = M.Ps[i];
+          a.x += r.x;
+          a.y += r.y;
+          a.z += r.z;
+          M.Ps[i] = a;
         }
         __syncwarp();
       }
     }
-    // this batch's sums (at most 32 terms per target) into the Kahan totals
-    // (FP64 variant: into the plain double sums)
-    {
-      const auto ps = M.Ps[lane];
-      if constexpr (F64) {
-        a64[0] += ps.x;
-        a64[1] += ps.y;
-        a64[2] += ps.z;
-        M.Ps[lane] = make_double3(0.0, 0.0, 0.0);
-      } else {
-        P[0] += ps.x;
-        P[1] += ps.y;
-        P[2] += ps.z;
-        M.Ps[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if constexpr (FUSED) {
-          const float4 pf = M.Pf[lane];
-          Pf[0] += pf.x;
-          Pf[1] += pf.y;
-          Pf[2] += pf.z;
-          M.Pf[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-      }
-      nint -= M.fneg[lane];
-      M.fneg[lane] = 0;
-    }
-    if constexpr (!F64) fold();
-    if (ADJ) {
-      const float4 g = gs;
-      if (has && (g.x != 0.f || g.y != 0.f || g.z != 0.f || g.w != 0.f)) {
-        const int id = St.sc[hb + lane].x;
-        double* Gd = id >= 0 ? A.Gp + 3 * (int64_t)id : A.Gn + 3 * (int64_t)(-2 - id);
-        double* Sd = id >= 0 ? A.Sp + id : A.Sn + (-2 - id);
-        atomicAdd(Gd, f2d_exact(g.x));
-        atomicAdd(Gd + 1, f2d_exact(g.y));
-        atomicAdd(Gd + 2, f2d_exact(g.z));
-        atomicAdd(Sd, f2d_exact(g.w));
-      }
-      gs = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    // this batch's sums into the plain double sums
+    const double3 ps = M.Ps[lane];
+    a64[0] += ps.x;
+    a64[1] += ps.y;
+    a64[2] += ps.z;
+    M.Ps[lane] = make_double3(0.0, 0.0, 0.0);
+    nint -= M.fneg[lane];
+    M.fneg[lane] = 0;
     // this batch held the target's own slot
     if (self_here) M.self[lane] = -1;
     __syncwarp();
@@ -960,7 +1176,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
   __shared__ int2 s_stack[kWarpsPerBlock][kStack];
   __shared__ int4 s_queue[kWarpsPerBlock][kQueue];
   __shared__ int s_qoff[kWarpsPerBlock][kQueue + 1];
-  __shared__ unsigned short s_list[kWarpsPerBlock][kList];
+  __shared__ unsigned short s_list[kWarpsPerBlock][Lane::kListSize];
   __shared__ WarpScratch<Lane> s_scr[kWarpsPerBlock];
   __shared__ typename Lane::Smem s_lane[kWarpsPerBlock];
   __shared__ float4 s_sgb[kWarpsPerBlock][2 * kSub];
@@ -1002,6 +1218,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
   typename Lane::Stage& St = s_scr[wib].stage;
   typename Lane::Smem& M = s_lane[wib];
   int nodes_total = 0;
+#pragma unroll 1
   for (int l = 0; l < kLevels; ++l) nodes_total += T.sb->level_cnt[l];
   if (nodes_total > T.cap) nodes_total = (int)T.cap;
 
@@ -1134,29 +1351,26 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
       // OPEN leaves and ACCEPTed nodes: queue them for evaluation
       const bool q = (cls == CL_OPEN && leaf) || cls == CL_ACCEPT;
       const uint32_t qm = __ballot_sync(0xffffffffu, q);
-      if (q) {
-        const int fl = image_flags(A, G, NC);
+      if (q)
         W.queue[nq + __popc(qm & lt)] =
-            cls == CL_ACCEPT ? make_int4(node, -1, (int)mask, fl) : make_int4(ND.x, ND.y, (int)mask, fl);
-      }
+            cls == CL_ACCEPT ? make_int4(node, -1, (int)mask, 0) : make_int4(ND.x, ND.y, (int)mask, 0);
       nq += __popc(qm);
-      // MIXED nodes: exact decisions for every (node, target in its mask),
-      // 32 at a time from a node-major list; the results are OR-ed into
+      // MIXED nodes: decisions for the targets in their masks, OR-ed into
       // per-node accept / open masks
       const uint32_t mm = __ballot_sync(0xffffffffu, cls == CL_MIXED);
       if (mm) {
         const int nm = __popc(mm);
         if (cls == CL_MIXED) {
           const int ix = __popc(mm & lt);
-          const int xfl = image_flags(A, G, NC);
+          float sx, sy, sz;
+          const bool uni = node_image(A, G, NC, sx, sy, sz);
           float4 SC = NC, SA = NA;
-          if (xfl & 1) {
-            const float sx = shift_of(xfl, 0), sy = shift_of(xfl, 1), sz = shift_of(xfl, 2);
+          if (uni) {
             SC.x -= sx; SC.y -= sy; SC.z -= sz;
             SA.x -= sx; SA.y -= sy; SA.z -= sz;
           }
           X.node[ix] = node;
-          X.fl[ix] = xfl;
+          X.fl[ix] = uni ? 1 : 0;
           X.D[ix] = ND;
           X.C[ix] = SC;
           X.A[ix] = SA;
@@ -1164,46 +1378,50 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
           X.mask[ix] = mask & vmask;
           X.acc[ix] = 0u;
           X.open[ix] = 0u;
-          X.dmask[ix] = 0u;
         }
         __syncwarp();
         // each (node, sub-group) pair is first classified against the
-        // sub-group's box; only undecided sub-groups need per-lane decisions
-        for (int j = lane; j < kSub * nm; j += 32) {
+        // sub-group's box; the undecided ones are listed
+        int nd = 0;
+#pragma unroll 1
+        for (int j0 = 0; j0 < kSub * nm; j0 += 32) {
+          const int j = j0 + lane;
           const int ix = j >> 2, g = j & 3;
-          const uint32_t gm = X.mask[ix] & (0xffu << (8 * g));
+          int cg = CL_NONE;
+          const uint32_t gm = j < kSub * nm ? X.mask[ix] & (0xffu << (8 * g)) : 0u;
           if (gm) {
             const float4 c4 = SGB[2 * g], e4 = SGB[2 * g + 1];
             GroupInfo Gs;
             Gs.cx = c4.x; Gs.cy = c4.y; Gs.cz = c4.z;
             Gs.ex = e4.x; Gs.ey = e4.y; Gs.ez = e4.z;
-            const int cg = classify(A, Gs, X.C[ix], X.A[ix], X.B[ix]);
+            cg = classify(A, Gs, X.C[ix], X.A[ix], X.B[ix]);
             if (cg == CL_OPEN) atomicOr(&X.open[ix], gm);
             else if (cg == CL_ACCEPT) atomicOr(&X.acc[ix], gm);
-            else if (cg == CL_MIXED) atomicOr(&X.dmask[ix], gm);
+          }
+          const uint32_t um = __ballot_sync(0xffffffffu, cg == CL_MIXED);
+          if (cg == CL_MIXED) W.list[nd + __popc(um & lt)] = (unsigned short)j;
+          nd += __popc(um);
+        }
+        __syncwarp();
+        // per-target decisions, four listed (node, sub-group) pairs at a
+        // time: lane = (pair of the four, target of the eight)
+#pragma unroll 1
+        for (int d0 = 0; d0 < nd; d0 += 4) {
+          const int d = d0 + (lane >> 3);
+          const int j = W.list[min(d, nd - 1)];
+          const int ix = j >> 2, t = 8 * (j & 3) + (lane & 7);
+          int dec = DEC_DISCARD;
+          if (d < nd && ((X.mask[ix] >> t) & 1u))
+            dec = decide_f32(A, gbase + t, M.tA[t], M.tB[t], X.node[ix], meta_level(X.D[ix].w), X.C[ix], X.A[ix],
+                             X.B[ix], X.fl[ix] != 0);
+          const uint32_t da = (__ballot_sync(0xffffffffu, dec == DEC_ACCEPT) >> (lane & 24)) & 0xffu;
+          const uint32_t dn = (__ballot_sync(0xffffffffu, dec == DEC_OPEN) >> (lane & 24)) & 0xffu;
+          if ((lane & 7) == 0) {
+            if (da) atomicOr(&X.acc[ix], da << (8 * (j & 3)));
+            if (dn) atomicOr(&X.open[ix], dn << (8 * (j & 3)));
           }
         }
         __syncwarp();
-        // at most kList / 32 nodes per list
-        for (int m0 = 0; m0 < nm; m0 += kList / 32) {
-          const int m1 = min(nm, m0 + kList / 32);
-          int nd = 0;
-          for (int ix = m0; ix < m1; ++ix) {
-            const uint32_t mk = X.dmask[ix];
-            if ((mk >> lane) & 1u) W.list[nd + __popc(mk & lt)] = (unsigned short)((ix << 5) | lane);
-            nd += __popc(mk);
-          }
-          __syncwarp();
-          for (int d = lane; d < nd; d += 32) {
-            const int e = W.list[d];
-            const int ix = e >> 5, t = e & 31;
-            const int dec =
-                L.decide_for(A, M, t, gbase + t, X.node[ix], X.D[ix], X.C[ix], X.A[ix], X.B[ix], (X.fl[ix] & 1) != 0);
-            if (dec == DEC_ACCEPT) atomicOr(&X.acc[ix], 1u << t);
-            else if (dec == DEC_OPEN) atomicOr(&X.open[ix], 1u << t);
-          }
-          __syncwarp();
-        }
         const bool hm = lane < nm;
         const int hx = hm ? lane : 0;
         const uint32_t am = hm ? X.acc[hx] : 0u;
@@ -1211,14 +1429,13 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
         const int4 XD = X.D[hx];
         const int xnode = X.node[hx];
         const bool xleaf = meta_leaf(XD.w);
-        const int fl = X.fl[hx];
         const bool qa = am != 0u, qo = om != 0u && xleaf, po = om != 0u && !xleaf;
         const uint32_t ba = __ballot_sync(0xffffffffu, qa);
         const uint32_t bo = __ballot_sync(0xffffffffu, qo);
         const uint32_t bp = __ballot_sync(0xffffffffu, po);
-        if (qa) W.queue[nq + __popc(ba & lt)] = make_int4(xnode, -1, (int)am, fl);
+        if (qa) W.queue[nq + __popc(ba & lt)] = make_int4(xnode, -1, (int)am, 0);
         nq += __popc(ba);
-        if (qo) W.queue[nq + __popc(bo & lt)] = make_int4(XD.x, XD.y, (int)om, fl);
+        if (qo) W.queue[nq + __popc(bo & lt)] = make_int4(XD.x, XD.y, (int)om, 0);
         nq += __popc(bo);
         if (po)
           W.stack[sp + __popc(bp & lt)] =
@@ -1227,7 +1444,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
       }
       __syncwarp();
     } else if (nq > 0) {
-      L.evaluate(A, W, St, M, nq, lane, G, gbase, vmask, Rg);
+      L.evaluate(A, W, St, M, nq, lane, G, SGB, gbase, vmask, Rg);
       nq = 0;
       __syncwarp();
     } else {
