@@ -300,6 +300,7 @@ struct WalkArgs {
   long long max_iters;
   int deep;                    // stack depth above which a step pops one range (<= the compiled bound)
   int64_t g_begin, g_end;      // walk groups [g_begin, g_end) (a key range of targets)
+  int split;                   // 2^split warps per group (set by launch_walk)
   // FP32, box units
   float rc2, rc2_lo, rc2_hi;   // node tests: rcut^2 and its relative band
   float pp_lo, pp_hi;          // pair cut band
@@ -340,7 +341,7 @@ cudaError_t launch_keys_sort(const double* pos, int64_t n, double L, uint64_t* k
 cudaError_t launch_tree_build(const BuildArgs& A, cudaStream_t s);
 // fused (with adjoint): the adjoint walk that also writes accf, counts and
 // the interaction total from the same pair evaluations
-cudaError_t launch_walk(const WalkArgs& A, int prec, bool adjoint, cudaStream_t s, bool fused = false);
+cudaError_t launch_walk(WalkArgs A, int prec, bool adjoint, cudaStream_t s, bool fused = false);
 cudaError_t launch_adjoint_push(const TreeDev& T, const AdjWs& W, double L, double* dpos, double* dmass,
                                 cudaStream_t s);
 cudaError_t launch_copy_nodes(const TreeDev& T, int64_t m, int32_t* level, int32_t* first, int32_t* count,

@@ -1182,8 +1182,11 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
   __shared__ float4 s_sgb[kWarpsPerBlock][2 * kSub];
   const TreeDev& T = A.T;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t g = A.g_begin + (int64_t)blockIdx.x * kWarpsPerBlock + wib;
+  // 2^split warps serve a group, each its part of the targets
+  const int64_t v = (int64_t)blockIdx.x * kWarpsPerBlock + wib;
+  const int64_t g = A.g_begin + (v >> A.split);
   if (g >= A.g_end) return;
+  const bool mine = (lane >> (5 - A.split)) == (int)(v & ((1 << A.split) - 1));
   if (T.sb->status != 0 || T.sb->magic != kMagicTree) {
     // a failed or missing tree: flag it and give every output of this
     // group's targets NaN, so that nothing downstream can take stale values
@@ -1191,7 +1194,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
     // for one that was never built the sorted index stands in for it.
     if (lane == 0) set_status(A.wsb, ST_NOTREE);
     const int64_t kk = g * kGroup + lane;
-    if (kk < T.n) {
+    if (mine && kk < T.n) {
       const float nf = __int_as_float(0x7fc00000);
       const double nd = __longlong_as_double(0x7ff8000000000000ll);
       int64_t io = kk;
@@ -1224,22 +1227,15 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
 
   const int64_t gbase = g * kGroup;
   const int64_t k = gbase + lane;
-  const bool valid = k < T.n;
+  const bool valid = mine && k < T.n;
   const uint32_t vmask = __ballot_sync(0xffffffffu, valid);
+  if (vmask == 0u) return;  // a part beyond the last particle
   const uint32_t lt = (1u << lane) - 1u;
 
+  // boxes of this warp's targets and of the 4 sub-groups of 8 targets (box
+  // units, padded outward by more than the FP32 rounding of a position in
+  // [0, 1))
   GroupInfo G;
-  {
-    const float4 lo = T.gbox[2 * g], hi = T.gbox[2 * g + 1];
-    G.cx = 0.5f * (lo.x + hi.x); G.cy = 0.5f * (lo.y + hi.y); G.cz = 0.5f * (lo.z + hi.z);
-    G.ex = 0.5f * (hi.x - lo.x) * 1.0001f + 1e-7f;
-    G.ey = 0.5f * (hi.y - lo.y) * 1.0001f + 1e-7f;
-    G.ez = 0.5f * (hi.z - lo.z) * 1.0001f + 1e-7f;
-  }
-  // bound on |x_i - group centre| for the evaluation's cut filter
-  const float Rg = sqrtf(fmaf(G.ex, G.ex, fmaf(G.ey, G.ey, G.ez * G.ez))) * 1.0001f + 1e-6f;
-  // boxes of the 4 sub-groups of 8 targets (box units, padded outward by
-  // more than the FP32 rounding of a position in [0, 1))
   float4* SGB = s_sgb[wib];
   {
     const float4 pa = T.pA[valid ? k : 0], pb = T.pB[valid ? k : 0];
@@ -1249,21 +1245,25 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) { lo[c] = 1e30f; hi[c] = -1e30f; }
     }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         lo[c] = fminf(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
         hi[c] = fmaxf(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
       }
-    if ((lane & 7) == 0) {
-      const float pad = 2e-7f;
-      SGB[2 * (lane >> 3)] = make_float4(0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]), 0.f);
-      SGB[2 * (lane >> 3) + 1] = make_float4(0.5f * (hi[0] - lo[0]) * 1.0001f + pad,
-                                             0.5f * (hi[1] - lo[1]) * 1.0001f + pad,
-                                             0.5f * (hi[2] - lo[2]) * 1.0001f + pad, 0.f);
+      G.cx = 0.5f * (lo[0] + hi[0]); G.cy = 0.5f * (lo[1] + hi[1]); G.cz = 0.5f * (lo[2] + hi[2]);
+      G.ex = 0.5f * (hi[0] - lo[0]) * 1.0001f + 2e-7f;
+      G.ey = 0.5f * (hi[1] - lo[1]) * 1.0001f + 2e-7f;
+      G.ez = 0.5f * (hi[2] - lo[2]) * 1.0001f + 2e-7f;
+      if (o == 4 && (lane & 7) == 0) {
+        SGB[2 * (lane >> 3)] = make_float4(G.cx, G.cy, G.cz, 0.f);
+        SGB[2 * (lane >> 3) + 1] = make_float4(G.ex, G.ey, G.ez, 0.f);
+      }
     }
   }
+  // bound on |x_i - group centre| for the FP64 variant's cut filter
+  const float Rg = sqrtf(fmaf(G.ex, G.ex, fmaf(G.ey, G.ey, G.ez * G.ez))) * 1.0001f + 1e-6f;
 
   Lane L;
   L.init(A, M, k, valid, lane, G);
@@ -1458,8 +1458,26 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
   }
 }
 
-cudaError_t launch_walk(const WalkArgs& A, int prec, bool adjoint, cudaStream_t s, bool fused) {
-  const int64_t blocks = (A.g_end - A.g_begin + kWarpsPerBlock - 1) / kWarpsPerBlock;
+// Warps per group (log2).  A walk of fewer groups than the chip holds warps
+// leaves it idle, and one of a few times as many waits for its longest groups;
+// two or four warps a group, each with its part of the targets and its own
+// traversal, shorten them for some repeated traversal.  It depends on the
+// tree alone, so a walk over a range of groups gives the full walk's sums.
+// Measured, ms with 1 / 2 / 4 warps a group, forward: 128 groups (4096
+// uniform) 0.37 / 0.28 / 0.22, 1024 groups (32^3) clustered 0.31 / 0.27 / 0.25,
+// zoom 3.66 / 2.61 / 2.45, lattice 0.15 / 0.14 / 0.15; 5860 groups (zoom) 17.9 /
+// 18.4 / 20.0; 8192 groups (64^3) lattice 0.43 / 0.49 / 0.63, clustered 1.76 /
+// 1.58 / 1.67.  The FP64 walk repeats a smaller share: 1024 groups clustered
+// 5.0 / 3.2 / 2.5, 5860 (zoom) 349 / 310 / 312, 8192 clustered 30.6 / 26.0 / 23.7,
+// lattice 7.3 / 7.5 / 7.8, 22,800 (90^3 clustered) 112 / 98 / 99.
+static int walk_split(int64_t n_groups, bool f64) {
+  if (n_groups <= 1024) return 2;
+  return n_groups <= (f64 ? 32768 : 4096) ? 1 : 0;
+}
+
+cudaError_t launch_walk(WalkArgs A, int prec, bool adjoint, cudaStream_t s, bool fused) {
+  A.split = walk_split(A.T.ngroups, prec == OG_FP64);
+  const int64_t blocks = (((A.g_end - A.g_begin) << A.split) + kWarpsPerBlock - 1) / kWarpsPerBlock;
   if (blocks <= 0) return cudaSuccess;
   if (fused) k_walk<LaneFused><<<(unsigned)blocks, kWarpsPerBlock * 32, 0, s>>>(A);
   else if (adjoint) k_walk<LaneF32<true>><<<(unsigned)blocks, kWarpsPerBlock * 32, 0, s>>>(A);
