@@ -10,11 +10,26 @@
 // parity fold is a bit-parallel suffix XOR and the final interleave uses
 // magic-mask bit spreading.
 //
-// K2: 8 passes of 8-bit digits (63-bit keys).  Each pass is a per-tile digit
-// histogram, a per-digit scan over tiles, and a stable scatter that ranks
-// equal digits with warp match masks, stages the tile in shared memory in
-// digit order and writes contiguous runs.  Stability of every pass gives the
-// (key, original index) order.  HBM-bound: ~32 B per key per pass.
+// K2: 8 passes of 8-bit digits (63-bit keys), one launch each.  K1 counts all
+// eight digits' histograms while it writes the keys.  A pass ranks its tile's
+// keys by digit with warp match masks, publishes the tile's digit counts, and
+// finds the keys of equal digit in the tiles before it by looking back over
+// their published counts (a tile publishes its own counts first and the sum
+// up to itself once it knows it, so a look-back ends at the nearest sum);
+// then it stages the tile in shared memory in digit order and writes
+// contiguous runs.  Tiles are numbered by a counter as blocks start, so every
+// tile that is looked back at is running or done.  Stability of every pass
+// gives the (key, original index) order.
+//
+// Bound by HBM: 220 B a key (32 for the keys, 20 for the first pass, whose
+// values are the indices themselves, 24 for each other pass), against 310 B and 25
+// launches for a histogram, a scan and a scatter per pass.
+// Measured (keys and sort): 4096 keys 95 -> 78 us, 2.1 M 0.38 -> 0.26 ms, 5.0 M
+// clustered 0.69 -> 0.48, 16.8 M 2.07 -> 1.38.  A pass takes 2.4 times its memory
+// time at 16.8 M keys: a tile's chain of ranking, look-back and scattered writes
+// is 12 us long and three tiles fit an SM.  Tile shapes, 5.0 M / 16.8 M: 256 x 16 keys
+// 0.481 / 1.38 ms, 256 x 12 0.488 / 1.43, 384 x 16 0.488 / 1.43, 512 x 8 0.52 / 1.57, 256 x 8
+// 0.55 / 1.63; predecessors read at a time 4 / 8 / 16: 0.481 / 0.488 / 0.524 ms at 5.0 M.
 #include "og_internal.cuh"
 
 namespace og {
@@ -65,9 +80,18 @@ __device__ __forceinline__ uint64_t hilbert63(uint32_t a, uint32_t b, uint32_t c
   return (spread3(a) << 2) | (spread3(b) << 1) | spread3(c);
 }
 
-__global__ void k_keys(const double* __restrict__ pos, int64_t n, BoxScale B, uint64_t* __restrict__ keys,
-                       int32_t* __restrict__ vals, StatusBlock* sb) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+constexpr int kKeyThreads = 256;
+
+__global__ void __launch_bounds__(kKeyThreads) k_keys(const double* __restrict__ pos, int64_t n, BoxScale B,
+                                                      uint64_t* __restrict__ keys, SortWs W) {
+  __shared__ uint32_t h[8 * 256];
+  for (int i = threadIdx.x; i < 8 * 256; i += kKeyThreads) h[i] = 0u;
+  __syncthreads();
+  const int64_t stride = (int64_t)gridDim.x * kKeyThreads;
+  const int64_t first = blockIdx.x * (int64_t)kKeyThreads + threadIdx.x;
+  // the first pass's tile counts start at zero
+  for (int64_t i = first; i < W.ntiles * 256; i += stride) W.tile_state[0][i] = 0u;
+  for (int64_t i = first; i < n; i += stride) {
     const double x0 = pos[3 * i], x1 = pos[3 * i + 1], x2 = pos[3 * i + 2];
     uint64_t key = 0;
     if (finite_bits(x0) && finite_bits(x1) && finite_bits(x2)) {
@@ -76,182 +100,192 @@ __global__ void k_keys(const double* __restrict__ pos, int64_t n, BoxScale B, ui
       const uint32_t q2 = quantise(wrap_coord(x2, B), B);
       key = hilbert63(q0, q1, q2);
     } else {
-      set_status(sb, ST_BADINPUT);
+      set_status(W.sb, ST_BADINPUT);
     }
     keys[i] = key;
-    vals[i] = static_cast<int32_t>(i);
+#pragma unroll
+    for (int d = 0; d < 8; ++d) atomicAdd(&h[256 * d + ((key >> (8 * d)) & 255u)], 1u);
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 8 * 256; i += kKeyThreads)
+    if (h[i]) atomicAdd(&W.hist[i], h[i]);
 }
 
-// Exclusive scan of one value per thread over a block of 256 threads.
-__device__ __forceinline__ uint32_t block_exscan256(uint32_t v, uint32_t* s_warp, uint32_t* total) {
+// A tile's published state for one digit: 0 nothing yet, 1 + count its own
+// count, kStateSum | sum the keys of the digit in all tiles up to it.
+constexpr uint32_t kStateSum = 1u << 31;
+// Polls of one state before a look-back gives up (seconds, far above any
+// tile's run time; the tiles looked at are always running).
+constexpr int kStatePolls = 1 << 22;
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kStateAhead = 4;
+
+// Shared memory of a pass (dynamic: above the static limit).
+struct SortSmem {
+  uint64_t keys[kSortTile];
+  int32_t vals[kSortTile];
+  uint32_t wcnt[kSortWarps][256];
+  uint32_t base[256];  // where the tile's first key of each digit goes, less its place in the tile
+  unsigned long long scan[8];
+  uint32_t tile;
+};
+
+template <bool FIRST>
+__global__ void __launch_bounds__(kSortThreads, 3)
+    k_sort_pass(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin, int64_t n, int pass, SortWs W,
+                uint64_t* __restrict__ kout, int32_t* __restrict__ vout) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  SortSmem& S = *reinterpret_cast<SortSmem*>(s_raw);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  uint32_t x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) s_warp[w] = x;
+  const int shift = 8 * pass;
+  if (threadIdx.x == 0) S.tile = (uint32_t)atomicAdd(&W.sb->pad[pass], 1);
+  for (int i = threadIdx.x; i < kSortWarps * 256; i += kSortThreads) (&S.wcnt[0][0])[i] = 0u;
   __syncthreads();
-  if (w == 0) {
-    uint32_t t = lane < 8 ? s_warp[lane] : 0u;
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-      uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
-      if (lane >= o) t += y;
-    }
-    if (lane < 8) s_warp[lane] = t;  // inclusive
-  }
-  __syncthreads();
-  const uint32_t warp_off = w ? s_warp[w - 1] : 0u;
-  if (total) *total = s_warp[7];
-  const uint32_t r = warp_off + x - v;
-  __syncthreads();
-  return r;
-}
-
-__global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint64_t* __restrict__ keys, int64_t n, int shift,
-                                                            uint32_t* __restrict__ hist, int64_t nblk) {
-  __shared__ uint32_t h[256];
-  h[threadIdx.x] = 0;
-  __syncthreads();
-  const int64_t base = blockIdx.x * (int64_t)kSortTile;
-#pragma unroll
-  for (int k = 0; k < kSortItems; ++k) {
-    const int64_t idx = base + k * kSortThreads + threadIdx.x;
-    if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & 255u], 1u);
-  }
-  __syncthreads();
-  hist[threadIdx.x * nblk + blockIdx.x] = h[threadIdx.x];
-}
-
-// One block per digit: exclusive scan over tiles, in place; digit total out.
-__global__ void __launch_bounds__(1024) k_sort_scan(uint32_t* hist, int64_t nblk, uint32_t* digit_tot) {
-  __shared__ uint32_t s_w[32];
-  __shared__ uint32_t s_carry;
-  uint32_t* row = hist + blockIdx.x * nblk;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (threadIdx.x == 0) s_carry = 0;
-  __syncthreads();
-  for (int64_t base = 0; base < nblk; base += 1024) {
-    const int64_t i = base + threadIdx.x;
-    const uint32_t v = i < nblk ? row[i] : 0u;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) s_w[w] = x;
-    __syncthreads();
-    if (w == 0) {
-      uint32_t t = s_w[lane];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t += y;
-      }
-      s_w[lane] = t;
-    }
-    __syncthreads();
-    const uint32_t carry = s_carry;
-    const uint32_t excl = carry + (w ? s_w[w - 1] : 0u) + x - v;
-    if (i < nblk) row[i] = excl;
-    __syncthreads();
-    if (threadIdx.x == 0) s_carry = carry + s_w[31];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) digit_tot[blockIdx.x] = s_carry;
-}
-
-__global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const uint64_t* __restrict__ kin,
-                                                               const int32_t* __restrict__ vin, int64_t n, int shift,
-                                                               const uint32_t* __restrict__ hist, int64_t nblk,
-                                                               const uint32_t* __restrict__ digit_tot,
-                                                               uint64_t* __restrict__ kout, int32_t* __restrict__ vout) {
-  __shared__ uint32_t s_wcnt[kSortThreads / 32][256];
-  __shared__ uint32_t s_tile_start[256];
-  __shared__ uint32_t s_gbase[256];
-  __shared__ uint32_t s_scan[8];
-  __shared__ uint64_t s_keys[kSortTile];
-  __shared__ int32_t s_vals[kSortTile];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t base = blockIdx.x * (int64_t)kSortTile;
+  const int64_t tile = S.tile;
+  const int64_t base = tile * kSortTile;
   const int tile_n = (int)((n - base) < kSortTile ? (n - base) : kSortTile);
-  for (int i = threadIdx.x; i < (kSortThreads / 32) * 256; i += kSortThreads) (&s_wcnt[0][0])[i] = 0u;
-  __syncthreads();
+  const int l0 = w * 32 * kSortItems + lane;  // this lane's first key of the tile
 
   uint64_t key[kSortItems];
-  int32_t val[kSortItems];
-  uint32_t rank[kSortItems];
+  uint32_t place[kSortItems];
   const uint32_t lt = (1u << lane) - 1u;
+  // padding slots lie behind every key of the tile: the largest digit keeps them last
+#pragma unroll
+  for (int k = 0; k < kSortItems; ++k) key[k] = l0 + 32 * k < tile_n ? kin[base + l0 + 32 * k] : ~0ull;
+  // rank among the warp's keys of the same digit: the first of the 32 lanes
+  // with the digit takes their number from the warp's counter; the rounds'
+  // atomics go out in order and are not waited for between rounds
 #pragma unroll
   for (int k = 0; k < kSortItems; ++k) {
-    const int li = w * 32 * kSortItems + k * 32 + lane;
-    const bool valid = li < tile_n;
-    key[k] = valid ? kin[base + li] : 0ull;
-    val[k] = valid ? vin[base + li] : 0;
-    const uint32_t d = valid ? (uint32_t)((key[k] >> shift) & 255u) : 256u;
-    const uint32_t peers = __match_any_sync(0xffffffffu, d);
-    const uint32_t before = valid ? s_wcnt[w][d] : 0u;
-    rank[k] = before + __popc(peers & lt);
-    __syncwarp();
-    if (valid && lane == __ffs(peers) - 1) s_wcnt[w][d] = before + __popc(peers);
-    __syncwarp();
-  }
-  __syncthreads();
-  // per digit: offsets of each warp inside the tile's run of that digit
-  const int d = threadIdx.x;
-  uint32_t run = 0;
+    const uint32_t d = (uint32_t)((key[k] >> shift) & 255u);
+    uint32_t peers = 0xffffffffu;
 #pragma unroll
-  for (int ww = 0; ww < kSortThreads / 32; ++ww) {
-    const uint32_t c = s_wcnt[ww][d];
-    s_wcnt[ww][d] = run;
-    run += c;
-  }
-  uint32_t tot_all;
-  const uint32_t tstart = block_exscan256(run, s_scan, &tot_all);
-  s_tile_start[d] = tstart;
-  const uint32_t dbase = block_exscan256(digit_tot[d], s_scan, nullptr);
-  s_gbase[d] = dbase + hist[d * nblk + blockIdx.x];
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < kSortItems; ++k) {
-    const int li = w * 32 * kSortItems + k * 32 + lane;
-    if (li < tile_n) {
-      const uint32_t dd = (uint32_t)((key[k] >> shift) & 255u);
-      const uint32_t p = s_tile_start[dd] + s_wcnt[w][dd] + rank[k];
-      s_keys[p] = key[k];
-      s_vals[p] = val[k];
+    for (int b = 0; b < 8; ++b) {
+      const uint32_t v = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+      peers &= (d >> b) & 1u ? v : ~v;
     }
+    const int first = __ffs(peers) - 1;
+    uint32_t before = 0;
+    if (lane == first) before = atomicAdd(&S.wcnt[w][d], (uint32_t)__popc(peers));
+    __syncwarp();
+    place[k] = __shfl_sync(0xffffffffu, before, first) + __popc(peers & lt);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < tile_n; i += kSortThreads) {
-    const uint64_t kk = s_keys[i];
-    const uint32_t dd = (uint32_t)((kk >> shift) & 255u);
-    const uint32_t o = s_gbase[dd] + (uint32_t)i - s_tile_start[dd];
-    kout[o] = kk;
-    vout[o] = s_vals[i];
+  // thread d serves digit d: the warps' offsets inside the tile's run of the
+  // digit, then one scan over the digits of (tile count, global count)
+  const int d = threadIdx.x;
+  uint32_t* state = W.tile_state[pass & 1];
+  uint32_t cnt = 0;
+  unsigned long long x = 0, own = 0;
+  if (d < 256) {
+    const uint32_t all = W.hist[256 * pass + d];
+#pragma unroll
+    for (int ww = 0; ww < kSortWarps; ++ww) {
+      const uint32_t c = S.wcnt[ww][d];
+      S.wcnt[ww][d] = cnt;
+      cnt += c;
+    }
+    own = ((unsigned long long)cnt << 32) | all;
+    if (d == 255) cnt -= (uint32_t)(kSortTile - tile_n);  // less the padding
+    __stcg(&state[tile * 256 + d], tile == 0 ? (kStateSum | cnt) : cnt + 1u);
+    if (pass < 7) W.tile_state[(pass + 1) & 1][tile * 256 + d] = 0u;  // the next pass's
+    x = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) S.scan[w] = x;
+  }
+  __syncthreads();
+  uint32_t tstart = 0, gbase = 0;
+  if (d < 256) {
+    for (int ww = 0; ww < w; ++ww) x += S.scan[ww];
+    x -= own;
+    tstart = (uint32_t)(x >> 32);
+    gbase = (uint32_t)x;
+#pragma unroll
+    for (int ww = 0; ww < kSortWarps; ++ww) S.wcnt[ww][d] += tstart;
+  }
+  __syncthreads();
+  // the tile in digit order
+  int32_t val[kSortItems];
+#pragma unroll
+  for (int k = 0; k < kSortItems; ++k) {
+    place[k] += S.wcnt[w][(key[k] >> shift) & 255u];
+    S.keys[place[k]] = key[k];
+  }
+#pragma unroll
+  for (int k = 0; k < kSortItems; ++k)
+    val[k] = FIRST ? (int32_t)(base + l0 + 32 * k) : l0 + 32 * k < tile_n ? vin[base + l0 + 32 * k] : 0;
+  // keys of this digit in the tiles before
+  if (d < 256) {
+    uint32_t sum = 0;
+    if (tile > 0) {
+      int64_t t = tile - 1;
+      int polls = 0;
+      for (;;) {
+        // several predecessors at a time: their loads are independent
+        uint32_t st[kStateAhead];
+#pragma unroll
+        for (int u = 0; u < kStateAhead; ++u) st[u] = t - u >= 0 ? __ldcg(state + (t - u) * 256 + d) : kStateSum;
+        bool done = false;
+        int used = 0;
+#pragma unroll
+        for (int u = 0; u < kStateAhead; ++u) {
+          if (done || used < u || st[u] == 0u) continue;
+          ++used;
+          done = (st[u] & kStateSum) != 0u;
+          sum += done ? st[u] & ~kStateSum : st[u] - 1u;
+        }
+        if (done) break;
+        t -= used;
+        if (used == 0 && ++polls > kStatePolls) {
+          set_status(W.sb, ST_WALKCAP);
+          break;
+        }
+      }
+      __stcg(&state[tile * 256 + d], kStateSum | (sum + cnt));
+    }
+    S.base[d] = gbase + sum - tstart;
+  }
+#pragma unroll
+  for (int k = 0; k < kSortItems; ++k) S.vals[place[k]] = val[k];
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kSortItems; ++k) key[k] = S.keys[k * kSortThreads + threadIdx.x];
+#pragma unroll
+  for (int k = 0; k < kSortItems; ++k) val[k] = S.vals[k * kSortThreads + threadIdx.x];
+#pragma unroll
+  for (int k = 0; k < kSortItems; ++k) place[k] = S.base[(key[k] >> shift) & 255u] + (uint32_t)(k * kSortThreads + threadIdx.x);
+#pragma unroll
+  for (int k = 0; k < kSortItems; ++k) {
+    if (k * kSortThreads + (int)threadIdx.x < tile_n && (int64_t)place[k] < n) {
+      kout[place[k]] = key[k];
+      vout[place[k]] = val[k];
+    }
   }
 }
 
 cudaError_t launch_keys_sort(const double* pos, int64_t n, double L, uint64_t* keys_out, int32_t* order_out,
                              const SortWs& W, cudaStream_t s) {
-  const int kb = 256;
-  int64_t kgrid = (n + kb - 1) / kb;
-  if (kgrid > grid_cap(64)) kgrid = grid_cap(64);
-  k_keys<<<(unsigned)kgrid, kb, 0, s>>>(pos, n, box_scale(L), keys_out, order_out, W.sb);
+  // status, tile counters and histograms start at zero
+  cudaError_t e = cudaMemsetAsync(W.sb, 0, kSortZeroBytes, s);
+  if (e != cudaSuccess) return e;
+  int64_t kgrid = (n + kKeyThreads - 1) / kKeyThreads;
+  if (kgrid > grid_cap(8)) kgrid = grid_cap(8);
+  k_keys<<<(unsigned)kgrid, kKeyThreads, 0, s>>>(pos, n, box_scale(L), keys_out, W);
   uint64_t* kin = keys_out;
   int32_t* vin = order_out;
   uint64_t* ko = W.keys_alt;
   int32_t* vo = W.vals_alt;
+  e = cudaFuncSetAttribute(k_sort_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_sort_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
+  if (e != cudaSuccess) return e;
   for (int pass = 0; pass < 8; ++pass) {
-    const int shift = 8 * pass;
-    k_sort_hist<<<(unsigned)W.nblk, kSortThreads, 0, s>>>(kin, n, shift, W.hist, W.nblk);
-    k_sort_scan<<<256, 1024, 0, s>>>(W.hist, W.nblk, W.digit_tot);
-    k_sort_scatter<<<(unsigned)W.nblk, kSortThreads, 0, s>>>(kin, vin, n, shift, W.hist, W.nblk, W.digit_tot, ko,
-                                                             vo);
+    auto kernel = pass == 0 ? k_sort_pass<true> : k_sort_pass<false>;
+    kernel<<<(unsigned)W.ntiles, kSortThreads, sizeof(SortSmem), s>>>(kin, vin, n, pass, W, ko, vo);
     uint64_t* tk = kin; kin = ko; ko = tk;
     int32_t* tv = vin; vin = vo; vo = tv;
   }
@@ -270,13 +304,11 @@ namespace {
 
 constexpr int64_t kNoAllocMaxN = int64_t(1) << 20;
 constexpr size_t noalloc_round(size_t x) { return (x + og::kAlign - 1) / og::kAlign * og::kAlign; }
-// Same carving as og::carve_sort: status block, alternate keys, alternate
-// indices, per-tile digit histograms, digit totals.
+// Same carving as og::carve_sort: status block, histograms, alternate keys,
+// alternate indices, two passes' tile counts.
 constexpr size_t kNoAllocBytes =
-    noalloc_round(sizeof(og::StatusBlock)) + noalloc_round(sizeof(uint64_t) * kNoAllocMaxN) +
-    noalloc_round(sizeof(int32_t) * kNoAllocMaxN) +
-    noalloc_round(sizeof(uint32_t) * 256 * ((kNoAllocMaxN + og::kSortTile - 1) / og::kSortTile)) +
-    noalloc_round(sizeof(uint32_t) * 256);
+    og::kSortZeroBytes + noalloc_round(sizeof(uint64_t) * kNoAllocMaxN) + noalloc_round(sizeof(int32_t) * kNoAllocMaxN) +
+    2 * noalloc_round(sizeof(uint32_t) * 256 * ((kNoAllocMaxN + og::kSortTile - 1) / og::kSortTile));
 
 // Held by every GPU that loads the library, until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_sort_ws[kNoAllocBytes];
@@ -309,7 +341,5 @@ extern "C" og_status og_keys_sort_noalloc(const double* pos, int64_t n, double b
   og::SortWs W;
   if (og::carve_sort(base, n, &W) > kNoAllocBytes) return OG_ENOSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // the array keeps the previous call's contents: the status block starts at zero
-  if (cudaMemsetAsync(W.sb, 0, sizeof(og::StatusBlock), s) != cudaSuccess) return OG_ECUDA;
   return og::launch_keys_sort(pos, n, box, keys_sorted, order, W, s) == cudaSuccess ? OG_OK : OG_ECUDA;
 }

@@ -70,8 +70,6 @@ og_status og_keys_sort(const double* pos, int64_t n, double box, uint64_t* keys_
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   SortWs W;
   carve_sort(ws, n, &W);
-  cudaError_t e = cudaMemsetAsync(W.sb, 0, sizeof(StatusBlock), s);
-  if (e != cudaSuccess) return OG_ECUDA;
   return cuda_status(launch_keys_sort(pos, n, box, keys_sorted, order, W, s));
 }
 

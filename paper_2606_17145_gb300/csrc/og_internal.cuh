@@ -130,17 +130,18 @@ inline TreeDev tree_view(const og_tree* t) {
 
 // Keys-sort workspace.
 struct SortWs {
-  StatusBlock* sb;
+  StatusBlock* sb;         // pad[pass]: the pass's tile counter
+  uint32_t* hist;          // [8][256] digit counts of all keys
   uint64_t* keys_alt;
   int32_t* vals_alt;
-  uint32_t* hist;       // [256][nblk]
-  uint32_t* digit_tot;  // [256]
-  int64_t nblk;
+  uint32_t* tile_state[2]; // [ntiles][256], even and odd passes
+  int64_t ntiles;
 };
 
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;
-constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per block
+constexpr int kSortItems = 16;
+constexpr int kSortTile = kSortThreads * kSortItems;  // 4096 keys per block
+constexpr size_t kSortZeroBytes = kAlign + sizeof(uint32_t) * 8 * 256;  // status block and histograms
 
 inline size_t carve_sort(void* buf, int64_t n, SortWs* W) {
   size_t off = 0;
@@ -151,12 +152,12 @@ inline size_t carve_sort(void* buf, int64_t n, SortWs* W) {
     return p;
   };
   SortWs w{};
-  w.nblk = (n + kSortTile - 1) / kSortTile;
+  w.ntiles = (n + kSortTile - 1) / kSortTile;
   w.sb = static_cast<StatusBlock*>(take(sizeof(StatusBlock)));
+  w.hist = static_cast<uint32_t*>(take(sizeof(uint32_t) * 8 * 256));
   w.keys_alt = static_cast<uint64_t*>(take(sizeof(uint64_t) * n));
   w.vals_alt = static_cast<int32_t*>(take(sizeof(int32_t) * n));
-  w.hist = static_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * w.nblk));
-  w.digit_tot = static_cast<uint32_t*>(take(sizeof(uint32_t) * 256));
+  for (int i = 0; i < 2; ++i) w.tile_state[i] = static_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * w.ntiles));
   if (W) *W = w;
   return off;
 }
