@@ -26,6 +26,7 @@ enum : uint32_t {
 constexpr int kMaxLevel = 21;         // 21 bits per axis
 constexpr int kLevels = kMaxLevel + 1;
 constexpr int kGroup = 32;            // targets per walk group (one warp)
+constexpr int kTopoBlock = 512;       // keys per block of the tree build's topology passes
 constexpr size_t kAlign = 256;
 
 // The first 256 bytes of every buffer the library carves.
@@ -68,8 +69,6 @@ struct TreeDev {
   double* h64;     // [n] softening support h = 2.8 eps
   int32_t* order;  // [n] sorted -> original index
   int32_t* leaf_of;// [n] leaf node of each sorted particle
-  // groups of 32
-  float4* gbox;    // [2 * ngroups]: min (xyz), max (xyz) in box units, rounded outward
   // nodes
   float4* nA;      // (com_hi xyz, M / L^2)
   float4* nB;      // (com_lo xyz, hmax / L)
@@ -81,6 +80,8 @@ struct TreeDev {
   double* mass64;  // [cap]
   double* hmax64;  // [cap]
   double* cen64;   // [cap][3] physical geometric centres
+  int* blk;        // [kLevels][nblk] build scratch: nodes of each level per block of kTopoBlock keys
+  int64_t nblk;
 };
 
 // Carves a tree buffer.  Returns the total byte count (buf may be null).
@@ -105,7 +106,6 @@ inline size_t carve_tree(void* buf, int64_t n, int64_t cap, TreeDev* T) {
   t.h64 = static_cast<double*>(take(sizeof(double) * n));
   t.order = static_cast<int32_t*>(take(sizeof(int32_t) * n));
   t.leaf_of = static_cast<int32_t*>(take(sizeof(int32_t) * n));
-  t.gbox = static_cast<float4*>(take(sizeof(float4) * 2 * G));
   t.nA = static_cast<float4*>(take(sizeof(float4) * cap));
   t.nB = static_cast<float4*>(take(sizeof(float4) * cap));
   t.nC = static_cast<float4*>(take(sizeof(float4) * cap));
@@ -116,6 +116,8 @@ inline size_t carve_tree(void* buf, int64_t n, int64_t cap, TreeDev* T) {
   t.mass64 = static_cast<double*>(take(sizeof(double) * cap));
   t.hmax64 = static_cast<double*>(take(sizeof(double) * cap));
   t.cen64 = static_cast<double*>(take(sizeof(double) * 3 * cap));
+  t.nblk = (n + kTopoBlock - 1) / kTopoBlock;
+  t.blk = static_cast<int*>(take(sizeof(int) * kLevels * t.nblk));
   if (T) *T = t;
   return off;
 }

@@ -1,18 +1,31 @@
-// tree_build.cu -- K3 permute, K4 level-by-level octree build, K5 walk groups.
+// tree_build.cu -- K3 permute, K4 octree build.
 //
-// Nodes are stored level by level (level-major), so the children of a node are
-// a contiguous range of the next level.  A node is a maximal run of sorted
-// keys sharing the top 3*level bits; it is split (level < 21, more than
-// leaf_size members) into the runs of its 8 possible next digits.
+// Nodes are stored level by level (level-major), each level in the order of
+// the sorted keys, so the children of a node are a contiguous range of the
+// next level.  A node is a maximal run of sorted keys sharing the top 3*level
+// bits; it is split (level < 21, more than leaf_size members) into the runs
+// of its 8 possible next digits.
 //
-// Top-down topology: one launch per level.  Eight lanes serve one parent; lane
-// d binary-searches the first key whose next digit is >= d inside the
-// parent's range, so the child runs come out without touching every key.
-// Child slots are taken per block with a single atomic on the level counter.
+// Topology without a pass per level.  With L_i the number of digits key i
+// shares with key i - 1, and D_i the deepest level at which more than
+// leaf_size keys around i share a prefix (the largest common prefix of two
+// keys leaf_size apart with i between them), the nodes that start at key i are
+// those of the levels L_i + 1 .. D_i + 1, and all but the deepest are split.  So
+// one pass counts the nodes of each level per block, a scan over the blocks
+// gives every node its index, and a second pass writes them.
 //
-// Bottom-up moments: one launch per level, deepest first.  One thread serves
-// one node and sums its children (or a leaf's particles) in FP64 in index
-// order, so the result does not depend on scheduling.
+// Moments: all leaves in one launch, then the split nodes from the deepest
+// level up in one cooperative launch with a grid barrier per level (one block
+// alone where the levels are small).  One thread serves one node and sums its
+// children (or a leaf's particles) in FP64 in index order, so the result does
+// not depend on scheduling.
+//
+// A launch and its gap cost 2 - 3 us: a launch per level and direction (46 in
+// all) cost 180 us on 4096 particles, most of it for empty levels.  Whole force
+// passes, build alone changed: 4096 particles 500 -> 294 us, 64^3 leapfrog step
+// 1050 -> 887 us, 100,003-particle SPH 1.15 -> 0.96 ms.  At 2.1 M particles the
+// kernels take 0.095 (permute), 0.02, 0.008, 0.083 (fill: the searches for the
+// ends of runs), 0.049 (leaves) and 0.09 ms (upward).
 #include "og_internal.cuh"
 
 namespace og {
@@ -58,41 +71,79 @@ __global__ void k_permute(BuildArgs A, BoxScale B) {
   }
 }
 
-__global__ void k_groups(TreeDev T, BoxScale B) {
-  // Wrapped positions are non-negative doubles, which order like their bit
-  // patterns, and division by L is monotonic: the box in box units is the
-  // division of the integer min / max.
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < T.ngroups; g += (int64_t)gridDim.x * blockDim.x) {
-    long long lo[3] = {0x7fffffffffffffffll, 0x7fffffffffffffffll, 0x7fffffffffffffffll};
-    long long hi[3] = {0, 0, 0};
-    const int64_t a = g * kGroup, b = (T.n < a + kGroup ? T.n : a + kGroup);
-    for (int64_t k = a; k < b; ++k)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const long long x = __double_as_longlong(T.x64[3 * k + c]);
-        lo[c] = x < lo[c] ? x : lo[c];
-        hi[c] = x > hi[c] ? x : hi[c];
-      }
-    float fl[3], fh[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      fl[c] = __double2float_rd(div_box(__longlong_as_double(lo[c]), B));
-      fh[c] = __double2float_ru(div_box(__longlong_as_double(hi[c]), B));
-    }
-    T.gbox[2 * g] = make_float4(fl[0], fl[1], fl[2], 0.f);
-    T.gbox[2 * g + 1] = make_float4(fh[0], fh[1], fh[2], 0.f);
-  }
+constexpr int kTopoThreads = kTopoBlock;
+constexpr int kMaxLeaf = 32;        // largest leaf_size
+
+// Octal digits two 63-bit keys share from the top (0 .. 21).
+__device__ __forceinline__ int common_digits(uint64_t a, uint64_t b) {
+  const uint64_t x = a ^ b;
+  return x == 0 ? kMaxLevel : (__clzll((long long)x) - 1) / 3;
 }
 
-__global__ void k_root(TreeDev T, int leaf_size) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    T.sb->magic = kMagicTree;
-    for (int l = 0; l < 24; ++l) T.sb->level_cnt[l] = 0;
-    T.sb->level_cnt[0] = 1;
-    const int leaf = (T.n <= leaf_size) ? 1 : 0;
-    T.nD[0] = make_int4(0, (int)T.n, -1, make_meta(0, 0, leaf));
-    T.nParent[0] = -1;
+// Levels [lo, hi] of the nodes that start at sorted key i of this block (none
+// if lo > hi); deep: the deepest level whose run around i is split (-1: none).
+// Every thread of the block calls it.
+__device__ __forceinline__ void node_levels(const uint64_t* __restrict__ keys, int64_t n, int leaf_size, int64_t i0,
+                                            signed char* s_far, int& lo, int& hi, int& deep) {
+  // s_far[j]: digits shared by keys i0 - leaf_size + j and i0 + j
+  for (int j = threadIdx.x; j < kTopoThreads + leaf_size; j += kTopoThreads) {
+    const int64_t a = i0 - leaf_size + j, b = i0 + j;
+    s_far[j] = (signed char)(a >= 0 && b < n ? common_digits(keys[a], keys[b]) : -1);
   }
+  __syncthreads();
+  const int64_t i = i0 + threadIdx.x;
+  lo = 1;
+  hi = 0;
+  deep = -1;
+  if (i < n) {
+    for (int j = 0; j <= leaf_size; ++j) deep = max(deep, (int)s_far[threadIdx.x + j]);
+    lo = i == 0 ? 0 : common_digits(keys[i - 1], keys[i]) + 1;
+    hi = min(deep + 1, kMaxLevel);
+  }
+  deep = min(deep, kMaxLevel - 1);
+}
+
+// Nodes of each level that start in this block's keys.
+__global__ void __launch_bounds__(kTopoThreads) k_count(TreeDev T, const uint64_t* __restrict__ keys, int leaf_size) {
+  __shared__ signed char s_far[kTopoThreads + kMaxLeaf];
+  __shared__ int s_cnt[kLevels];
+  if (blockIdx.x == 0 && threadIdx.x == 0) T.sb->magic = kMagicTree;
+  if (threadIdx.x < kLevels) s_cnt[threadIdx.x] = 0;
+  int lo, hi, deep;
+  node_levels(keys, T.n, leaf_size, blockIdx.x * (int64_t)kTopoThreads, s_far, lo, hi, deep);
+  for (int l = lo; l <= hi; ++l) atomicAdd(&s_cnt[l], 1);
+  __syncthreads();
+  if (threadIdx.x < kLevels) T.blk[threadIdx.x * T.nblk + blockIdx.x] = s_cnt[threadIdx.x];
+}
+
+// One block per level: exclusive scan of its counts over the blocks, in
+// place, and the level's total.
+__global__ void __launch_bounds__(1024) k_scan(TreeDev T) {
+  __shared__ int s_w[32];
+  int* row = T.blk + blockIdx.x * T.nblk;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int carry = 0;
+  for (int64_t b0 = 0; b0 < T.nblk; b0 += 1024) {
+    const int64_t i = b0 + threadIdx.x;
+    const int v = i < T.nblk ? row[i] : 0;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_w[w] = x;
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int ww = 0; ww < 32; ++ww) {
+      if (ww < w) before += s_w[ww];
+      all += s_w[ww];
+    }
+    if (i < T.nblk) row[i] = carry + before + x - v;
+    carry += all;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) T.sb->level_cnt[blockIdx.x] = carry;
 }
 
 __device__ __forceinline__ int level_base(const StatusBlock* sb, int level) {
@@ -101,158 +152,236 @@ __device__ __forceinline__ int level_base(const StatusBlock* sb, int level) {
   return b;
 }
 
-// Expand level `lev` into level lev + 1.  256 threads = 32 parents per step.
-__global__ void __launch_bounds__(256) k_expand(TreeDev T, const uint64_t* __restrict__ keys, int lev, int leaf_size) {
-  __shared__ int s_cnt[32];
-  __shared__ int s_base;
-  const int base = level_base(T.sb, lev);
-  const int cnt = T.sb->level_cnt[lev];
-  const int next_base = base + cnt;
-  if (next_base > T.cap) return;  // capacity exceeded at an upper level (flagged there)
-  const int lane = threadIdx.x & 31;
-  const int sub = lane & 7;                      // digit handled by this lane
-  const int slot = threadIdx.x >> 3;             // parent slot in the block (0..31)
-  const int shift = 63 - 3 * (lev + 1);
-  for (int step = blockIdx.x * 32; step < cnt; step += gridDim.x * 32) {
-    const int p = base + step + slot;
-    const bool live = (step + slot) < cnt;
-    int4 D = make_int4(0, 0, -1, 0);
-    bool split = false;
-    if (live) {
-      D = T.nD[p];
-      split = !meta_leaf(D.w);
+// Writes the nodes' ranges.  nchild and the parent links follow with the
+// moments, where a node meets its children.
+__global__ void __launch_bounds__(kTopoThreads) k_fill(TreeDev T, const uint64_t* __restrict__ keys, int leaf_size) {
+  __shared__ signed char s_far[kTopoThreads + kMaxLeaf];
+  __shared__ int s_first[kLevels];                      // index of this block's first node of each level
+  __shared__ int s_warp[kTopoThreads / 32][kLevels];    // nodes of each level in each warp, then in the warps before it
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (threadIdx.x < kLevels) {
+    s_first[threadIdx.x] = level_base(T.sb, threadIdx.x) + T.blk[threadIdx.x * T.nblk + blockIdx.x];
+#pragma unroll
+    for (int ww = 0; ww < kTopoThreads / 32; ++ww) s_warp[ww][threadIdx.x] = 0;
+  }
+  int lo, hi, deep;
+  const int64_t i = blockIdx.x * (int64_t)kTopoThreads + threadIdx.x;
+  node_levels(keys, T.n, leaf_size, blockIdx.x * (int64_t)kTopoThreads, s_far, lo, hi, deep);
+  const bool any = lo <= hi;
+  const int wlo = (int)__reduce_min_sync(0xffffffffu, (unsigned)(any ? lo : kLevels));
+  const int whi = (int)__reduce_max_sync(0xffffffffu, (unsigned)(any ? hi + 1 : 0)) - 1;
+  for (int l = wlo; l <= whi; ++l) {
+    const uint32_t m = __ballot_sync(0xffffffffu, l >= lo && l <= hi);
+    if (lane == 0) s_warp[w][l] = __popc(m);
+  }
+  __syncthreads();
+  if (threadIdx.x < kLevels) {
+    int run = s_first[threadIdx.x];
+#pragma unroll
+    for (int ww = 0; ww < kTopoThreads / 32; ++ww) {
+      const int c = s_warp[ww][threadIdx.x];
+      s_warp[ww][threadIdx.x] = run;
+      run += c;
     }
-    int start = 0, end = 0;
-    if (split) {
-      // first index in [f, f + c) whose digit at level lev+1 is >= sub
-      int lo = D.x, hi = D.x + D.y;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        const uint32_t dg = (uint32_t)((keys[mid] >> shift) & 7u);
-        if (dg < (uint32_t)sub) lo = mid + 1; else hi = mid;
-      }
-      start = lo;
-    }
-    const int nxt = __shfl_down_sync(0xffffffffu, start, 1, 8);
-    end = (sub == 7) ? D.x + D.y : nxt;
-    const bool has = split && end > start;
-    const uint32_t seg = (__ballot_sync(0xffffffffu, has) >> (lane & 24)) & 0xffu;
-    const int nchild = __popc(seg);
-    const int rank = __popc(seg & ((1u << sub) - 1u));
-    // block-wide allocation of child slots
-    if (sub == 0) s_cnt[slot] = split ? nchild : 0;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int run = 0;
-      for (int s2 = 0; s2 < 32; ++s2) {
-        const int c = s_cnt[s2];
-        s_cnt[s2] = run;
-        run += c;
-      }
-      s_base = run ? atomicAdd(&T.sb->level_cnt[lev + 1], run) : 0;
-    }
-    __syncthreads();
-    const int child_first = next_base + s_base + s_cnt[slot];
-    if (split) {
-      const bool fits = child_first + nchild <= T.cap;
-      if (!fits) {
-        if (sub == 0) set_status(T.sb, ST_NOSPACE);
-      } else {
-        if (has) {
-          const int c = child_first + rank;
-          const int ccount = end - start;
-          const int leaf = (ccount <= leaf_size || lev + 1 >= kMaxLevel) ? 1 : 0;
-          T.nD[c] = make_int4(start, ccount, -1, make_meta(0, lev + 1, leaf));
-          T.nParent[c] = p;
-        }
-        if (sub == 0) {
-          D.z = child_first;
-          D.w = make_meta(nchild, lev, 0);
-          T.nD[p] = D;
+  }
+  __syncthreads();
+  // deepest level first: a node's run lies inside its parent's, so the end
+  // found for one level is where the search for the next one up begins
+  int64_t end = i + 1;
+  int below = -1;  // index of this key's node one level down
+  for (int l = whi; l >= wlo; --l) {
+    const bool here = l >= lo && l <= hi;
+    const uint32_t m = __ballot_sync(0xffffffffu, here);
+    if (!here) continue;
+    const int64_t p = (int64_t)s_warp[w][l] + __popc(m & ((1u << lane) - 1u));
+    if (l == 0) {
+      end = T.n;
+    } else {
+      // first key at or after `end` whose top l digits differ
+      const int shift = 63 - 3 * l;
+      const uint64_t pre = keys[i] >> shift;
+      int64_t step = 1;
+      while (end < T.n && (keys[end] >> shift) == pre) {
+        const int64_t probe = end + step;
+        if (probe < T.n && (keys[probe] >> shift) == pre) {
+          end = probe + 1;
+          step <<= 1;
+        } else if (step > 1) {
+          // the run ends in (end, probe]
+          int64_t a = end + 1, b = probe < T.n ? probe : T.n;
+          while (a < b) {
+            const int64_t mid = (a + b) >> 1;
+            if ((keys[mid] >> shift) == pre) a = mid + 1;
+            else b = mid;
+          }
+          end = a;
+          break;
+        } else {
+          ++end;
         }
       }
     }
-    __syncthreads();
+    if (p < T.cap) {
+      const bool leaf = l > deep;
+      T.nD[p] = make_int4((int)i, (int)(end - i), leaf ? -1 : below, make_meta(0, l, leaf));
+      if (l == 0) T.nParent[p] = -1;
+    } else {
+      set_status(T.sb, ST_NOSPACE);
+    }
+    below = (int)p;
   }
 }
 
-// Bottom-up moments for one level, one thread per node.  A leaf sums its
-// particles and an internal node its children, in index order; then the
-// node's centre of mass, split FP32 copies and cube centre are written.  On
-// this GPU an FP64 warp instruction costs the same however many lanes are
-// active, so giving each lane its own node (rather than spreading one node
-// over several lanes) minimises FP64 instructions per node.
-__global__ void __launch_bounds__(256) k_moments(TreeDev T, int lev, BoxScale B) {
-  const int base = level_base(T.sb, lev);
-  const int cnt = T.sb->level_cnt[lev];
-  if (base + cnt > T.cap) return;  // capacity already exceeded (flagged by k_expand)
+// A node's sums and everything derived from them: centre of mass, split FP32
+// copies and cube centre.  On this GPU an FP64 warp instruction costs the same
+// however many lanes are active, so each lane serves its own node (rather than
+// one node spread over several lanes).
+__device__ __forceinline__ void write_moments(const TreeDev& T, const BoxScale& B, int p, const int4& D, double M,
+                                              double S0, double S1, double S2, double H) {
+  const int lev = meta_level(D.w);
   const double side = ldexp(B.L, -lev);
   const float side_b = ldexpf(1.0f, -lev);
   const double invL = B.invL, invL2 = B.invL * B.invL;
-  for (int step = blockIdx.x * blockDim.x + threadIdx.x; step < cnt; step += gridDim.x * blockDim.x) {
-    const int p = base + step;
+  const double invM = 1.0 / M;
+  const double com[3] = {S0 * invM, S1 * invM, S2 * invM};
+  float hi[3], lo[3];
+  double cen[3];
+  float cenb[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    if (!(B.pow2 && split_bits((uint64_t)__double_as_longlong(com[c]), B.e, hi[c], lo[c])))
+      split_coord(com[c] * invL, hi[c], lo[c]);
+    const uint32_t q = quantise(T.x64[3 * (int64_t)D.x + c], B) >> (kMaxLevel - lev);
+    // (q + 1/2) side, exact for a power-of-two box: (2q + 1) 2^(e - lev - 1)
+    if (!(B.pow2 && double_odd_scaled(2u * q + 1u, B.e - lev - 1, cen[c]))) cen[c] = __dmul_rn((double)q + 0.5, side);
+    cenb[c] = ((float)q + 0.5f) * side_b;
+  }
+  // M / L^2 and (hmax / L)^2 in FP32, as in k_permute
+  const bool sq = B.pow2 && B.e >= -511 && B.e <= 537;
+  float mw, h2;
+  if (!(sq && d2f_scaled((uint64_t)__double_as_longlong(M), 2 * B.e, mw))) mw = (float)(M * invL2);
+  const double HH = H * H;
+  if (!(sq && d2f_scaled((uint64_t)__double_as_longlong(HH), 2 * B.e, h2))) {
+    const double hb = H * invL;
+    h2 = (float)(hb * hb);
+  }
+  T.mass64[p] = M;
+  T.hmax64[p] = H;
+  T.S64[3 * (int64_t)p] = S0;
+  T.S64[3 * (int64_t)p + 1] = S1;
+  T.S64[3 * (int64_t)p + 2] = S2;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    T.com64[3 * (int64_t)p + c] = com[c];
+    T.cen64[3 * (int64_t)p + c] = cen[c];
+  }
+  T.nA[p] = make_float4(hi[0], hi[1], hi[2], mw);
+  T.nB[p] = make_float4(lo[0], lo[1], lo[2], h2);
+  T.nC[p] = make_float4(cenb[0], cenb[1], cenb[2], side_b);
+}
+
+// The leaves of all levels.  hmax as an integer max of the bit patterns:
+// softenings are positive (checked by k_permute), and positive doubles order
+// like their bits.
+__global__ void __launch_bounds__(256) k_leaves(TreeDev T, BoxScale B) {
+  const int total = level_base(T.sb, kLevels);
+  if (total > T.cap) return;  // flagged by k_fill
+  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < total; p += gridDim.x * blockDim.x) {
     const int4 D = T.nD[p];
+    if (!meta_leaf(D.w)) continue;
     double M = 0.0, S0 = 0.0, S1 = 0.0, S2 = 0.0;
-    // hmax as an integer max of the bit patterns: softenings are positive
-    // (checked by k_permute), and positive doubles order like their bits
     long long Hb = 0;
-    if (meta_leaf(D.w)) {
-      for (int j = D.x; j < D.x + D.y; ++j) {
-        const double m = T.m64[j];
-        M += m;
-        S0 += m * T.x64[3 * (int64_t)j];
-        S1 += m * T.x64[3 * (int64_t)j + 1];
-        S2 += m * T.x64[3 * (int64_t)j + 2];
-        Hb = max(Hb, __double_as_longlong(T.h64[j]));
-        T.leaf_of[j] = p;
+    for (int j = D.x; j < D.x + D.y; ++j) {
+      const double m = T.m64[j];
+      M += m;
+      S0 += m * T.x64[3 * (int64_t)j];
+      S1 += m * T.x64[3 * (int64_t)j + 1];
+      S2 += m * T.x64[3 * (int64_t)j + 2];
+      Hb = max(Hb, __double_as_longlong(T.h64[j]));
+      T.leaf_of[j] = p;
+    }
+    write_moments(T, B, p, D, M, S0, S1, S2, __longlong_as_double(Hb));
+  }
+}
+
+// Polls of the grid barrier before it gives up (seconds, far above a level).
+constexpr int kBarrierPolls = 1 << 24;
+
+// Barrier over the grid of a cooperative launch; false if it gave up.  Every
+// block passes the same number of blocks * phase.
+__device__ bool grid_barrier(unsigned long long* count, unsigned long long target) {
+  __shared__ int s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(count, 1ull);
+    int ok = 0;
+    for (int i = 0; i < kBarrierPolls && !ok; ++i) ok = *(volatile unsigned long long*)count >= target;
+    __threadfence();
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+// The split nodes, from the deepest level up.
+constexpr int kUpThreads = 512;
+__global__ void __launch_bounds__(kUpThreads) k_upward(TreeDev T, BoxScale B) {
+  int cnt[kLevels];
+  int total = 0;
+#pragma unroll
+  for (int l = 0; l < kLevels; ++l) {
+    cnt[l] = T.sb->level_cnt[l];
+    total += cnt[l];
+  }
+  if (total > T.cap) return;  // flagged by k_fill
+  // levels 0 .. lone have at most kUpThreads nodes each: block 0 does them
+  int lone = -1;
+#pragma unroll
+  for (int l = 0; l < kLevels; ++l)
+    if (lone == l - 1 && cnt[l] <= kUpThreads) lone = l;
+  int base = total;
+  unsigned long long phase = 0;
+#pragma unroll 1
+  for (int l = kLevels - 1; l >= 0; --l) {
+    const int c_l = T.sb->level_cnt[l];
+    base -= c_l;
+    if (c_l == 0) continue;
+    const bool single = l <= lone;
+    if (single && blockIdx.x != 0) return;
+    const int stride = single ? kUpThreads : gridDim.x * kUpThreads;
+    for (int s = (single ? 0 : blockIdx.x * kUpThreads) + threadIdx.x; s < c_l; s += stride) {
+      const int p = base + s;
+      int4 D = T.nD[p];
+      if (meta_leaf(D.w)) continue;
+      double M = 0.0, S0 = 0.0, S1 = 0.0, S2 = 0.0;
+      long long Hb = 0;
+      int c = D.z, left = D.y;
+      while (left > 0 && c < total) {
+        M += __ldcg(&T.mass64[c]);
+        S0 += __ldcg(&T.S64[3 * (int64_t)c]);
+        S1 += __ldcg(&T.S64[3 * (int64_t)c + 1]);
+        S2 += __ldcg(&T.S64[3 * (int64_t)c + 2]);
+        Hb = max(Hb, __double_as_longlong(__ldcg(&T.hmax64[c])));
+        T.nParent[c] = p;
+        left -= T.nD[c].y;
+        ++c;
       }
+      D.w = make_meta(c - D.z, l, 0);
+      T.nD[p] = D;
+      write_moments(T, B, p, D, M, S0, S1, S2, __longlong_as_double(Hb));
+    }
+    if (l == 0) break;
+    if (single) {
+      __threadfence_block();
+      __syncthreads();
     } else {
-      const int c1 = D.z + meta_nchild(D.w);
-      for (int c = D.z; c < c1; ++c) {
-        M += T.mass64[c];
-        S0 += T.S64[3 * (int64_t)c];
-        S1 += T.S64[3 * (int64_t)c + 1];
-        S2 += T.S64[3 * (int64_t)c + 2];
-        Hb = max(Hb, __double_as_longlong(T.hmax64[c]));
+      ++phase;
+      if (!grid_barrier(&T.sb->work, phase * gridDim.x)) {
+        if (threadIdx.x == 0) set_status(T.sb, ST_WALKCAP);
+        return;
       }
     }
-    const double H = __longlong_as_double(Hb);
-    const double invM = 1.0 / M;
-    const double com[3] = {S0 * invM, S1 * invM, S2 * invM};
-    float hi[3], lo[3];
-    double cen[3];
-    float cenb[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (!(B.pow2 && split_bits((uint64_t)__double_as_longlong(com[c]), B.e, hi[c], lo[c])))
-        split_coord(com[c] * invL, hi[c], lo[c]);
-      const uint32_t q = quantise(T.x64[3 * (int64_t)D.x + c], B) >> (kMaxLevel - lev);
-      // (q + 1/2) side, exact for a power-of-two box: (2q + 1) 2^(e - lev - 1)
-      if (!(B.pow2 && double_odd_scaled(2u * q + 1u, B.e - lev - 1, cen[c]))) cen[c] = __dmul_rn((double)q + 0.5, side);
-      cenb[c] = ((float)q + 0.5f) * side_b;
-    }
-    // M / L^2 and (hmax / L)^2 in FP32, as in k_permute
-    const bool sq = B.pow2 && B.e >= -511 && B.e <= 537;
-    float mw, h2;
-    if (!(sq && d2f_scaled((uint64_t)__double_as_longlong(M), 2 * B.e, mw))) mw = (float)(M * invL2);
-    const double HH = H * H;
-    if (!(sq && d2f_scaled((uint64_t)__double_as_longlong(HH), 2 * B.e, h2))) {
-      const double hb = H * invL;
-      h2 = (float)(hb * hb);
-    }
-    T.mass64[p] = M;
-    T.hmax64[p] = H;
-    T.S64[3 * (int64_t)p] = S0;
-    T.S64[3 * (int64_t)p + 1] = S1;
-    T.S64[3 * (int64_t)p + 2] = S2;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      T.com64[3 * (int64_t)p + c] = com[c];
-      T.cen64[3 * (int64_t)p + c] = cen[c];
-    }
-    T.nA[p] = make_float4(hi[0], hi[1], hi[2], mw);
-    T.nB[p] = make_float4(lo[0], lo[1], lo[2], h2);
-    T.nC[p] = make_float4(cenb[0], cenb[1], cenb[2], side_b);
   }
 }
 
@@ -262,16 +391,23 @@ cudaError_t launch_tree_build(const BuildArgs& A, cudaStream_t s) {
   if (grid > grid_cap(32)) grid = grid_cap(32);
   const BoxScale B = box_scale(A.L);
   k_permute<<<(unsigned)grid, 256, 0, s>>>(A, B);
-  int64_t ggrid = (T.ngroups + 127) / 128;
-  if (ggrid > grid_cap(16)) ggrid = grid_cap(16);
-  k_groups<<<(unsigned)ggrid, 128, 0, s>>>(T, B);
-  k_root<<<1, 32, 0, s>>>(T, A.leaf_size);
-  // Grids are fixed (the per-level node count lives on the device); blocks
-  // stride over the level.
-  const unsigned egrid = grid_cap(8);
-  for (int lev = 0; lev < kMaxLevel; ++lev) k_expand<<<egrid, 256, 0, s>>>(T, A.keys, lev, A.leaf_size);
-  for (int lev = kMaxLevel; lev >= 0; --lev) k_moments<<<egrid, 256, 0, s>>>(T, lev, B);
-  return cudaGetLastError();
+  k_count<<<(unsigned)T.nblk, kTopoThreads, 0, s>>>(T, A.keys, A.leaf_size);
+  k_scan<<<kLevels, 1024, 0, s>>>(T);
+  k_fill<<<(unsigned)T.nblk, kTopoThreads, 0, s>>>(T, A.keys, A.leaf_size);
+  // the node counts live on the device: grids are sized for the particles
+  int64_t lgrid = (T.n / 2 + 255) / 256;
+  if (lgrid > grid_cap(8)) lgrid = grid_cap(8);
+  if (lgrid < 1) lgrid = 1;
+  k_leaves<<<(unsigned)lgrid, 256, 0, s>>>(T, B);
+  TreeDev Tv = T;
+  BoxScale Bv = B;
+  void* args[] = {&Tv, &Bv};
+  int64_t ugrid = (T.n / 8 + kUpThreads - 1) / kUpThreads;
+  if (ugrid > grid_cap(1)) ugrid = grid_cap(1);
+  if (ugrid < 1) ugrid = 1;
+  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_upward, dim3((unsigned)ugrid), dim3(kUpThreads), args,
+                                                    0, s);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 __global__ void k_copy_nodes(TreeDev T, int64_t m, int32_t* level, int32_t* first, int32_t* count, int32_t* parent,
