@@ -153,10 +153,14 @@ static og_status walk_common(const og_tree* t, double r_s, double theta, WalkArg
   const double rsb = r_s / L;
   A.fp_c = (float)(-1.0 / (2.0 * std::sqrt(M_PI) * rsb * rsb * rsb));
   A.rc2_64 = rcut * rcut;
+  const double rc2_lo = A.rc2_64 * (1.0 - 1e-12), rc2_hi = A.rc2_64 * (1.0 + 1e-12);
+  std::memcpy(&A.rc2_lo_bits, &rc2_lo, sizeof(rc2_lo));
+  std::memcpy(&A.rc2_hi_bits, &rc2_hi, sizeof(rc2_hi));
   A.th2_64 = theta * theta;
   A.box = L;
   A.r_s64 = r_s;
   A.inv2rs64 = 1.0 / (2.0 * r_s);
+  A.inv2rs = (float)A.inv2rs64;
   A.fp_c64 = -1.0 / (2.0 * std::sqrt(M_PI) * r_s * r_s * r_s);
   return OG_OK;
 }

@@ -314,8 +314,10 @@ struct WalkArgs {
   float t_scale;               // t = r * t_scale - 1  (= u / 1.125 - 1)
   float ex2c;                  // exp(-u^2) = ex2(r2 * ex2c)
   float fp_c;                  // f'(r)/r = fp_c * r * exp(-u^2)
+  float inv2rs;                // 1 / (2 r_s), physical units
   // FP64, physical units (exact re-checks, FP64 walk)
   double rc2_64, th2_64, box, r_s64, inv2rs64, fp_c64;
+  long long rc2_lo_bits, rc2_hi_bits;  // bits of rc2_64 (1 -+ 1e-12)
   // outputs
   float* accf;
   double* accd;

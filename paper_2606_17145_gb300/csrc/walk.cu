@@ -46,6 +46,7 @@
 
 #include "og_internal.cuh"
 #include "short_range_poly.inc"
+#include "short_range_table.inc"
 
 namespace og {
 
@@ -395,11 +396,23 @@ __device__ __forceinline__ int decide_f32(const WalkArgs& A, int64_t k, const fl
   return decide_exact(A, k, node, level);
 }
 
-// One pair's result in the FP64 variant and whether it lies inside the cut.
-struct Term64 {
-  double x, y, z;
-  bool in;
-};
+// The short-range factor f(u) = erfc(u) + (2 u / sqrt(pi)) exp(-u^2) in FP64:
+// a degree-6 polynomial about the centre of each interval of width 1 / 64
+// (its error, below 1e-17, is far under the rounding), four 16-byte loads and
+// seven FP64 operations.  uf: u to FP32 accuracy (beside a boundary either
+// interval's polynomial serves).  u stays below 2.25 at the default cut of
+// 4.5 r_s; beyond the table CUDA's functions take over.
+__device__ __forceinline__ double short_range_f64(double u, float uf) {
+  const float fi = uf * (float)OG_SR_TABLE_PER_UNIT;
+  if (fi < (float)OG_SR_TABLE_N) {
+    const int i = (int)fi;
+    const double2* e = reinterpret_cast<const double2*>(og_sr_table) + 4 * i;
+    const double2 a = __ldg(e), b = __ldg(e + 1), c = __ldg(e + 2), d = __ldg(e + 3);
+    const double x = u - a.x;
+    return fma(fma(fma(fma(fma(fma(d.y, x, d.x), x, c.y), x, c.x), x, b.y), x, b.x), x, a.y);
+  }
+  return erfc(u) + 1.1283791670955126 * u * exp(-u * u);
+}
 
 // Lane of the walk: FP32 + Kahan forward (ADJ = false) or adjoint
 // (ADJ = true), or the all-FP64 forward variant (F64 = true: FP64 pair
@@ -419,8 +432,11 @@ struct LaneFP {
     float4 tW[ADJ ? kGroup : 1];   // adjoint: dL/da of each target
     float4 SG[ADJ ? kStage : 1];   // adjoint: source-side sums (G, S) of each staged slot over the batch
     int self[kGroup];     // staged slot holding the target itself, or -1
-    double3 Ps[F64 ? kGroup : 1];  // FP64 variant: each target's sum over the batch
-    int fneg[F64 ? kGroup : 1];  // FP64 variant: listed pairs of the batch outside the exact cut
+    // FP64 variant: targets; each target's sum over the batch; the sum of each
+    // lane's first run where that run began in an earlier lane
+    double tx[F64 ? 3 : 1][F64 ? kGroup : 1], th2[F64 ? kGroup : 1];
+    double Ps[F64 ? 3 : 1][F64 ? kGroup : 1], Hd[F64 ? 3 : 1][F64 ? kGroup : 1];
+    int fneg[F64 ? kGroup : 1];  // listed pairs of the batch outside the exact cut
   };
   // per-batch staging (dead between evaluations; shares memory with the
   // traversal's scratch)
@@ -436,6 +452,7 @@ struct LaneFP {
     float4 ra[F64 ? 1 : kSlots], rb[F64 ? 1 : kSlots];  // the next 32 sources as they arrive from the tree
     int id[kStage];       // particle, or -2 - node
     uint32_t sq[kStage];  // lane mask of the source's queue entry
+    double sx[F64 ? 3 : 1][F64 ? kStage : 1], sm[F64 ? kStage : 1], sh2[F64 ? kStage : 1];  // FP64: position, -mass, h^2
     float fX[F64 ? kStage : 1], fY[F64 ? kStage : 1], fZ[F64 ? kStage : 1], fW[F64 ? kStage : 1];  // filter form (see put)
   };
   // a slot's source as read from the tree
@@ -443,6 +460,7 @@ struct LaneFP {
     float4 a, b;
     int id;  // particle, or -2 - node
     uint32_t q;
+    bool shifted;  // FP64 variant: not at its stored image
   };
 
   int64_t k;          // sorted index of this lane's target
@@ -462,7 +480,12 @@ struct LaneFP {
     const float4 b = A.T.pB[kc];
     M.tA[lane] = make_float4(a.x, a.y, a.z, b.w);
     M.tB[lane] = make_float4(b.x, b.y, b.z, 0.f);
-    if constexpr (F64) M.Ps[lane] = make_double3(0.0, 0.0, 0.0);
+    if constexpr (F64) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) M.tx[c][lane] = A.T.x64[3 * kc + c];
+      const double h = A.T.h64[kc];
+      M.th2[lane] = h * h;
+    }
     a64[0] = a64[1] = a64[2] = 0.0;
     if constexpr (F64) M.fneg[lane] = 0;
     if constexpr (ADJ) M.SG[lane] = M.SG[lane + 32] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -483,52 +506,58 @@ struct LaneFP {
     nint = 0;
   }
 
-  // FP64 variant: target gbase + i against staged slot s, read from the
-  // FP64 tree arrays; the cut is taken on the FP64 distance (accepted nodes
-  // are inside by decision).
-  __device__ __forceinline__ Term64 pair_eval64(const WalkArgs& A, const Stage& St, int i, int s,
-                                                    int64_t gbase) const {
-    const int id = St.id[s];
-    const int64_t kt = gbase + i;
-    const double* x = A.T.x64;
-    double sp[3], m, h;
-    if (id >= 0) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) sp[c] = x[3 * (int64_t)id + c];
-      m = A.T.m64[id];
-      h = A.T.h64[id];
-    } else {
-      const int64_t n = -2 - id;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) sp[c] = A.T.com64[3 * n + c];
-      m = A.T.mass64[n];
-      h = A.T.hmax64[n];
+  // FP64 variant: force of staged slot s on target i, added to acc; false
+  // (and nothing added) outside the cut.  1 / r by a third-order step from the
+  // FP32 reciprocal root.  The cut is taken on r^2 in the reference's order of
+  // operations where the contracted r^2 is within rounding of it (accepted
+  // nodes are inside by decision).  Bound by the FP64 pipe, 1/64 of the FP32
+  // rate: 28 operations a pair (displacement 3, r^2 3, 1 / r and r 6, factor 8,
+  // force 8) where CUDA's erfc, exp, sqrt and divisions and a segmented scan of
+  // the sums took about 220.  64^3 clustered 30.6 -> 7.0 ms, 128^3 lattice 52.9 ->
+  // 12.4, zoom set 347 -> 72; error against 64 bits unchanged (1.4e-14).
+  __device__ __forceinline__ bool pair_eval64(const WalkArgs& A, const Stage& St, const Smem& M, int i, int s,
+                                              bool wrap, double (&acc)[3]) const {
+    double d0 = M.tx[0][i] - St.sx[0][s], d1 = M.tx[1][i] - St.sx[1][s], d2 = M.tx[2][i] - St.sx[2][s];
+    if (wrap) {
+      d0 = mi64(d0, A.box);
+      d1 = mi64(d1, A.box);
+      d2 = mi64(d2, A.box);
     }
-    double dv[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) dv[c] = mi64(__dsub_rn(x[3 * kt + c], sp[c]), A.box);
-    const double r2 = norm2_64(dv[0], dv[1], dv[2]);
-    Term64 t = {0.0, 0.0, 0.0, false};
-    if (id >= 0 && !(r2 < A.rc2_64)) return t;
-    const double r = sqrt(r2);
-    const double hh = fmax(A.T.h64[kt], h);
-    double K;
-    if (r >= hh) {
-      K = 1.0 / (r * r * r);
+    const double r2 = fma(d0, d0, fma(d1, d1, d2 * d2));
+    // positive doubles order like their bits
+    const long long rb = __double_as_longlong(r2);
+    if (rb >= A.rc2_lo_bits && St.id[s] >= 0 && !(rb <= A.rc2_hi_bits && norm2_64(d0, d1, d2) < A.rc2_64)) return false;
+    const long long hb = max(__double_as_longlong(M.th2[i]), __double_as_longlong(St.sh2[s]));
+    double r, K;
+    float uf;
+    if (rb < hb || (uint32_t)(rb >> 52) - 923u > 200u) {  // softened, or r^2 outside 2^-100 .. 2^101
+      const double hh = sqrt(__longlong_as_double(hb));
+      r = sqrt(r2);
+      uf = (float)(r * A.inv2rs64);
+      if (r >= hh) {
+        K = 1.0 / (r * r * r);
+      } else {
+        const double v = r / hh;
+        const double h3 = 1.0 / (hh * hh * hh);
+        if (v < 0.5) K = h3 * (32.0 / 3.0 + v * v * (32.0 * v - 38.4));
+        else K = h3 * (64.0 / 3.0 - 48.0 * v + 38.4 * v * v - (32.0 / 3.0) * v * v * v - (1.0 / 15.0) / (v * v * v));
+      }
     } else {
-      const double v = r / hh;
-      const double h3 = 1.0 / (hh * hh * hh);
-      if (v < 0.5) K = h3 * (32.0 / 3.0 + v * v * (32.0 * v - 38.4));
-      else K = h3 * (64.0 / 3.0 - 48.0 * v + 38.4 * v * v - (32.0 / 3.0) * v * v * v - (1.0 / 15.0) / (v * v * v));
+      // conversions on the integer pipe
+      const float r2f = __uint_as_float((uint32_t)((rb >> 29) - (896ll << 23)));
+      const float yf = rsqrt_approx(r2f);
+      const double y = __longlong_as_double(((long long)__float_as_uint(yf) << 29) + (896ll << 52));
+      const double e = fma(-(r2 * y), y, 1.0);
+      const double y1 = fma(y * e, fma(e, 0.375, 0.5), y);
+      r = r2 * y1;
+      K = y1 * y1 * y1;
+      uf = r2f * yf * A.inv2rs;
     }
-    const double u = r * A.inv2rs64;
-    const double f = erfc(u) + 1.1283791670955126 * u * exp(-u * u);
-    const double sc = -m * K * f;
-    t.x = sc * dv[0];
-    t.y = sc * dv[1];
-    t.z = sc * dv[2];
-    t.in = true;
-    return t;
+    const double sc = St.sm[s] * (K * short_range_f64(r * A.inv2rs64, uf));
+    acc[0] = fma(sc, d0, acc[0]);
+    acc[1] = fma(sc, d1, acc[1]);
+    acc[2] = fma(sc, d2, acc[2]);
+    return true;
   }
 
   // Start fetching slot s of queue entry e: its two 16-byte records go to
@@ -576,6 +605,7 @@ struct LaneFP {
     x[2] = (x[2] - n2) + f.b.z;
     const float a0 = fabsf(x[0]), a1 = fabsf(x[1]), a2 = fabsf(x[2]);
     uni = fmaxf(a0 + G.ex, fmaxf(a1 + G.ey, a2 + G.ez)) < A.uni_lim;
+    if (F64) f.shifted = n0 != 0.f || n1 != 0.f || n2 != 0.f;
     const float g0 = fmaxf(a0 - G.ex, 0.f), g1 = fmaxf(a1 - G.ey, 0.f), g2 = fmaxf(a2 - G.ez, 0.f);
     return fmaf(g0, g0, fmaf(g1, g1, g2 * g2)) <= A.grp_rc2;
   }
@@ -613,6 +643,13 @@ struct LaneFP {
         fz = -2.f * x[2];
         fw = (sj - A.rc2_hi) - 3.814697265625e-06f * fmaf(rr, rr, A.rc2_hi);
       }
+      const int64_t j = f.id >= 0 ? f.id : -2 - f.id;
+      const double* sp = f.id >= 0 ? A.T.x64 : A.T.com64;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) S.sx[c][pos] = sp[3 * j + c];
+      S.sm[pos] = -(f.id >= 0 ? A.T.m64 : A.T.mass64)[j];
+      const double h = (f.id >= 0 ? A.T.h64 : A.T.hmax64)[j];
+      S.sh2[pos] = h * h;
       S.fX[pos] = fx;
       S.fY[pos] = fy;
       S.fZ[pos] = fz;
@@ -655,7 +692,9 @@ struct LaneFP {
     // in entry ecur + (number of starts at or before bit l).
     // The next window is fetched while the current one is staged and evaluated.
     int pend = 0;
-    bool mi = false;  // some staged source has no image common to the whole group
+    // some staged source has no image common to the whole group (FP64 variant:
+    // or one that is not its stored position)
+    bool mi = false;
     int ecur = 0;
     Fetch cur = {};
     auto window = [&](int rb, Fetch& f) {
@@ -675,14 +714,14 @@ struct LaneFP {
       const bool kp = rb + lane < total && arrive(A, St, lane, G, cur, x, uni);
       const uint32_t km = __ballot_sync(0xffffffffu, kp);
       if (kp) put(A, St, M, cur, pend + __popc(km & lt), x, uni, gbase, Rg);
-      mi = mi || __any_sync(0xffffffffu, kp && !uni);
+      mi = mi || __any_sync(0xffffffffu, kp && (!uni || (F64 && cur.shifted)));
       pend += __popc(km);
       if (rb + 32 < total) window(rb + 32, cur);
       __syncwarp();
       if (pend > 0 && (pend > kStage - 32 || rb + 32 >= total)) {
         if constexpr (F64) {
 #pragma unroll 1
-          for (int hb = 0; hb < pend; hb += 32) batch_list(A, W, St, M, hb, min(pend - hb, 32), lane, gbase, vmask);
+          for (int hb = 0; hb < pend; hb += 32) batch_list(A, W, St, M, hb, min(pend - hb, 32), lane, vmask, mi);
         } else {
           batch_tiles(A, W, St, M, SGB, pend, lane, gbase, vmask, mi);
         }
@@ -1025,9 +1064,14 @@ struct LaneFP {
 
   // One FP64 batch: the cnt staged sources at slots [hb, hb + cnt).  The FP64
   // pipe runs a warp instruction at the same cost however few lanes are
-  // active, so the hit pairs are listed and each iteration evaluates 32.
+  // active (16 cycles of the SM), so the hit pairs are listed target by target
+  // and each lane evaluates an equal share of consecutive pairs.  A run of
+  // one target's pairs sums in the lane's registers; the lane in which the run
+  // begins stores its part, the lanes that continue it keep theirs aside, and
+  // the target's owner adds them in lane order: three FP64 additions a
+  // target where a segmented scan took fifteen an iteration.
   __device__ void batch_list(const WalkArgs& A, const WarpBufs& W, Stage& St, Smem& M, int hb, int cnt, int lane,
-                             int64_t gbase, uint32_t vmask) {
+                             uint32_t vmask, bool wrap) {
     // bit s of msk: slot s is in this lane's part of its entry's lane mask
     const bool has = lane < cnt;
     const uint32_t q = has ? St.sq[hb + lane] : 0u;
@@ -1079,55 +1123,54 @@ struct LaneFP {
       }
       nint += c;  // listed pairs; those outside the exact cut are subtracted below
       __syncwarp();
+      if (T == 0) continue;
+      const int share = (T + 31) >> 5;  // consecutive pairs of each lane
+      const int p0 = lane * share, p1 = min(p0 + share, T);
+      int cur = p0 < T ? W.list[p0] >> 5 : -1;               // target of the run being summed
+      bool head = p0 > 0 && p0 < T && (W.list[p0 - 1] >> 5) == cur;  // it began in an earlier lane
+      double sum[3] = {0.0, 0.0, 0.0};
 #pragma unroll 1
-      for (int p0 = 0; p0 < T; p0 += 32) {
-        const int p = p0 + lane;
-        const bool hv = p < T;
-        int i = 0;
-        Term64 r = {0.0, 0.0, 0.0, false};
-        if (hv) {
+      for (int u = 0; u < share; ++u) {
+        const int p = p0 + u;
+        if (p < p1) {
           const int e = W.list[p];
-          i = e >> 5;
-          r = pair_eval64(A, St, i, hb + (e & 31), gbase);
-          if (!r.in) atomicAdd(&M.fneg[i], 1);
-        }
-        // segmented inclusive scan over the lanes: the pairs of one target
-        // are consecutive, so each target's run is summed in a fixed tree
-        // order and its last lane adds the sum to the target's batch total
-        const int oi = __shfl_sync(0xffffffffu, off, i);
-        const int ci = __shfl_sync(0xffffffffu, c, i);
-        const int first = max(oi - p0, 0);
-        // the longest run reaching back into this iteration: steps beyond
-        // it add nothing (warp-uniform, so skipping them changes no sum)
-        const int span = (int)__reduce_max_sync(0xffffffffu, (unsigned)(hv ? lane - first : 0));
+          const int i = e >> 5;
+          if (i != cur) {
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          if (d > 4 && span < d) break;
-          const double y0 = __shfl_up_sync(0xffffffffu, r.x, d);
-          const double y1 = __shfl_up_sync(0xffffffffu, r.y, d);
-          const double y2 = __shfl_up_sync(0xffffffffu, r.z, d);
-          if (lane - d >= first) {
-            r.x += y0;
-            r.y += y1;
-            r.z += y2;
+            for (int a = 0; a < 3; ++a) {
+              if (head) M.Hd[a][lane] = sum[a];
+              else M.Ps[a][cur] = sum[a];
+              sum[a] = 0.0;
+            }
+            head = false;
+            cur = i;
           }
+          if (!pair_eval64(A, St, M, i, hb + (e & 31), wrap, sum)) atomicAdd(&M.fneg[i], 1);
         }
-        if (hv && p == min(min(oi + ci, T), p0 + 32) - 1) {
-          double3 a = M.Ps[i];
-          a.x += r.x;
-          a.y += r.y;
-          a.z += r.z;
-          M.Ps[i] = a;
-        }
-        __syncwarp();
       }
+      if (p0 < T) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          if (head) M.Hd[a][lane] = sum[a];
+          else M.Ps[a][cur] = sum[a];
+        }
+      }
+      __syncwarp();
+      if (c > 0) {
+        // the run began in lane off / share and goes on in those after it
+        const int l1 = (off + c - 1) / share;
+        double s0 = M.Ps[0][lane], s1 = M.Ps[1][lane], s2 = M.Ps[2][lane];
+        for (int l = off / share + 1; l <= l1; ++l) {
+          s0 += M.Hd[0][l];
+          s1 += M.Hd[1][l];
+          s2 += M.Hd[2][l];
+        }
+        a64[0] += s0;
+        a64[1] += s1;
+        a64[2] += s2;
+      }
+      __syncwarp();
     }
-    // this batch's sums into the plain double sums
-    const double3 ps = M.Ps[lane];
-    a64[0] += ps.x;
-    a64[1] += ps.y;
-    a64[2] += ps.z;
-    M.Ps[lane] = make_double3(0.0, 0.0, 0.0);
     nint -= M.fneg[lane];
     M.fneg[lane] = 0;
     // this batch held the target's own slot
@@ -1467,12 +1510,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
 // uniform) 0.37 / 0.28 / 0.22, 1024 groups (32^3) clustered 0.31 / 0.27 / 0.25,
 // zoom 3.66 / 2.61 / 2.45, lattice 0.15 / 0.14 / 0.15; 5860 groups (zoom) 17.9 /
 // 18.4 / 20.0; 8192 groups (64^3) lattice 0.43 / 0.49 / 0.63, clustered 1.76 /
-// 1.58 / 1.67.  The FP64 walk repeats a smaller share: 1024 groups clustered
-// 5.0 / 3.2 / 2.5, 5860 (zoom) 349 / 310 / 312, 8192 clustered 30.6 / 26.0 / 23.7,
-// lattice 7.3 / 7.5 / 7.8, 22,800 (90^3 clustered) 112 / 98 / 99.
+// 1.58 / 1.67.  FP64: 128 groups 1.59 / 0.94 / 0.68, 1024 clustered 1.60 / 1.06 /
+// 0.91, zoom 8.2 / 8.0 / 9.1, lattice 0.40 / 0.37 / 0.44; 5860 (zoom) 71.6 / 72.9 / 83.0,
+// 8192 clustered 7.7 / 6.8 / 6.7, lattice 1.90 / 1.94 / 2.31.
 static int walk_split(int64_t n_groups, bool f64) {
   if (n_groups <= 1024) return 2;
-  return n_groups <= (f64 ? 32768 : 4096) ? 1 : 0;
+  return n_groups <= (f64 ? 8192 : 4096) ? 1 : 0;
 }
 
 cudaError_t launch_walk(WalkArgs A, int prec, bool adjoint, cudaStream_t s, bool fused) {

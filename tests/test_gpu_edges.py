@@ -1,0 +1,59 @@
+"""Sizes at which the sort, the tree build and the walks change path: tile and
+block edges of the sort and the topology passes, one to four warps a group, a
+ragged last group, coincident particles down to the last level."""
+import numpy as np
+import pytest
+
+import ics
+from gpu_util import GRAD_TOL, device, grad_scaled_err, og, torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(n, seed, clumps=0):
+    rng = np.random.default_rng(seed)
+    pos = rng.random((n, 3))
+    if clumps:  # exact duplicates, more than a leaf of each: leaves of the last level
+        pos[: n // 2] = pos[rng.integers(0, clumps, n // 2)]
+    return pos, 0.5 + rng.random(n), np.full(n, 0.3 * n ** (-1 / 3))
+
+
+@pytest.mark.parametrize("n", [1, 511, 512, 513, 4095, 4096, 4097, 8193, 1024 * 32, 1024 * 32 + 1, 4096 * 32 + 33])
+@pytest.mark.parametrize("clumps", [0, 5])
+def test_sort_tree_and_walks(orc, n, clumps):
+    dev = device()
+    m = og()
+    pos, mass, eps = _case(n, n + clumps, clumps if n > 400 else 0)
+    p, mt, e = (torch.tensor(x, dtype=torch.float64, device=dev) for x in (pos, mass, eps))
+    keys, order = m.keys_sort(p, 1.0)
+    ks, o = orc.sort(orc.keys(pos, 1.0)[0])
+    assert np.array_equal(keys.cpu().numpy().view(np.uint64), ks) and np.array_equal(order.cpu().numpy(), o)
+    tree = m.tree_build(keys, order, p, mt, e, 1.0)
+    r_s = min(0.1, 0.7 * n ** (-1 / 3))
+    T = orc.Tree(pos, mass, 2.8 * eps, leaf_size=16)
+    assert tree.node_count() == T.nodes()["level"].shape[0]
+    tg = np.unique(np.concatenate([np.arange(max(0, n - 40), n), np.linspace(0, n - 1, 300).astype(int)]))
+    ref, cnt = T.walk(r_s, 4.5 * r_s, 0.5, targets=tg)
+    scale = max(np.sqrt((ref ** 2).sum(1).mean()), 1e-300)
+    # FP32 terms are good to about 2e-6 and FP64 ones to a few ulp; a target's
+    # error is that of its largest terms (close pairs), within 10 rms here
+    for prec, tol in (("fp32", 2e-5), ("fp64", 1e-13)):
+        acc, total, c = m.shortrange_accel(tree, r_s, 0.5, prec=prec, counts=True)
+        assert np.array_equal(c.cpu().numpy()[tg], cnt)
+        assert int(total.item()) == int(c.sum().item())
+        assert np.abs(acc.double().cpu().numpy()[tg] - ref).max() <= tol * max(scale, np.abs(ref).max())
+    # a range of groups gives the full walk's sums, and the fused walk the forward's
+    acc, total, _ = m.shortrange_accel(tree, r_s, 0.5)
+    part = torch.zeros_like(acc)
+    g = int(tree.header.n_groups)
+    for a, b in ((0, g // 3), (g // 3, g)):
+        m.shortrange_accel(tree, r_s, 0.5, out=part, groups=(a, b))
+    assert torch.equal(acc, part)
+    w = torch.tensor(ics.loss_weights(n, 5), dtype=torch.float32, device=dev)
+    fa, ft, _, dx, dm = m.shortrange_accel_adjoint(tree, r_s, 0.5, w)
+    assert torch.equal(fa, acc) and int(ft.item()) == int(total.item())
+    if n <= 8193:
+        s = tg[:: max(1, len(tg) // 60)]
+        gp, gm, sp, sm = T.adjoint(r_s, 4.5 * r_s, 0.5, w.double().cpu().numpy(), s, with_scale=True)
+        assert grad_scaled_err(dx.cpu().numpy()[s], gp, sp) < GRAD_TOL
+        assert grad_scaled_err(dm.cpu().numpy()[s], gm, sm) < GRAD_TOL
