@@ -57,3 +57,26 @@ def test_sort_tree_and_walks(orc, n, clumps):
         gp, gm, sp, sm = T.adjoint(r_s, 4.5 * r_s, 0.5, w.double().cpu().numpy(), s, with_scale=True)
         assert grad_scaled_err(dx.cpu().numpy()[s], gp, sp) < GRAD_TOL
         assert grad_scaled_err(dm.cpu().numpy()[s], gm, sm) < GRAD_TOL
+
+
+@pytest.mark.parametrize("n,n_ngb", [(97, 16), (129, 16), (1024 * 32, 32), (1024 * 32 + 5, 100)])
+def test_sph_sizes(n, n_ngb):
+    """SPH at few particles, one against four warps a group, more neighbours
+    than a list holds, in a set with denser clumps; h and rho as in
+    test_gpu_sph.py (float-float distances, second-order steps up to 3e-4)."""
+    from oracle import og_sph as S
+    dev = device()
+    m = og()
+    rng = np.random.default_rng(n)
+    pos = rng.random((n, 3))
+    pos[: n // 2] = np.mod(0.5 + 0.02 * rng.standard_normal((n // 2, 3)), 1.0)
+    mass = 0.5 + rng.random(n)
+    p, mt = (torch.tensor(x, dtype=torch.float64, device=dev) for x in (pos, mass))
+    keys, order = m.keys_sort(p, 1.0)
+    h, rho, ngb = m.sph_density(m.tree_build(keys, order, p, mt, 1e-3, 1.0), n_ngb)
+    tg = np.linspace(0, n - 1, min(n, 60)).astype(int)
+    ho = S.smoothing_length(pos, 1.0, n_ngb, targets=tg)
+    np.testing.assert_allclose(h.cpu().numpy()[tg], ho, rtol=1e-9)
+    np.testing.assert_allclose(rho.cpu().numpy()[tg], S.density(pos, mass, ho, 1.0, targets=tg), rtol=1e-9)
+    cnt = [int((S.distances(pos, int(i), 1.0) < ho[k]).sum()) - 1 for k, i in enumerate(tg)]
+    np.testing.assert_array_equal(ngb.cpu().numpy()[tg], cnt)
