@@ -24,8 +24,8 @@ _lib = None
 
 # Kernels libog.so launches per call (fixed sequences, see csrc/): keys (1) +
 # 8 radix passes; permute + count + scan + fill + leaves + upward; one walk;
-# adjoint walk + 22 push-down levels + the particle gather; SPH radius + density.
-LAUNCHES_PER_CALL = {"keys_sort": 1 + 8, "tree_build": 6, "accel": 1, "adjoint": 1 + 22 + 1,
+# adjoint walk + push-down + the particle gather; SPH radius + density.
+LAUNCHES_PER_CALL = {"keys_sort": 1 + 8, "tree_build": 6, "accel": 1, "adjoint": 3,
                      "pm": 3, "kick": 1, "drift": 1, "sph": 2}  # pm: deposit, Green, interpolation (plus cuFFT's kernels)
 
 

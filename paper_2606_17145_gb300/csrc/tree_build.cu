@@ -31,22 +31,48 @@
 namespace og {
 
 
+// The bucket of a group in the order of the walks: half an octave of its box's
+// volume each, the smallest volume (the densest group, whose targets have the
+// most terms) first.  Every lane of the warp calls it.
+__device__ __forceinline__ void group_bucket(const TreeDev& T, int64_t g, bool live, const float hi[3]) {
+  float v = 1.0f;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {  // split parts are not negative: they order like their bits
+    const uint32_t a = __reduce_min_sync(0xffffffffu, live ? __float_as_uint(hi[c]) : 0x7f800000u);
+    const uint32_t b = __reduce_max_sync(0xffffffffu, live ? __float_as_uint(hi[c]) : 0u);
+    v *= __uint_as_float(b) - __uint_as_float(a) + 1.1920929e-07f;
+  }
+  const int bucket = min(max((int)(__float_as_uint(v) >> 22) - 2 * (127 - 63), 0), kBuckets - 1);
+  if ((threadIdx.x & 31) == 0) {
+    T.gbucket[g] = (unsigned char)bucket;
+    atomicAdd(&T.gcount[bucket], 1);
+  }
+}
+
 __global__ void k_permute(BuildArgs A, BoxScale B) {
   const TreeDev& T = A.T;
   const double invL2 = B.invL * B.invL;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < T.n; k += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t i = A.order[k];
+  // a warp's 32 particles are one walk group
+  for (int64_t k0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); k0 < T.n;
+       k0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k = k0 + (threadIdx.x & 31);
+    const bool live = k < T.n;
+    const int32_t i = live ? A.order[k] : 0;
     double w[3];
-    float hi[3], lo[3];
+    float hi[3] = {0.f, 0.f, 0.f}, lo[3];
     bool ok = true;
+    if (live) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double x = A.pos[3 * (int64_t)i + c];
-      ok = ok && finite_bits(x);
-      w[c] = wrap_coord(x, B);
-      split_box(w[c], B, hi[c], lo[c]);
-      T.x64[3 * k + c] = w[c];
+      for (int c = 0; c < 3; ++c) {
+        const double x = A.pos[3 * (int64_t)i + c];
+        ok = ok && finite_bits(x);
+        w[c] = wrap_coord(x, B);
+        split_box(w[c], B, hi[c], lo[c]);
+        T.x64[3 * k + c] = w[c];
+      }
     }
+    if (T.ngroups <= kOrderedGroups) group_bucket(T, k0 / kGroup, live, hi);
+    if (!live) continue;
     const double m = A.mass[i];
     const double eps = A.eps ? A.eps[i] : A.eps_scalar;
     if (!(ok && positive_finite_bits(m) && positive_finite_bits(eps))) set_status(T.sb, ST_BADINPUT);
@@ -117,9 +143,30 @@ __global__ void __launch_bounds__(kTopoThreads) k_count(TreeDev T, const uint64_
 }
 
 // One block per level: exclusive scan of its counts over the blocks, in
-// place, and the level's total.
+// place, and the level's total.  The blocks after those write the walks' order
+// of the groups, bucket by bucket (within one in the order their warps get
+// there; no result depends on it).
 __global__ void __launch_bounds__(1024) k_scan(TreeDev T) {
   __shared__ int s_w[32];
+  if (blockIdx.x >= kLevels) {
+    __shared__ int s_base[kBuckets];
+    if (threadIdx.x < kBuckets) {
+      int b = 0;
+      for (int i = 0; i < (int)threadIdx.x; ++i) b += T.gcount[i];
+      s_base[threadIdx.x] = b;
+    }
+    __syncthreads();
+    const int64_t g = (int64_t)(blockIdx.x - kLevels) * 1024 + threadIdx.x;
+    const int bucket = g < T.ngroups ? T.gbucket[g] : kBuckets;
+    const uint32_t peers = __match_any_sync(0xffffffffu, bucket);
+    const int first = __ffs(peers) - 1;
+    const int lane = threadIdx.x & 31;
+    int at = 0;
+    if (lane == first && bucket < kBuckets) at = atomicAdd(&T.gcount[kBuckets + bucket], __popc(peers));
+    at = __shfl_sync(0xffffffffu, at, first) + __popc(peers & ((1u << lane) - 1u));
+    if (bucket < kBuckets) T.gorder[s_base[bucket] + at] = (int32_t)g;
+    return;
+  }
   int* row = T.blk + blockIdx.x * T.nblk;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int carry = 0;
@@ -304,26 +351,6 @@ __global__ void __launch_bounds__(256) k_leaves(TreeDev T, BoxScale B) {
   }
 }
 
-// Polls of the grid barrier before it gives up (seconds, far above a level).
-constexpr int kBarrierPolls = 1 << 24;
-
-// Barrier over the grid of a cooperative launch; false if it gave up.  Every
-// block passes the same number of blocks * phase.
-__device__ bool grid_barrier(unsigned long long* count, unsigned long long target) {
-  __shared__ int s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(count, 1ull);
-    int ok = 0;
-    for (int i = 0; i < kBarrierPolls && !ok; ++i) ok = *(volatile unsigned long long*)count >= target;
-    __threadfence();
-    s_ok = ok;
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
-
 // The split nodes, from the deepest level up.
 constexpr int kUpThreads = 512;
 __global__ void __launch_bounds__(kUpThreads) k_upward(TreeDev T, BoxScale B) {
@@ -392,7 +419,8 @@ cudaError_t launch_tree_build(const BuildArgs& A, cudaStream_t s) {
   const BoxScale B = box_scale(A.L);
   k_permute<<<(unsigned)grid, 256, 0, s>>>(A, B);
   k_count<<<(unsigned)T.nblk, kTopoThreads, 0, s>>>(T, A.keys, A.leaf_size);
-  k_scan<<<kLevels, 1024, 0, s>>>(T);
+  const int64_t oblocks = T.ngroups <= kOrderedGroups ? (T.ngroups + 1023) / 1024 : 0;
+  k_scan<<<(unsigned)(kLevels + oblocks), 1024, 0, s>>>(T);
   k_fill<<<(unsigned)T.nblk, kTopoThreads, 0, s>>>(T, A.keys, A.leaf_size);
   // the node counts live on the device: grids are sized for the particles
   int64_t lgrid = (T.n / 2 + 255) / 256;

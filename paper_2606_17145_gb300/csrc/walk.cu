@@ -1227,10 +1227,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   // 2^split warps serve a group, each its part of the targets
   const int64_t v = (int64_t)blockIdx.x * kWarpsPerBlock + wib;
-  const int64_t g = A.g_begin + (v >> A.split);
-  if (g >= A.g_end) return;
+  const int64_t gi = A.g_begin + (v >> A.split);
+  if (gi >= A.g_end) return;
+  const bool usable = T.sb->status == 0 && T.sb->magic == kMagicTree;
+  const int64_t g = A.ordered && usable ? T.gorder[gi] : gi;
   const bool mine = (lane >> (5 - A.split)) == (int)(v & ((1 << A.split) - 1));
-  if (T.sb->status != 0 || T.sb->magic != kMagicTree) {
+  if (!usable) {
     // a failed or missing tree: flag it and give every output of this
     // group's targets NaN, so that nothing downstream can take stale values
     // for forces.  A tree whose build started wrote its permutation first;
@@ -1513,13 +1515,11 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
 // 1.58 / 1.67.  FP64: 128 groups 1.59 / 0.94 / 0.68, 1024 clustered 1.60 / 1.06 /
 // 0.91, zoom 8.2 / 8.0 / 9.1, lattice 0.40 / 0.37 / 0.44; 5860 (zoom) 71.6 / 72.9 / 83.0,
 // 8192 clustered 7.7 / 6.8 / 6.7, lattice 1.90 / 1.94 / 2.31.
-static int walk_split(int64_t n_groups, bool f64) {
-  if (n_groups <= 1024) return 2;
-  return n_groups <= (f64 ? 8192 : 4096) ? 1 : 0;
-}
+static int walk_split(int64_t n_groups) { return n_groups <= 1024 ? 2 : n_groups <= 4096 ? 1 : 0; }
 
 cudaError_t launch_walk(WalkArgs A, int prec, bool adjoint, cudaStream_t s, bool fused) {
-  A.split = walk_split(A.T.ngroups, prec == OG_FP64);
+  A.split = walk_split(A.T.ngroups);
+  A.ordered = A.g_begin == 0 && A.g_end == A.T.ngroups && A.T.ngroups <= kOrderedGroups;
   const int64_t blocks = (((A.g_end - A.g_begin) << A.split) + kWarpsPerBlock - 1) / kWarpsPerBlock;
   if (blocks <= 0) return cudaSuccess;
   if (fused) k_walk<LaneFused><<<(unsigned)blocks, kWarpsPerBlock * 32, 0, s>>>(A);
