@@ -80,3 +80,61 @@ def test_sph_sizes(n, n_ngb):
     np.testing.assert_allclose(rho.cpu().numpy()[tg], S.density(pos, mass, ho, 1.0, targets=tg), rtol=1e-9)
     cnt = [int((S.distances(pos, int(i), 1.0) < ho[k]).sum()) - 1 for k, i in enumerate(tg)]
     np.testing.assert_array_equal(ngb.cpu().numpy()[tg], cnt)
+
+
+def _mesh_ref(pos, mass, N, r_s):
+    """The mesh force in torch FP64 on the device (unit box)."""
+    dev = pos.device
+    u = pos * N
+    i0 = torch.floor(u).long()
+    f = u - i0
+    w = [(1 - f[:, a], f[:, a]) for a in range(3)]
+    rho = torch.zeros(N ** 3, dtype=torch.float64, device=dev)
+    nodes = []
+    for o in range(8):
+        b = (o >> 2, (o >> 1) & 1, o & 1)
+        i = [(i0[:, a] + b[a]) % N for a in range(3)]
+        nodes.append(((i[0] * N + i[1]) * N + i[2], w[0][b[0]] * w[1][b[1]] * w[2][b[2]]))
+        rho.index_add_(0, nodes[-1][0], mass * nodes[-1][1])
+    hat = torch.fft.rfftn(rho.view(N, N, N))
+    del rho
+    k = torch.fft.fftfreq(N, 1.0 / N, dtype=torch.float64, device=dev)
+    kz = torch.arange(N // 2 + 1, dtype=torch.float64, device=dev)
+    for x in range(N):  # plane by plane: the largest mesh has 10^9 nodes
+        k2 = (2 * np.pi) ** 2 * (k[x] ** 2 + k[:, None] ** 2 + kz[None, :] ** 2)
+        S = (torch.sinc(k[x] / N) * torch.sinc(k / N)[:, None] * torch.sinc(kz / N)[None, :]) ** 4
+        g = -4 * np.pi * torch.exp(-k2 * r_s ** 2) / (k2 * S) * N ** 3
+        if x == 0:
+            g[0, 0] = 0.0
+        hat[x] *= g
+    phi = torch.fft.irfftn(hat, s=(N, N, N))
+    del hat
+    acc = torch.zeros_like(pos)
+    st = (N * N, N, 1)
+    for j, wt in nodes:
+        c = [j // (N * N), (j // N) % N, j % N]
+        for a in range(3):
+            v = [phi.view(-1)[j + ((c[a] + s) % N - c[a]) * st[a]] for s in (-2, -1, 1, 2)]
+            acc[:, a] -= wt * N * ((2 / 3) * (v[2] - v[1]) - (1 / 12) * (v[3] - v[0]))
+    return acc
+
+
+@pytest.mark.parametrize("N", [8, 12, 16, 32, 64, 100, 128, 256, 512, 1024])
+def test_pm_mesh_sides(N):
+    """Every side's transform path (3-D, or planes and the fused x pass), with
+    particles beside every face; bounds of test_gpu_pm.py."""
+    dev = device()
+    m = og()
+    rng = np.random.default_rng(N)
+    pos = rng.random((3000, 3))
+    pos[:600] = np.mod(rng.normal(scale=1.5 / N, size=(600, 3)), 1.0)
+    pos[600:900, 2] = np.mod(rng.normal(scale=2.0 / N, size=300), 1.0)
+    p = torch.tensor(pos, dtype=torch.float64, device=dev)
+    mt = torch.tensor(0.5 + rng.random(3000), dtype=torch.float64, device=dev)
+    plan = m.PMPlan(N)
+    a = m.pm_accel(plan, p, mt, 1.0, 1.25 / N).double()
+    ref = _mesh_ref(p, mt, N, 1.25 / N)
+    d = (a - ref).norm(dim=1)
+    scale = ref.square().sum(1).mean().sqrt()
+    plan.close()
+    assert float(d.square().mean().sqrt() / scale) < 5e-6 and float(d.max() / scale) < 5e-5
