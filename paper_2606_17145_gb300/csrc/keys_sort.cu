@@ -82,33 +82,44 @@ __device__ __forceinline__ uint64_t hilbert63(uint32_t a, uint32_t b, uint32_t c
 
 constexpr int kKeyThreads = 256;
 
+// Key of one position; 0 and the status flag for a non-finite one.
+__device__ __forceinline__ uint64_t position_key(const double* __restrict__ pos, int64_t i, const BoxScale& B,
+                                                 StatusBlock* sb) {
+  const double x0 = pos[3 * i], x1 = pos[3 * i + 1], x2 = pos[3 * i + 2];
+  if (!(finite_bits(x0) && finite_bits(x1) && finite_bits(x2))) {
+    set_status(sb, ST_BADINPUT);
+    return 0;
+  }
+  return hilbert63(quantise(wrap_coord(x0, B), B), quantise(wrap_coord(x1, B), B), quantise(wrap_coord(x2, B), B));
+}
+
+// PASSES: also what the radix passes need, the digits' counts and clear tile counts.
+template <bool PASSES>
 __global__ void __launch_bounds__(kKeyThreads) k_keys(const double* __restrict__ pos, int64_t n, BoxScale B,
                                                       uint64_t* __restrict__ keys, SortWs W) {
-  __shared__ uint32_t h[8 * 256];
-  for (int i = threadIdx.x; i < 8 * 256; i += kKeyThreads) h[i] = 0u;
-  __syncthreads();
+  __shared__ uint32_t h[PASSES ? 8 * 256 : 1];
+  if (PASSES) {
+    for (int i = threadIdx.x; i < 8 * 256; i += kKeyThreads) h[i] = 0u;
+    __syncthreads();
+  }
   const int64_t stride = (int64_t)gridDim.x * kKeyThreads;
   const int64_t first = blockIdx.x * (int64_t)kKeyThreads + threadIdx.x;
   // the first pass's tile counts start at zero
-  for (int64_t i = first; i < W.ntiles * 256; i += stride) W.tile_state[0][i] = 0u;
+  if (PASSES)
+    for (int64_t i = first; i < W.ntiles * 256; i += stride) W.tile_state[0][i] = 0u;
   for (int64_t i = first; i < n; i += stride) {
-    const double x0 = pos[3 * i], x1 = pos[3 * i + 1], x2 = pos[3 * i + 2];
-    uint64_t key = 0;
-    if (finite_bits(x0) && finite_bits(x1) && finite_bits(x2)) {
-      const uint32_t q0 = quantise(wrap_coord(x0, B), B);
-      const uint32_t q1 = quantise(wrap_coord(x1, B), B);
-      const uint32_t q2 = quantise(wrap_coord(x2, B), B);
-      key = hilbert63(q0, q1, q2);
-    } else {
-      set_status(W.sb, ST_BADINPUT);
-    }
+    const uint64_t key = position_key(pos, i, B, W.sb);
     keys[i] = key;
+    if (PASSES) {
 #pragma unroll
-    for (int d = 0; d < 8; ++d) atomicAdd(&h[256 * d + ((key >> (8 * d)) & 255u)], 1u);
+      for (int d = 0; d < 8; ++d) atomicAdd(&h[256 * d + ((key >> (8 * d)) & 255u)], 1u);
+    }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 8 * 256; i += kKeyThreads)
-    if (h[i]) atomicAdd(&W.hist[i], h[i]);
+  if (PASSES) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < 8 * 256; i += kKeyThreads)
+      if (h[i]) atomicAdd(&W.hist[i], h[i]);
+  }
 }
 
 // A tile's published state for one digit: 0 nothing yet, 1 + count its own
@@ -267,6 +278,60 @@ __global__ void __launch_bounds__(kSortThreads, 3)
   }
 }
 
+// A small sort by counting: a key's place is the number of keys before it.  32
+// keys a block (lane = key), which compare themselves with all keys, a chunk
+// at a time from shared memory, each warp its share of the chunk.  n^2
+// comparisons, but two launches and no pass after pass: 4096 keys 78 -> 18 us
+// (host-bound), 8192 83 -> 28, 16,384 83 -> 63; at 20,000 the passes (82 us) catch up.
+constexpr int kRankWarps = 16;
+constexpr int kRankChunk = 4096;
+constexpr int64_t kRankMax = 16384;
+__global__ void __launch_bounds__(kRankWarps * 32) k_sort_rank(const uint64_t* __restrict__ keys, int n,
+                                                               uint64_t* __restrict__ keys_out,
+                                                               int32_t* __restrict__ order_out) {
+  __shared__ __align__(16) uint64_t s_keys[kRankChunk];
+  __shared__ int s_before[kRankWarps][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
+  const uint64_t key = i < n ? keys[i] : 0;
+  int before = 0;
+  constexpr int kShare = kRankChunk / kRankWarps;
+  for (int c0 = 0; c0 < n; c0 += kRankChunk) {
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kRankChunk; k += kRankWarps * 32) {
+      const int j = c0 + k + threadIdx.x;
+      s_keys[k + threadIdx.x] = j < n ? keys[j] : ~0ull;  // past the end: behind every key
+    }
+    __syncthreads();
+    const ulonglong2* s = reinterpret_cast<const ulonglong2*>(s_keys + w * kShare);
+    const int j0 = c0 + w * kShare, own = blockIdx.x * 32;
+    // equal keys keep their order: those ahead of this block's keys count,
+    // those behind do not, and in its own part the index decides
+    if (j0 + kShare <= own) {
+#pragma unroll 8
+      for (int k = 0; k < kShare / 2; ++k) before += (s[k].x <= key ? 1 : 0) + (s[k].y <= key ? 1 : 0);
+    } else if (j0 >= own + 32) {
+#pragma unroll 8
+      for (int k = 0; k < kShare / 2; ++k) before += (s[k].x < key ? 1 : 0) + (s[k].y < key ? 1 : 0);
+    } else {
+      for (int k = 0; k < kShare; ++k) {
+        const uint64_t other = s_keys[w * kShare + k];
+        before += other < key || (other == key && j0 + k < i) ? 1 : 0;
+      }
+    }
+  }
+  s_before[w][lane] = before;
+  __syncthreads();
+  if (w == 0 && i < n) {
+    int at = 0;
+#pragma unroll
+    for (int ww = 0; ww < kRankWarps; ++ww) at += s_before[ww][lane];
+    keys_out[at] = key;
+    order_out[at] = i;
+  }
+}
+
 cudaError_t launch_keys_sort(const double* pos, int64_t n, double L, uint64_t* keys_out, int32_t* order_out,
                              const SortWs& W, cudaStream_t s) {
   // status, tile counters and histograms start at zero
@@ -274,7 +339,12 @@ cudaError_t launch_keys_sort(const double* pos, int64_t n, double L, uint64_t* k
   if (e != cudaSuccess) return e;
   int64_t kgrid = (n + kKeyThreads - 1) / kKeyThreads;
   if (kgrid > grid_cap(8)) kgrid = grid_cap(8);
-  k_keys<<<(unsigned)kgrid, kKeyThreads, 0, s>>>(pos, n, box_scale(L), keys_out, W);
+  if (n <= kRankMax) {
+    k_keys<false><<<(unsigned)kgrid, kKeyThreads, 0, s>>>(pos, n, box_scale(L), W.keys_alt, W);
+    k_sort_rank<<<(unsigned)((n + 31) / 32), kRankWarps * 32, 0, s>>>(W.keys_alt, (int)n, keys_out, order_out);
+    return cudaGetLastError();
+  }
+  k_keys<true><<<(unsigned)kgrid, kKeyThreads, 0, s>>>(pos, n, box_scale(L), keys_out, W);
   uint64_t* kin = keys_out;
   int32_t* vin = order_out;
   uint64_t* ko = W.keys_alt;

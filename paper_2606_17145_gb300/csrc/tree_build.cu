@@ -24,8 +24,8 @@
 // all) cost 180 us on 4096 particles, most of it for empty levels.  Whole force
 // passes, build alone changed: 4096 particles 500 -> 294 us, 64^3 leapfrog step
 // 1050 -> 887 us, 100,003-particle SPH 1.15 -> 0.96 ms.  At 2.1 M particles the
-// kernels take 0.095 (permute), 0.02, 0.008, 0.083 (fill: the searches for the
-// ends of runs), 0.049 (leaves) and 0.09 ms (upward).
+// kernels take 0.063 (permute), 0.020, 0.008, 0.077 (fill), 0.048 (leaves) and
+// 0.084 ms (upward).
 #include "og_internal.cuh"
 
 namespace og {
@@ -203,6 +203,7 @@ __device__ __forceinline__ int level_base(const StatusBlock* sb, int level) {
 // moments, where a node meets its children.
 __global__ void __launch_bounds__(kTopoThreads) k_fill(TreeDev T, const uint64_t* __restrict__ keys, int leaf_size) {
   __shared__ signed char s_far[kTopoThreads + kMaxLeaf];
+  __shared__ uint32_t s_ends[kLevels][kTopoThreads / 32];  // keys at which a run of the level (and a node) starts
   __shared__ int s_first[kLevels];                      // index of this block's first node of each level
   __shared__ int s_warp[kTopoThreads / 32][kLevels];    // nodes of each level in each warp, then in the warps before it
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -212,14 +213,18 @@ __global__ void __launch_bounds__(kTopoThreads) k_fill(TreeDev T, const uint64_t
     for (int ww = 0; ww < kTopoThreads / 32; ++ww) s_warp[ww][threadIdx.x] = 0;
   }
   int lo, hi, deep;
-  const int64_t i = blockIdx.x * (int64_t)kTopoThreads + threadIdx.x;
-  node_levels(keys, T.n, leaf_size, blockIdx.x * (int64_t)kTopoThreads, s_far, lo, hi, deep);
+  const int64_t i0 = blockIdx.x * (int64_t)kTopoThreads, i = i0 + threadIdx.x;
+  node_levels(keys, T.n, leaf_size, i0, s_far, lo, hi, deep);
   const bool any = lo <= hi;
   const int wlo = (int)__reduce_min_sync(0xffffffffu, (unsigned)(any ? lo : kLevels));
   const int whi = (int)__reduce_max_sync(0xffffffffu, (unsigned)(any ? hi + 1 : 0)) - 1;
   for (int l = wlo; l <= whi; ++l) {
     const uint32_t m = __ballot_sync(0xffffffffu, l >= lo && l <= hi);
     if (lane == 0) s_warp[w][l] = __popc(m);
+  }
+  for (int l = 1; l < kLevels; ++l) {
+    const uint32_t m = __ballot_sync(0xffffffffu, any && lo <= l);
+    if (lane == 0) s_ends[l][w] = m;
   }
   __syncthreads();
   if (threadIdx.x < kLevels) {
@@ -244,11 +249,23 @@ __global__ void __launch_bounds__(kTopoThreads) k_fill(TreeDev T, const uint64_t
     if (l == 0) {
       end = T.n;
     } else {
-      // first key at or after `end` whose top l digits differ
+      // The run ends at the next key that starts a run of level l.  A node
+      // starts there too: the two keys' deepest common node is split, so the
+      // first level at which they differ has one.  In this block the starts
+      // are in s_ends; past it the end is searched for.
       const int shift = 63 - 3 * l;
       const uint64_t pre = keys[i] >> shift;
       int64_t step = 1;
-      while (end < T.n && (keys[end] >> shift) == pre) {
+      int ww = w;
+      uint32_t next = lane < 31 ? s_ends[l][w] & (0xfffffffeu << lane) : 0u;
+      while (next == 0u && ++ww < kTopoThreads / 32) next = s_ends[l][ww];
+      if (next) {
+        end = i0 + 32 * ww + __ffs(next) - 1;
+        step = 0;
+      } else {
+        end = max(end, min(i0 + kTopoThreads, T.n));
+      }
+      while (step > 0 && end < T.n && (keys[end] >> shift) == pre) {
         const int64_t probe = end + step;
         if (probe < T.n && (keys[probe] >> shift) == pre) {
           end = probe + 1;
@@ -381,20 +398,42 @@ __global__ void __launch_bounds__(kUpThreads) k_upward(TreeDev T, BoxScale B) {
       const int p = base + s;
       int4 D = T.nD[p];
       if (meta_leaf(D.w)) continue;
+      // the children's counts first (independent loads), which give their
+      // number, then their sums: two memory latencies a level instead of one
+      // a child (4096 particles: 28 -> 23 us)
+      int nch = 0, left = D.y;
+      int cy[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) cy[c] = D.z + c < total ? T.nD[D.z + c].y : 0;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        if (left > 0) ++nch;
+        left -= cy[c];
+      }
+      double m8[8], s8[3][8], h8[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const int64_t q = D.z + (c < nch ? c : 0);
+        m8[c] = __ldcg(&T.mass64[q]);
+        s8[0][c] = __ldcg(&T.S64[3 * q]);
+        s8[1][c] = __ldcg(&T.S64[3 * q + 1]);
+        s8[2][c] = __ldcg(&T.S64[3 * q + 2]);
+        h8[c] = __ldcg(&T.hmax64[q]);
+      }
       double M = 0.0, S0 = 0.0, S1 = 0.0, S2 = 0.0;
       long long Hb = 0;
-      int c = D.z, left = D.y;
-      while (left > 0 && c < total) {
-        M += __ldcg(&T.mass64[c]);
-        S0 += __ldcg(&T.S64[3 * (int64_t)c]);
-        S1 += __ldcg(&T.S64[3 * (int64_t)c + 1]);
-        S2 += __ldcg(&T.S64[3 * (int64_t)c + 2]);
-        Hb = max(Hb, __double_as_longlong(__ldcg(&T.hmax64[c])));
-        T.nParent[c] = p;
-        left -= T.nD[c].y;
-        ++c;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        if (c < nch) {
+          M += m8[c];
+          S0 += s8[0][c];
+          S1 += s8[1][c];
+          S2 += s8[2][c];
+          Hb = max(Hb, __double_as_longlong(h8[c]));
+          T.nParent[D.z + c] = p;
+        }
       }
-      D.w = make_meta(c - D.z, l, 0);
+      D.w = make_meta(nch, l, 0);
       T.nD[p] = D;
       write_moments(T, B, p, D, M, S0, S1, S2, __longlong_as_double(Hb));
     }
