@@ -891,10 +891,11 @@ struct LaneFP {
   // lanes once per batch.  Measured against listing the pairs one by one,
   // 32 per iteration, with a segmented scan for the sums (full lanes, but the
   // list, the gathered operands and the scan cost two thirds of the pair
-  // work): forward 3.17 -> 2.68 ms on the 128^3 lattice, 23.2 -> 19.2 ms on the
+  // work): forward 3.17 -> 2.56 ms on the 128^3 lattice, 23.2 -> 18.5 ms on the
   // 128^3 clustered set, 0.66 -> 0.36 ms on 4096 particles (one group per SM);
-  // adjoint 4.61 -> 3.73 and 33.3 -> 25.0 ms.  Loading the next iteration's pair
-  // before the current one is evaluated is a fifth of that on 4096 particles.
+  // adjoint 4.61 -> 3.73 and 33.3 -> 25.0 ms.  The next list entry is read
+  // ahead; loading its pair ahead as well costs 4 % (19.2 and 2.68 ms forward,
+  // 27.3 against 25.3 ms with both directions in one walk).
   __device__ void batch_tiles(const WalkArgs& A, const WarpBufs& W, Stage& St, Smem& M, const float4* SGB,
                               int cnt, int lane, int64_t gbase, uint32_t vmask, bool mi) {
     // an odd count leaves the last pair's second slot empty: its data must be finite
@@ -968,17 +969,14 @@ struct LaneFP {
       }
       Sums S = {0, 0, 0, 0, 0, 0};
       uint32_t rare = 0u;  // bit i: iteration i of the list holds a pair the packed form does not cover
-      // the next iteration's pair is loaded, up to its squared distances,
-      // before the current one is evaluated
+      // the next iteration's list entry is read ahead
       int kn = list[32 * g + min(lane >> 3, n - 1)];
-      Pair pn = load_pair(St, T, kn, mi);
 #pragma unroll 1
       for (int e0 = 0; e0 < n; e0 += 4) {
         const int e = e0 + (lane >> 3);
         const int k = kn;
-        const Pair p = pn;
         kn = list[32 * g + min(e + 4, n - 1)];
-        pn = load_pair(St, T, kn, mi);
+        const Pair p = load_pair(St, T, k, mi);
         const bool h0 = e < n && ((q0m >> k) & 1u) && lo2(p.r2) <= A.pp_hi;
         const bool h1 = e < n && ((q1m >> k) & 1u) && hi2(p.r2) <= A.pp_hi;
         const bool p0 = h0 && plain(A, lo2(p.r2), p.h20), p1 = h1 && plain(A, hi2(p.r2), p.h21);
