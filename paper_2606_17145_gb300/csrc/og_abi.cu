@@ -112,7 +112,7 @@ og_status og_tree_build(const uint64_t* keys_sorted, const int32_t* order, const
   A.eps_scalar = eps_scalar;
   A.L = box;
   A.leaf_size = q.leaf_size;
-  cudaError_t e = cudaMemsetAsync(A.T.sb, 0, kTreeZeroBytes, s);
+  cudaError_t e = cudaMemsetAsync(A.T.sb, 0, A.T.zero_bytes, s);
   if (e != cudaSuccess) return OG_ECUDA;
   e = launch_tree_build(A, s);
   if (e != cudaSuccess) return OG_ECUDA;

@@ -26,14 +26,8 @@ enum : uint32_t {
 constexpr int kMaxLevel = 21;         // 21 bits per axis
 constexpr int kLevels = kMaxLevel + 1;
 constexpr int kGroup = 32;            // targets per walk group (one warp)
-constexpr int kBuckets = 128;         // of the walk groups' volumes
-// Walks of up to this many groups take them densest first: the groups with the
-// most terms then do not start last.  With 187,501 zoom particles (5860 groups)
-// 17.6 -> 14.7 ms forward, 22.7 -> 18.8 adjoint, 72 -> 64 FP64; 64^3 clustered (8192
-// groups) 1.78 -> 1.76, 2.34 -> 2.37.  Many waves lose more to the scattered order
-// than they gain: 128^3 clustered (65,536) 19.4 -> 22.1, 24.7 -> 28.1 (20.7 and 26.5
-// with two classes instead of 128), 90^3 4.97 -> 5.07.
-constexpr int kOrderedGroups = 8192;
+constexpr int kBuckets = 128;         // of the walk groups' estimated work
+constexpr int kOrderTile = 1024;      // walk groups per row of the bucket counts
 constexpr int kTopoBlock = 512;       // keys per block of the tree build's topology passes
 constexpr size_t kAlign = 256;
 
@@ -88,15 +82,26 @@ struct TreeDev {
   double* mass64;  // [cap]
   double* hmax64;  // [cap]
   double* cen64;   // [cap][3] physical geometric centres
-  // up to kOrderedGroups walk groups, densest first
-  int32_t* gorder;         // [ngroups]
-  unsigned char* gbucket;  // [ngroups]
-  int* gcount;             // [2 * kBuckets]: groups of each bucket, groups placed
+  // the walk groups by estimated work, most first (tree_build.cu): in the FP32
+  // walks, in the FP64 walk
+  int32_t* gorder[2];         // [ngroups]; during the build, [0]: the volume of each group's box
+  unsigned char* gbucket[2];  // [ngroups]
+  int* gtile[2];              // [ntiles][kBuckets] build scratch: groups per bucket of each kOrderTile groups
+  int* gcell;              // [8^cell_level] build scratch: particles per cell
+  int64_t ntiles;
+  int cell_level;
+  size_t zero_bytes;
   int* blk;        // [kLevels][nblk] build scratch: nodes of each level per block of kTopoBlock keys
   int64_t nblk;
 };
 
-constexpr size_t kTreeZeroBytes = kAlign + sizeof(int) * 2 * kBuckets;  // status block and bucket counts
+// Level of the cells that the groups' work is estimated from: a side of 4 to 8
+// mean particle spacings.
+inline int order_cell_level(int64_t n) {
+  int lg = 0;
+  while ((n >> (lg + 1)) > 0) ++lg;
+  return lg / 3 > 2 ? lg / 3 - 2 : 0;
+}
 
 // Carves a tree buffer.  Returns the total byte count (buf may be null).
 inline size_t carve_tree(void* buf, int64_t n, int64_t cap, TreeDev* T) {
@@ -110,7 +115,11 @@ inline size_t carve_tree(void* buf, int64_t n, int64_t cap, TreeDev* T) {
   int64_t G = (n + kGroup - 1) / kGroup;
   TreeDev t{};
   t.sb = static_cast<StatusBlock*>(take(sizeof(StatusBlock)));
-  t.gcount = static_cast<int*>(take(sizeof(int) * 2 * kBuckets));
+  t.ntiles = (G + kOrderTile - 1) / kOrderTile;
+  t.cell_level = order_cell_level(n);
+  for (int o = 0; o < 2; ++o) t.gtile[o] = static_cast<int*>(take(sizeof(int) * kBuckets * t.ntiles));
+  t.gcell = static_cast<int*>(take(sizeof(int) << (3 * t.cell_level)));
+  t.zero_bytes = off;  // all of the above is zeroed before a build
   t.n = n;
   t.cap = cap;
   t.ngroups = G;
@@ -131,8 +140,8 @@ inline size_t carve_tree(void* buf, int64_t n, int64_t cap, TreeDev* T) {
   t.mass64 = static_cast<double*>(take(sizeof(double) * cap));
   t.hmax64 = static_cast<double*>(take(sizeof(double) * cap));
   t.cen64 = static_cast<double*>(take(sizeof(double) * 3 * cap));
-  t.gorder = static_cast<int32_t*>(take(sizeof(int32_t) * G));
-  t.gbucket = static_cast<unsigned char*>(take(G));
+  for (int o = 0; o < 2; ++o) t.gorder[o] = static_cast<int32_t*>(take(sizeof(int32_t) * G));
+  for (int o = 0; o < 2; ++o) t.gbucket[o] = static_cast<unsigned char*>(take(G));
   t.nblk = (n + kTopoBlock - 1) / kTopoBlock;
   t.blk = static_cast<int*>(take(sizeof(int) * kLevels * t.nblk));
   if (T) *T = t;

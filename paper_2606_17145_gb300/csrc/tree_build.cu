@@ -31,22 +31,139 @@
 namespace og {
 
 
-// The bucket of a group in the order of the walks: half an octave of its box's
-// volume each, the smallest volume (the densest group, whose targets have the
-// most terms) first.  Every lane of the warp calls it.
-__device__ __forceinline__ void group_bucket(const TreeDev& T, int64_t g, bool live, const float hi[3]) {
+// The order of the walk groups.  A walk takes the groups with the most work
+// first, so that no long group starts when the others are done.  Started in
+// tree order, the SMs of a 90^3 clustered walk are busy 75 % of its time, and
+// with 78 % of their warps.  Work follows the sources within reach, and grows
+// with the group's own box (its targets then share fewer of them):
+//   w = (particles in the 8 cells nearest a target) (box volume / mean volume)^(1/4),
+// the count averaged over four targets of the group, cells of 4 to 8 mean
+// spacings.  Groups are sorted by half octaves of w, in tree order within one
+// (which keeps neighbours together).  Forward walk, ms, tree order / this
+// order / sorted by measured time: 187,501 zoom particles 16.7 / 12.3 / 11.8,
+// clustered 64^3 1.74 / 1.38 / 1.38, 90^3 4.62 / 3.52 / 3.21, 128^3 18.2 / 16.8 /
+// 15.8; 128^3 lattice 2.52 / 2.51.  The box volume alone says little (18.2 ->
+// 20.0 at 128^3): the heavy groups are those that lie between dense clumps.  In
+// the FP64 walk, where the pairs are nearly all of the work, the count alone
+// tells more (clustered 64^3 7.6 / 6.5 / 6.8 ms, 7.7 with the volume).  Whole
+// octaves: zoom 13.7 ms; other powers of the volume from 0.2 to 0.3: zoom
+// 14.0 - 12.3, 90^3 3.50 - 3.69.  The orders cost the build 4 us at 2.1 M.
+
+// Counts the particles per cell (consecutive particles of a cell together) and
+// leaves each group's box volume in T.gorder.  Every lane of the warp calls it.
+__device__ __forceinline__ void group_cells(const TreeDev& T, int64_t g, bool live, const float hi[3]) {
+  const int lane = threadIdx.x & 31;
+  const int N = 1 << T.cell_level;
+  int cell = 0;
   float v = 1.0f;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {  // split parts are not negative: they order like their bits
     const uint32_t a = __reduce_min_sync(0xffffffffu, live ? __float_as_uint(hi[c]) : 0x7f800000u);
     const uint32_t b = __reduce_max_sync(0xffffffffu, live ? __float_as_uint(hi[c]) : 0u);
     v *= __uint_as_float(b) - __uint_as_float(a) + 1.1920929e-07f;
+    cell = cell * N + min(max((int)(hi[c] * (float)N), 0), N - 1);
   }
-  const int bucket = min(max((int)(__float_as_uint(v) >> 22) - 2 * (127 - 63), 0), kBuckets - 1);
-  if ((threadIdx.x & 31) == 0) {
-    T.gbucket[g] = (unsigned char)bucket;
-    atomicAdd(&T.gcount[bucket], 1);
+  const int before = __shfl_up_sync(0xffffffffu, cell, 1);
+  const uint32_t lives = __ballot_sync(0xffffffffu, live);
+  const bool head = live && (lane == 0 || before != cell);
+  const uint32_t heads = __ballot_sync(0xffffffffu, head);
+  if (head) {
+    const uint32_t after = heads & ~((2u << lane) - 1u);
+    const int end = after ? __ffs(after) - 1 : __popc(lives);
+    atomicAdd(&T.gcell[cell], end - lane);
   }
+  if (lane == 0) T.gorder[0][g] = __float_as_int(v);
+}
+
+// The buckets of this block's kTopoThreads / 4 groups, four threads a group.
+__device__ __forceinline__ void group_buckets(const TreeDev& T, int64_t block) {
+  const int64_t g = (block * kTopoBlock + threadIdx.x) >> 2;
+  const int N = 1 << T.cell_level;
+  float cnt = 0.f;
+  if (g < T.ngroups) {
+    const int64_t k = min(g * kGroup + 4 + 8 * (threadIdx.x & 3), T.n - 1);
+    const float4 p = T.pA[k];
+    const float x[3] = {p.x, p.y, p.z};
+    int c0[3], c1[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int f = (int)(x[c] * (float)N + 0.5f);  // the nearest face: the cells on both sides of it
+      c0[c] = (f + N - 1) & (N - 1);
+      c1[c] = f & (N - 1);
+    }
+    int s = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      s += T.gcell[((i & 4 ? c1[0] : c0[0]) * N + (i & 2 ? c1[1] : c0[1])) * N + (i & 1 ? c1[2] : c0[2])];
+    cnt = (float)s;
+  }
+  cnt += __shfl_xor_sync(0xffffffffu, cnt, 1);
+  cnt += __shfl_xor_sync(0xffffffffu, cnt, 2);
+  if (g < T.ngroups && (threadIdx.x & 3) == 0) {
+    const float v = __int_as_float(T.gorder[0][g]) * (float)T.ngroups;
+    const float n2 = 2.0f * __log2f(cnt);  // half octaves
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      const float w2 = o ? n2 : n2 + 0.5f * __log2f(v);
+      const int bucket = (int)fminf(fmaxf(96.0f - w2, 0.0f), (float)(kBuckets - 1));
+      T.gbucket[o][g] = (unsigned char)bucket;
+      atomicAdd(&T.gtile[o][(g / kOrderTile) * kBuckets + bucket], 1);
+    }
+  }
+}
+
+// Order o of one tile's groups, kOrderTile threads.
+__device__ __forceinline__ void group_places(const TreeDev& T, int64_t tile, int o) {
+  __shared__ int s_at[kOrderTile / 32][kBuckets];
+  __shared__ int s_base[kBuckets];
+  __shared__ int s_part[2][kOrderTile / kBuckets][kBuckets];  // all tiles, the tiles before this one
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  {
+    const int b = threadIdx.x % kBuckets, q = threadIdx.x / kBuckets;
+    int all = 0, before = 0;
+    for (int64_t t = q; t < T.ntiles; t += kOrderTile / kBuckets) {
+      const int c = T.gtile[o][t * kBuckets + b];
+      all += c;
+      if (t < tile) before += c;
+    }
+    s_part[0][q][b] = all;
+    s_part[1][q][b] = before;
+#pragma unroll
+    for (int i = lane; i < kBuckets; i += 32) s_at[w][i] = 0;
+  }
+  __syncthreads();
+  const int64_t g = tile * kOrderTile + threadIdx.x;
+  const int bucket = g < T.ngroups ? T.gbucket[o][g] : -1;
+  const uint32_t peers = __match_any_sync(0xffffffffu, bucket);
+  if (bucket >= 0 && lane == __ffs(peers) - 1) s_at[w][bucket] = __popc(peers);
+  if (w == 0) {  // exclusive scan of the buckets' totals, 4 a lane
+    int tot[kBuckets / 32], sum = 0;
+#pragma unroll
+    for (int i = 0; i < kBuckets / 32; ++i) {
+      tot[i] = sum;
+      for (int q = 0; q < kOrderTile / kBuckets; ++q) sum += s_part[0][q][lane * (kBuckets / 32) + i];
+    }
+    int x = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, d);
+      if (lane >= d) x += y;
+    }
+#pragma unroll
+    for (int i = 0; i < kBuckets / 32; ++i) s_base[lane * (kBuckets / 32) + i] = x - sum + tot[i];
+  }
+  __syncthreads();
+  if (threadIdx.x < kBuckets) {
+    int at = s_base[threadIdx.x];
+    for (int q = 0; q < kOrderTile / kBuckets; ++q) at += s_part[1][q][threadIdx.x];
+    for (int i = 0; i < kOrderTile / 32; ++i) {
+      const int c = s_at[i][threadIdx.x];
+      s_at[i][threadIdx.x] = at;
+      at += c;
+    }
+  }
+  __syncthreads();
+  if (bucket >= 0) T.gorder[o][s_at[w][bucket] + __popc(peers & ((1u << lane) - 1u))] = (int32_t)g;
 }
 
 __global__ void k_permute(BuildArgs A, BoxScale B) {
@@ -71,7 +188,7 @@ __global__ void k_permute(BuildArgs A, BoxScale B) {
         T.x64[3 * k + c] = w[c];
       }
     }
-    if (T.ngroups <= kOrderedGroups) group_bucket(T, k0 / kGroup, live, hi);
+    group_cells(T, k0 / kGroup, live, hi);
     if (!live) continue;
     const double m = A.mass[i];
     const double eps = A.eps ? A.eps[i] : A.eps_scalar;
@@ -129,10 +246,15 @@ __device__ __forceinline__ void node_levels(const uint64_t* __restrict__ keys, i
   deep = min(deep, kMaxLevel - 1);
 }
 
-// Nodes of each level that start in this block's keys.
+// Nodes of each level that start in this block's keys.  The blocks after those
+// of the keys find the groups' buckets.
 __global__ void __launch_bounds__(kTopoThreads) k_count(TreeDev T, const uint64_t* __restrict__ keys, int leaf_size) {
   __shared__ signed char s_far[kTopoThreads + kMaxLeaf];
   __shared__ int s_cnt[kLevels];
+  if (blockIdx.x >= T.nblk) {
+    group_buckets(T, blockIdx.x - T.nblk);
+    return;
+  }
   if (blockIdx.x == 0 && threadIdx.x == 0) T.sb->magic = kMagicTree;
   if (threadIdx.x < kLevels) s_cnt[threadIdx.x] = 0;
   int lo, hi, deep;
@@ -143,28 +265,12 @@ __global__ void __launch_bounds__(kTopoThreads) k_count(TreeDev T, const uint64_
 }
 
 // One block per level: exclusive scan of its counts over the blocks, in
-// place, and the level's total.  The blocks after those write the walks' order
-// of the groups, bucket by bucket (within one in the order their warps get
-// there; no result depends on it).
+// place, and the level's total.  The blocks after those write the walks' orders
+// of the groups, one tile in one order each.
 __global__ void __launch_bounds__(1024) k_scan(TreeDev T) {
   __shared__ int s_w[32];
   if (blockIdx.x >= kLevels) {
-    __shared__ int s_base[kBuckets];
-    if (threadIdx.x < kBuckets) {
-      int b = 0;
-      for (int i = 0; i < (int)threadIdx.x; ++i) b += T.gcount[i];
-      s_base[threadIdx.x] = b;
-    }
-    __syncthreads();
-    const int64_t g = (int64_t)(blockIdx.x - kLevels) * 1024 + threadIdx.x;
-    const int bucket = g < T.ngroups ? T.gbucket[g] : kBuckets;
-    const uint32_t peers = __match_any_sync(0xffffffffu, bucket);
-    const int first = __ffs(peers) - 1;
-    const int lane = threadIdx.x & 31;
-    int at = 0;
-    if (lane == first && bucket < kBuckets) at = atomicAdd(&T.gcount[kBuckets + bucket], __popc(peers));
-    at = __shfl_sync(0xffffffffu, at, first) + __popc(peers & ((1u << lane) - 1u));
-    if (bucket < kBuckets) T.gorder[s_base[bucket] + at] = (int32_t)g;
+    group_places(T, (blockIdx.x - kLevels) >> 1, (blockIdx.x - kLevels) & 1);
     return;
   }
   int* row = T.blk + blockIdx.x * T.nblk;
@@ -457,9 +563,9 @@ cudaError_t launch_tree_build(const BuildArgs& A, cudaStream_t s) {
   if (grid > grid_cap(32)) grid = grid_cap(32);
   const BoxScale B = box_scale(A.L);
   k_permute<<<(unsigned)grid, 256, 0, s>>>(A, B);
-  k_count<<<(unsigned)T.nblk, kTopoThreads, 0, s>>>(T, A.keys, A.leaf_size);
-  const int64_t oblocks = T.ngroups <= kOrderedGroups ? (T.ngroups + 1023) / 1024 : 0;
-  k_scan<<<(unsigned)(kLevels + oblocks), 1024, 0, s>>>(T);
+  const int64_t gblocks = (4 * T.ngroups + kTopoThreads - 1) / kTopoThreads;
+  k_count<<<(unsigned)(T.nblk + gblocks), kTopoThreads, 0, s>>>(T, A.keys, A.leaf_size);
+  k_scan<<<(unsigned)(kLevels + 2 * T.ntiles), kOrderTile, 0, s>>>(T);
   k_fill<<<(unsigned)T.nblk, kTopoThreads, 0, s>>>(T, A.keys, A.leaf_size);
   // the node counts live on the device: grids are sized for the particles
   int64_t lgrid = (T.n / 2 + 255) / 256;

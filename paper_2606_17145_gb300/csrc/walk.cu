@@ -425,6 +425,7 @@ template <bool ADJ, bool F64, bool FUSED = false>
 struct LaneFP {
   static_assert(!FUSED || (ADJ && !F64), "the fused walk is the FP32 adjoint plus the forward sums");
   static constexpr int kListSize = F64 ? kList : kSub * kGroup;
+  static constexpr int kOrder = F64 ? 1 : 0;  // of T.gorder
   // per-warp data that lives through the whole walk
   struct Smem {
     float4 tA[kGroup];    // targets: hi part, h^2
@@ -1228,7 +1229,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_walk(WalkArgs A) {
   const int64_t gi = A.g_begin + (v >> A.split);
   if (gi >= A.g_end) return;
   const bool usable = T.sb->status == 0 && T.sb->magic == kMagicTree;
-  const int64_t g = A.ordered && usable ? T.gorder[gi] : gi;
+  const int64_t g = A.ordered && usable ? T.gorder[Lane::kOrder][gi] : gi;
   const bool mine = (lane >> (5 - A.split)) == (int)(v & ((1 << A.split) - 1));
   if (!usable) {
     // a failed or missing tree: flag it and give every output of this
@@ -1517,7 +1518,7 @@ static int walk_split(int64_t n_groups) { return n_groups <= 1024 ? 2 : n_groups
 
 cudaError_t launch_walk(WalkArgs A, int prec, bool adjoint, cudaStream_t s, bool fused) {
   A.split = walk_split(A.T.ngroups);
-  A.ordered = A.g_begin == 0 && A.g_end == A.T.ngroups && A.T.ngroups <= kOrderedGroups;
+  A.ordered = A.g_begin == 0 && A.g_end == A.T.ngroups;
   const int64_t blocks = (((A.g_end - A.g_begin) << A.split) + kWarpsPerBlock - 1) / kWarpsPerBlock;
   if (blocks <= 0) return cudaSuccess;
   if (fused) k_walk<LaneFused><<<(unsigned)blocks, kWarpsPerBlock * 32, 0, s>>>(A);

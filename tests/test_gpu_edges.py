@@ -59,6 +59,34 @@ def test_sort_tree_and_walks(orc, n, clumps):
         assert grad_scaled_err(dm.cpu().numpy()[s], gm, sm) < GRAD_TOL
 
 
+@pytest.mark.parametrize("n", [31, 1024 * 32 - 1, 3 * 1024 * 32 + 1])
+def test_orders_hold_every_group(n):
+    """The walks' orders of the groups (tiles of 1024 groups, buckets of
+    estimated work): a full walk leaves no target out in either precision and
+    agrees with walks over ranges, which go in tree order; SPH likewise."""
+    dev = device()
+    m = og()
+    rng = np.random.default_rng(n)
+    pos = rng.random((n, 3))
+    pos[: n // 2] = np.mod(0.98 + 0.01 * rng.standard_normal((n // 2, 3)), 1.0)  # a clump across the box's corner
+    p = torch.tensor(pos, dtype=torch.float64, device=dev)
+    keys, order = m.keys_sort(p, 1.0)
+    tree = m.tree_build(keys, order, p, torch.ones(n, dtype=torch.float64, device=dev), 0.3 * n ** (-1 / 3), 1.0)
+    r_s = min(0.1, 0.625 * n ** (-1 / 3))
+    g = int(tree.header.n_groups)
+    for prec in ("fp32", "fp64"):
+        full = torch.full((n, 3), float("nan"), dtype=torch.float32 if prec == "fp32" else torch.float64, device=dev)
+        part = full.clone()
+        m.shortrange_accel(tree, r_s, 0.5, prec=prec, out=full)
+        for a, b in ((0, g // 2), (g // 2, g)):
+            if b > a:
+                m.shortrange_accel(tree, r_s, 0.5, prec=prec, out=part, groups=(a, b))
+        assert torch.isfinite(full).all() and torch.equal(full, part)
+    if n > 100:
+        h, rho, ngb = m.sph_density(tree, 32)
+        assert (h > 0).all() and (rho > 0).all() and (ngb > 0).all()
+
+
 @pytest.mark.parametrize("n,n_ngb", [(97, 16), (129, 16), (1024 * 32, 32), (1024 * 32 + 5, 100)])
 def test_sph_sizes(n, n_ngb):
     """SPH at few particles, one against four warps a group, more neighbours
