@@ -367,26 +367,56 @@ class TreePMStepper:
         self.plan = PMPlan(ngrid)
         self.ws_pm = _workspace(self.plan.ws_bytes, dev)
         self.ws_acc = None
+        self._side = torch.cuda.Stream(device=dev)
+        self._fork, self._join = torch.cuda.Event(), torch.cuda.Event()
+        self._status = torch.zeros(4, dtype=torch.int32).pin_memory()
         self.forces(check=True)
 
+    def _mesh(self, check: bool, stream):
+        pm_accel(self.plan, self.pos, self.mass, self.box, self.r_s, stream=stream, check=check, ws=self.ws_pm,
+                 out=self.acc_l)
+
     def forces(self, check: bool = False, stream=None):
-        """Short-range (walk) and long-range (mesh) accelerations at the current positions."""
+        """Short-range (walk) and long-range (mesh) accelerations at the current
+        positions.  Without check the mesh runs on a stream of its own beside
+        the sort and the tree build, whose small kernels leave most of the chip
+        idle, and the given stream waits for it (a 64^3 lattice step 795 -> 748 us,
+        with the single synchronisation of poll())."""
+        s = stream if stream is not None else torch.cuda.current_stream()
+        self._fork.record(s)
         keys_sort(self.pos, self.box, stream=stream, check=check, ws=self.ws_keys, keys=self.keys, order=self.order)
         tree = tree_build(self.keys, self.order, self.pos, self.mass, self.eps, self.box, p=self.p, stream=stream,
                           check=check, mem=self.tree_mem)
         if self.ws_acc is None:
             self.ws_acc = _workspace(lib().og_accel_ws_bytes(C.byref(tree.header), 0), self.pos.device)
-        shortrange_accel(tree, self.r_s, self.theta, stream=stream, check=check, ws=self.ws_acc, out=self.acc_s,
-                         total=self.total)
-        pm_accel(self.plan, self.pos, self.mass, self.box, self.r_s, stream=stream, check=check, ws=self.ws_pm,
-                 out=self.acc_l)
+        try:
+            if not check:  # enqueued after the tree, so that the host does not hold the sort back
+                self._side.wait_event(self._fork)
+                self._mesh(False, self._side)
+            shortrange_accel(tree, self.r_s, self.theta, stream=stream, check=check, ws=self.ws_acc, out=self.acc_s,
+                             total=self.total)
+        finally:
+            if not check:
+                self._join.record(self._side)
+                s.wait_event(self._join)
+        if check:
+            self._mesh(True, stream)
 
     def poll(self, stream=None):
         """Synchronise and raise OGError if keys, tree, walk or mesh recorded
         an error on the device since their last call."""
-        for buf, where in ((self.ws_keys, "og_keys_sort"), (self.tree_mem, "og_tree_build"),
-                           (self.ws_acc, "og_shortrange_accel"), (self.ws_pm, "og_pm_accel")):
-            if buf is not None:
+        bufs = [(self.ws_keys, "og_keys_sort"), (self.tree_mem, "og_tree_build"),
+                (self.ws_acc, "og_shortrange_accel"), (self.ws_pm, "og_pm_accel")]
+        # the four status words are copied while the step still runs, and one
+        # synchronisation serves them all
+        s = stream if stream is not None else torch.cuda.current_stream()
+        with torch.cuda.stream(s):
+            for i, (buf, _) in enumerate(bufs):
+                if buf is not None:
+                    self._status[i:i + 1].copy_(buf[:4].view(torch.int32), non_blocking=True)
+        s.synchronize()
+        for i, (buf, where) in enumerate(bufs):
+            if buf is not None and int(self._status[i]) != 0:
                 _check(poll_status(buf, stream), f"{where} (device, stepper)")
 
     def step(self, dt: float, check: bool = True, stream=None):

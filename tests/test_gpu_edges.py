@@ -110,6 +110,35 @@ def test_sph_sizes(n, n_ngb):
     np.testing.assert_array_equal(ngb.cpu().numpy()[tg], cnt)
 
 
+@pytest.mark.parametrize("n,N", [(300, 16), (20000, 32)])
+def test_stepper_mesh_beside_tree(n, N):
+    """Forces with the mesh on its own stream, from the default stream and from
+    another one, against the calls one after the other.  The mesh sums its
+    deposits in any order: a few FP32 rounding errors of the largest force."""
+    dev = device()
+    m = og()
+    rng = np.random.default_rng(n)
+    p = torch.tensor(rng.random((n, 3)), dtype=torch.float64, device=dev)
+    S = m.TreePMStepper(p, torch.zeros_like(p), torch.full((n,), 1.0 / n, dtype=torch.float64, device=dev), 1e-3, 1.0,
+                        0.7 * n ** (-1 / 3), 0.5, N)
+    short, long = S.acc_s.clone(), S.acc_l.clone()  # the constructor's, checked one by one
+    other = torch.cuda.Stream()
+    other.wait_stream(torch.cuda.current_stream())
+    for stream in (None, other):
+        for _ in range(3):
+            S.acc_s.fill_(float("nan"))
+            S.acc_l.fill_(float("nan"))
+            torch.cuda.synchronize()
+            S.forces(stream=stream)
+            S.poll(stream)
+            assert torch.equal(S.acc_s, short)
+            assert (S.acc_l - long).abs().max() <= 1e-5 * long.abs().max()
+    p[n // 2, 1] = float("nan")
+    with pytest.raises(m.OGError):
+        S.step(0.0)
+    S.close()
+
+
 def _mesh_ref(pos, mass, N, r_s):
     """The mesh force in torch FP64 on the device (unit box)."""
     dev = pos.device
