@@ -110,6 +110,25 @@ def test_sph_sizes(n, n_ngb):
     np.testing.assert_array_equal(ngb.cpu().numpy()[tg], cnt)
 
 
+@pytest.mark.parametrize("groups", [24575, 24576, 24577])
+def test_walk_of_many_groups(groups):
+    """Either side of the group count from which the forward walk runs in
+    blocks of one warp, the last group ragged: the sums of the walk in both
+    directions at once, which goes in blocks of two at any size."""
+    dev = device()
+    m = og()
+    n = 32 * groups - 31
+    p = torch.rand((n, 3), dtype=torch.float64, device=dev, generator=torch.Generator(dev).manual_seed(groups))
+    p[: n // 8] = (0.5 + 0.05 * (p[: n // 8] - 0.5)).contiguous()
+    keys, order = m.keys_sort(p, 1.0)
+    tree = m.tree_build(keys, order, p, torch.ones(n, dtype=torch.float64, device=dev), 0.05 * n ** (-1 / 3), 1.0)
+    r_s = 0.625 * n ** (-1 / 3)
+    acc, total, counts = m.shortrange_accel(tree, r_s, 0.5, counts=True)
+    both, total2, counts2, _, _ = m.shortrange_accel_adjoint(tree, r_s, 0.5, torch.ones_like(acc), counts=True)
+    assert torch.isfinite(acc).all() and torch.equal(acc, both)
+    assert torch.equal(counts, counts2) and int(total.item()) == int(total2.item()) == int(counts.sum().item())
+
+
 @pytest.mark.parametrize("n,N", [(300, 16), (20000, 32)])
 def test_stepper_mesh_beside_tree(n, N):
     """Forces with the mesh on its own stream, from the default stream and from
