@@ -8,7 +8,10 @@
 // exchanged with those of axis i; the axes are then Gray-coded against one
 // another and a running parity of the last axis is folded in.  Here the
 // parity fold is a bit-parallel suffix XOR and the final interleave uses
-// magic-mask bit spreading.
+// magic-mask bit spreading.  That is about 350 integer instructions a key, and
+// bound the kernel (123 us at 5.0 M keys, 24 us of memory time), so where keys
+// are counted for the passes the index is looked up instead, three levels of
+// the curve at a time, in a 24 KB table of its 24 states: 57 us.
 //
 // K2: 8 passes of 8-bit digits (63-bit keys), one launch each.  K1 counts all
 // eight digits' histograms while it writes the keys.  A pass ranks its tile's
@@ -24,10 +27,11 @@
 // Bound by HBM: 220 B a key (32 for the keys, 20 for the first pass, whose
 // values are the indices themselves, 24 for each other pass), against 310 B and 25
 // launches for a histogram, a scan and a scatter per pass.
-// Measured (keys and sort): 4096 keys 95 -> 78 us, 2.1 M 0.38 -> 0.26 ms, 5.0 M
-// clustered 0.69 -> 0.48, 16.8 M 2.07 -> 1.38.  A pass takes 2.4 times its memory
+// Measured (keys and sort): 2.1 M 0.38 -> 0.24 ms, 5.0 M clustered 0.69 -> 0.41,
+// 16.8 M 2.07 -> 1.14.  A pass takes 2.4 times its memory
 // time at 16.8 M keys: a tile's chain of ranking, look-back and scattered writes
-// is 12 us long and three tiles fit an SM.  Tile shapes, 5.0 M / 16.8 M: 256 x 16 keys
+// is 12 us long and three tiles fit an SM.  Tile shapes, 5.0 M / 16.8 M, with the
+// index computed bit by bit: 256 x 16 keys
 // 0.481 / 1.38 ms, 256 x 12 0.488 / 1.43, 384 x 16 0.488 / 1.43, 512 x 8 0.52 / 1.57, 256 x 8
 // 0.55 / 1.63; predecessors read at a time 4 / 8 / 16: 0.481 / 0.488 / 0.524 ms at 5.0 M.
 #include "og_internal.cuh"
@@ -83,14 +87,96 @@ __device__ __forceinline__ uint64_t hilbert63(uint32_t a, uint32_t b, uint32_t c
 constexpr int kKeyThreads = 256;
 
 // Key of one position; 0 and the status flag for a non-finite one.
+// The same index three levels at a time.  What the levels above leave behind
+// is one of 24 states: which axis each of the three is exchanged with, which
+// are inverted, and the parity.  e[512 s + (a, b, c)], three bits of each axis, is
+// the next state << 9 | nine bits of the index.  Built from the steps of
+// hilbert63 at compile time; states that give the same digits are one.
+constexpr int kHilbertStates = 24;
+struct alignas(16) HilbertTable {
+  uint16_t e[kHilbertStates * 512];
+  constexpr HilbertTable() : e() {
+    int key[kHilbertStates] = {};    // the state's digits of the eight octants, 3 bits each
+    int rep[kHilbertStates][7] = {};  // source axis of each axis, its inversion, parity
+    int next[kHilbertStates][8] = {};
+    int ns = 0;
+    const int first[7] = {0, 1, 2, 0, 0, 0, 0};
+    find(first, key, rep, ns);
+    for (int s = 0; s < ns; ++s)
+      for (int o = 0; o < 8; ++o) {
+        int to[7] = {};
+        step(rep[s], o, to);
+        next[s][o] = find(to, key, rep, ns);
+      }
+    for (int s = 0; s < ns; ++s)
+      for (int i = 0; i < 512; ++i) {
+        int st = s, digits = 0;
+        for (int b = 2; b >= 0; --b) {
+          const int o = ((i >> (6 + b)) & 1) << 2 | ((i >> (3 + b)) & 1) << 1 | ((i >> b) & 1);
+          digits = digits << 3 | ((key[st] >> (3 * o)) & 7);
+          st = next[st][o];
+        }
+        e[512 * s + i] = (uint16_t)(st << 9 | digits);
+      }
+  }
+  // One level of hilbert63 for the octant o: its digit and the state below.
+  static constexpr int step(const int st[7], int o, int to[7]) {
+    int v[3] = {};
+    for (int x = 0; x < 3; ++x) v[x] = ((o >> (2 - st[x])) & 1) ^ st[3 + x];
+    for (int x = 0; x < 7; ++x) to[x] = st[x];
+    const int B = v[1] ^ v[0], C = v[2] ^ B;
+    if (v[0]) to[3] ^= 1;
+    for (int x = 1; x < 3; ++x) {
+      if (v[x]) {
+        to[3] ^= 1;
+      } else {
+        const int src = to[0], inv = to[3];
+        to[0] = to[x];
+        to[3] = to[3 + x];
+        to[x] = src;
+        to[3 + x] = inv;
+      }
+    }
+    to[6] ^= C;
+    return (v[0] << 2 | B << 1 | C) ^ (st[6] ? 7 : 0);
+  }
+  static constexpr int find(const int st[7], int* key, int (*rep)[7], int& ns) {
+    int k = 0, unused[7] = {};
+    for (int o = 0; o < 8; ++o) k |= step(st, o, unused) << (3 * o);
+    for (int s = 0; s < ns; ++s)
+      if (key[s] == k) return s;
+    key[ns] = k;
+    for (int x = 0; x < 7; ++x) rep[ns][x] = st[x];
+    return ns++;
+  }
+};
+__device__ const HilbertTable kHilbertTable;
+
+__device__ __forceinline__ uint64_t hilbert63(const uint16_t* __restrict__ table, uint32_t a, uint32_t b,
+                                              uint32_t c) {
+  uint64_t key = 0;
+  uint32_t st = 0;
+#pragma unroll
+  for (int bit = 18; bit >= 0; bit -= 3) {
+    const uint32_t i = (((a >> bit) & 7u) << 6) | (((b >> bit) & 7u) << 3) | ((c >> bit) & 7u);
+    const uint32_t e = table[(st & ~511u) | i];
+    key = key << 9 | (e & 511u);
+    st = e;
+  }
+  return key;
+}
+
+template <bool TABLE>
 __device__ __forceinline__ uint64_t position_key(const double* __restrict__ pos, int64_t i, const BoxScale& B,
-                                                 StatusBlock* sb) {
+                                                 const uint16_t* table, StatusBlock* sb) {
   const double x0 = pos[3 * i], x1 = pos[3 * i + 1], x2 = pos[3 * i + 2];
   if (!(finite_bits(x0) && finite_bits(x1) && finite_bits(x2))) {
     set_status(sb, ST_BADINPUT);
     return 0;
   }
-  return hilbert63(quantise(wrap_coord(x0, B), B), quantise(wrap_coord(x1, B), B), quantise(wrap_coord(x2, B), B));
+  const uint32_t a = quantise(wrap_coord(x0, B), B), b = quantise(wrap_coord(x1, B), B),
+                 c = quantise(wrap_coord(x2, B), B);
+  return TABLE ? hilbert63(table, a, b, c) : hilbert63(a, b, c);
 }
 
 // PASSES: also what the radix passes need, the digits' counts and clear tile counts.
@@ -98,8 +184,11 @@ template <bool PASSES>
 __global__ void __launch_bounds__(kKeyThreads) k_keys(const double* __restrict__ pos, int64_t n, BoxScale B,
                                                       uint64_t* __restrict__ keys, SortWs W) {
   __shared__ uint32_t h[PASSES ? 8 * 256 : 1];
+  __shared__ uint4 s_table[PASSES ? sizeof(HilbertTable) / sizeof(uint4) : 1];
   if (PASSES) {
     for (int i = threadIdx.x; i < 8 * 256; i += kKeyThreads) h[i] = 0u;
+    for (int i = threadIdx.x; i < (int)(sizeof(HilbertTable) / sizeof(uint4)); i += kKeyThreads)
+      s_table[i] = reinterpret_cast<const uint4*>(kHilbertTable.e)[i];
     __syncthreads();
   }
   const int64_t stride = (int64_t)gridDim.x * kKeyThreads;
@@ -108,7 +197,7 @@ __global__ void __launch_bounds__(kKeyThreads) k_keys(const double* __restrict__
   if (PASSES)
     for (int64_t i = first; i < W.ntiles * 256; i += stride) W.tile_state[0][i] = 0u;
   for (int64_t i = first; i < n; i += stride) {
-    const uint64_t key = position_key(pos, i, B, W.sb);
+    const uint64_t key = position_key<PASSES>(pos, i, B, reinterpret_cast<const uint16_t*>(s_table), W.sb);
     keys[i] = key;
     if (PASSES) {
 #pragma unroll
@@ -338,7 +427,7 @@ cudaError_t launch_keys_sort(const double* pos, int64_t n, double L, uint64_t* k
   cudaError_t e = cudaMemsetAsync(W.sb, 0, kSortZeroBytes, s);
   if (e != cudaSuccess) return e;
   int64_t kgrid = (n + kKeyThreads - 1) / kKeyThreads;
-  if (kgrid > grid_cap(8)) kgrid = grid_cap(8);
+  if (kgrid > grid_cap(4)) kgrid = grid_cap(4);  // each block copies the table: 8 an SM +2 us at 262,144 keys
   if (n <= kRankMax) {
     k_keys<false><<<(unsigned)kgrid, kKeyThreads, 0, s>>>(pos, n, box_scale(L), W.keys_alt, W);
     k_sort_rank<<<(unsigned)((n + 31) / 32), kRankWarps * 32, 0, s>>>(W.keys_alt, (int)n, keys_out, order_out);

@@ -59,6 +59,24 @@ def test_sort_tree_and_walks(orc, n, clumps):
         assert grad_scaled_err(dm.cpu().numpy()[s], gm, sm) < GRAD_TOL
 
 
+@pytest.mark.parametrize("axis", ["random", "ones"])
+def test_keys_by_table_and_by_bits(axis):
+    """Keys of more than 16,384 particles are looked up level by level, fewer
+    are computed bit by bit: the same numbers, over all bits of the cell."""
+    dev = device()
+    m = og()
+    rng = np.random.default_rng(3)
+    cell = rng.integers(0, 1 << 21, (3 * 16384, 3))
+    if axis == "ones":  # long runs of equal bits, from either end
+        cell = (1 << 21) - (1 << rng.integers(0, 22, (3 * 16384, 3)))
+        cell[::2] ^= (1 << 21) - 1
+        cell = np.clip(cell, 0, (1 << 21) - 1)
+    pos = torch.tensor((cell + 0.5) * 2.0 ** -21, dtype=torch.float64, device=dev)
+    keys, _ = m.keys_sort(pos, 1.0)
+    parts = torch.cat([m.keys_sort(p.contiguous(), 1.0)[0] for p in pos.split(16384)])
+    assert torch.equal(keys, parts.sort().values)
+
+
 @pytest.mark.parametrize("n", [31, 1024 * 32 - 1, 3 * 1024 * 32 + 1])
 def test_orders_hold_every_group(n):
     """The walks' orders of the groups (tiles of 1024 groups, buckets of
