@@ -33,7 +33,8 @@
 // is 12 us long and three tiles fit an SM.  Tile shapes, 5.0 M / 16.8 M, with the
 // index computed bit by bit: 256 x 16 keys
 // 0.481 / 1.38 ms, 256 x 12 0.488 / 1.43, 384 x 16 0.488 / 1.43, 512 x 8 0.52 / 1.57, 256 x 8
-// 0.55 / 1.63; predecessors read at a time 4 / 8 / 16: 0.481 / 0.488 / 0.524 ms at 5.0 M.
+// 0.55 / 1.63; predecessors read at a time 4 / 8 / 16: 0.481 / 0.488 / 0.524 ms at 5.0 M.  Up to
+// 262,144 keys a tile is 256 x 4 (sort_items).
 #include "og_internal.cuh"
 
 namespace og {
@@ -221,42 +222,44 @@ constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kStateAhead = 4;
 
 // Shared memory of a pass (dynamic: above the static limit).
+template <int ITEMS>
 struct SortSmem {
-  uint64_t keys[kSortTile];
-  int32_t vals[kSortTile];
+  uint64_t keys[kSortThreads * ITEMS];
+  int32_t vals[kSortThreads * ITEMS];
   uint32_t wcnt[kSortWarps][256];
   uint32_t base[256];  // where the tile's first key of each digit goes, less its place in the tile
   unsigned long long scan[8];
   uint32_t tile;
 };
 
-template <bool FIRST>
-__global__ void __launch_bounds__(kSortThreads, 3)
+template <bool FIRST, int ITEMS>
+__global__ void __launch_bounds__(kSortThreads, ITEMS == 16 ? 3 : 6)
     k_sort_pass(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin, int64_t n, int pass, SortWs W,
                 uint64_t* __restrict__ kout, int32_t* __restrict__ vout) {
   extern __shared__ __align__(16) unsigned char s_raw[];
-  SortSmem& S = *reinterpret_cast<SortSmem*>(s_raw);
+  constexpr int kTile = kSortThreads * ITEMS;
+  SortSmem<ITEMS>& S = *reinterpret_cast<SortSmem<ITEMS>*>(s_raw);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int shift = 8 * pass;
   if (threadIdx.x == 0) S.tile = (uint32_t)atomicAdd(&W.sb->pad[pass], 1);
   for (int i = threadIdx.x; i < kSortWarps * 256; i += kSortThreads) (&S.wcnt[0][0])[i] = 0u;
   __syncthreads();
   const int64_t tile = S.tile;
-  const int64_t base = tile * kSortTile;
-  const int tile_n = (int)((n - base) < kSortTile ? (n - base) : kSortTile);
-  const int l0 = w * 32 * kSortItems + lane;  // this lane's first key of the tile
+  const int64_t base = tile * kTile;
+  const int tile_n = (int)((n - base) < kTile ? (n - base) : kTile);
+  const int l0 = w * 32 * ITEMS + lane;  // this lane's first key of the tile
 
-  uint64_t key[kSortItems];
-  uint32_t place[kSortItems];
+  uint64_t key[ITEMS];
+  uint32_t place[ITEMS];
   const uint32_t lt = (1u << lane) - 1u;
   // padding slots lie behind every key of the tile: the largest digit keeps them last
 #pragma unroll
-  for (int k = 0; k < kSortItems; ++k) key[k] = l0 + 32 * k < tile_n ? kin[base + l0 + 32 * k] : ~0ull;
+  for (int k = 0; k < ITEMS; ++k) key[k] = l0 + 32 * k < tile_n ? kin[base + l0 + 32 * k] : ~0ull;
   // rank among the warp's keys of the same digit: the first of the 32 lanes
   // with the digit takes their number from the warp's counter; the rounds'
   // atomics go out in order and are not waited for between rounds
 #pragma unroll
-  for (int k = 0; k < kSortItems; ++k) {
+  for (int k = 0; k < ITEMS; ++k) {
     const uint32_t d = (uint32_t)((key[k] >> shift) & 255u);
     uint32_t peers = 0xffffffffu;
 #pragma unroll
@@ -286,7 +289,7 @@ __global__ void __launch_bounds__(kSortThreads, 3)
       cnt += c;
     }
     own = ((unsigned long long)cnt << 32) | all;
-    if (d == 255) cnt -= (uint32_t)(kSortTile - tile_n);  // less the padding
+    if (d == 255) cnt -= (uint32_t)(kTile - tile_n);  // less the padding
     __stcg(&state[tile * 256 + d], tile == 0 ? (kStateSum | cnt) : cnt + 1u);
     if (pass < 7) W.tile_state[(pass + 1) & 1][tile * 256 + d] = 0u;  // the next pass's
     x = own;
@@ -309,14 +312,14 @@ __global__ void __launch_bounds__(kSortThreads, 3)
   }
   __syncthreads();
   // the tile in digit order
-  int32_t val[kSortItems];
+  int32_t val[ITEMS];
 #pragma unroll
-  for (int k = 0; k < kSortItems; ++k) {
+  for (int k = 0; k < ITEMS; ++k) {
     place[k] += S.wcnt[w][(key[k] >> shift) & 255u];
     S.keys[place[k]] = key[k];
   }
 #pragma unroll
-  for (int k = 0; k < kSortItems; ++k)
+  for (int k = 0; k < ITEMS; ++k)
     val[k] = FIRST ? (int32_t)(base + l0 + 32 * k) : l0 + 32 * k < tile_n ? vin[base + l0 + 32 * k] : 0;
   // keys of this digit in the tiles before
   if (d < 256) {
@@ -350,16 +353,16 @@ __global__ void __launch_bounds__(kSortThreads, 3)
     S.base[d] = gbase + sum - tstart;
   }
 #pragma unroll
-  for (int k = 0; k < kSortItems; ++k) S.vals[place[k]] = val[k];
+  for (int k = 0; k < ITEMS; ++k) S.vals[place[k]] = val[k];
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < kSortItems; ++k) key[k] = S.keys[k * kSortThreads + threadIdx.x];
+  for (int k = 0; k < ITEMS; ++k) key[k] = S.keys[k * kSortThreads + threadIdx.x];
 #pragma unroll
-  for (int k = 0; k < kSortItems; ++k) val[k] = S.vals[k * kSortThreads + threadIdx.x];
+  for (int k = 0; k < ITEMS; ++k) val[k] = S.vals[k * kSortThreads + threadIdx.x];
 #pragma unroll
-  for (int k = 0; k < kSortItems; ++k) place[k] = S.base[(key[k] >> shift) & 255u] + (uint32_t)(k * kSortThreads + threadIdx.x);
+  for (int k = 0; k < ITEMS; ++k) place[k] = S.base[(key[k] >> shift) & 255u] + (uint32_t)(k * kSortThreads + threadIdx.x);
 #pragma unroll
-  for (int k = 0; k < kSortItems; ++k) {
+  for (int k = 0; k < ITEMS; ++k) {
     if (k * kSortThreads + (int)threadIdx.x < tile_n && (int64_t)place[k] < n) {
       kout[place[k]] = key[k];
       vout[place[k]] = val[k];
@@ -421,6 +424,17 @@ __global__ void __launch_bounds__(kRankWarps * 32) k_sort_rank(const uint64_t* _
   }
 }
 
+template <int ITEMS>
+static cudaError_t launch_sort_pass(const uint64_t* kin, const int32_t* vin, int64_t n, int pass, const SortWs& W,
+                                    uint64_t* ko, int32_t* vo, cudaStream_t s) {
+  auto kernel = pass == 0 ? k_sort_pass<true, ITEMS> : k_sort_pass<false, ITEMS>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)sizeof(SortSmem<ITEMS>));
+  if (e != cudaSuccess) return e;
+  kernel<<<(unsigned)W.ntiles, kSortThreads, sizeof(SortSmem<ITEMS>), s>>>(kin, vin, n, pass, W, ko, vo);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_keys_sort(const double* pos, int64_t n, double L, uint64_t* keys_out, int32_t* order_out,
                              const SortWs& W, cudaStream_t s) {
   // status, tile counters and histograms start at zero
@@ -438,13 +452,11 @@ cudaError_t launch_keys_sort(const double* pos, int64_t n, double L, uint64_t* k
   int32_t* vin = order_out;
   uint64_t* ko = W.keys_alt;
   int32_t* vo = W.vals_alt;
-  e = cudaFuncSetAttribute(k_sort_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_sort_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
-  if (e != cudaSuccess) return e;
+  const int items = sort_items(n);
   for (int pass = 0; pass < 8; ++pass) {
-    auto kernel = pass == 0 ? k_sort_pass<true> : k_sort_pass<false>;
-    kernel<<<(unsigned)W.ntiles, kSortThreads, sizeof(SortSmem), s>>>(kin, vin, n, pass, W, ko, vo);
+    e = items == 4 ? launch_sort_pass<4>(kin, vin, n, pass, W, ko, vo, s)
+                   : launch_sort_pass<16>(kin, vin, n, pass, W, ko, vo, s);
+    if (e != cudaSuccess) return e;
     uint64_t* tk = kin; kin = ko; ko = tk;
     int32_t* tv = vin; vin = vo; vo = tv;
   }
@@ -463,11 +475,15 @@ namespace {
 
 constexpr int64_t kNoAllocMaxN = int64_t(1) << 20;
 constexpr size_t noalloc_round(size_t x) { return (x + og::kAlign - 1) / og::kAlign * og::kAlign; }
+// The most tiles of any n up to that: at the last n of either tile size.
+constexpr int64_t kNoAllocTiles = og::sort_tiles(og::kSortFew) > og::sort_tiles(kNoAllocMaxN)
+                                      ? og::sort_tiles(og::kSortFew) : og::sort_tiles(kNoAllocMaxN);
+static_assert(og::kSortFew <= kNoAllocMaxN, "either tile size is reached");
 // Same carving as og::carve_sort: status block, histograms, alternate keys,
 // alternate indices, two passes' tile counts.
 constexpr size_t kNoAllocBytes =
     og::kSortZeroBytes + noalloc_round(sizeof(uint64_t) * kNoAllocMaxN) + noalloc_round(sizeof(int32_t) * kNoAllocMaxN) +
-    2 * noalloc_round(sizeof(uint32_t) * 256 * ((kNoAllocMaxN + og::kSortTile - 1) / og::kSortTile));
+    2 * noalloc_round(sizeof(uint32_t) * 256 * kNoAllocTiles);
 
 // Held by every GPU that loads the library, until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_sort_ws[kNoAllocBytes];

@@ -59,6 +59,16 @@ def test_sort_tree_and_walks(orc, n, clumps):
         assert grad_scaled_err(dm.cpu().numpy()[s], gm, sm) < GRAD_TOL
 
 
+@pytest.mark.parametrize("n", [16385, 17 * 1024 - 1, (1 << 18) - 1, 1 << 18, (1 << 18) + 1])
+def test_sort_tile_sizes(orc, n):
+    """Either side of the key counts at which the tiles of the sort change size."""
+    pos = np.random.default_rng(n).random((n, 3))
+    pos[: n // 4] = pos[0]  # one digit that fills whole tiles
+    keys, order = og().keys_sort(torch.tensor(pos, dtype=torch.float64, device=device()), 1.0)
+    ks, o = orc.sort(orc.keys(pos, 1.0)[0])
+    assert np.array_equal(keys.cpu().numpy().view(np.uint64), ks) and np.array_equal(order.cpu().numpy(), o)
+
+
 @pytest.mark.parametrize("axis", ["random", "ones"])
 def test_keys_by_table_and_by_bits(axis):
     """Keys of more than 16,384 particles are looked up level by level, fewer
