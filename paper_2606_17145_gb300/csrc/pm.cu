@@ -61,6 +61,7 @@ __device__ __forceinline__ void cic_axis(double x, const BoxScale& B, int N, int
   i0 = i;
 }
 
+template <bool EVEN>
 __global__ void k_pm_deposit(const double* __restrict__ pos, const double* __restrict__ mass, int64_t n,
                              BoxScale B, int N, int log2N, float* __restrict__ R, StatusBlock* sb) {
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
@@ -81,7 +82,7 @@ __global__ void k_pm_deposit(const double* __restrict__ pos, const double* __res
     const int ax[2] = {ix, jx}, ay[2] = {iy, jy};
     // two neighbouring nodes per atomic where they are 8-byte aligned (an even
     // lower node and an even row length)
-    const bool pair = (iz & 1) == 0 && (N & 1) == 0;
+    const bool pair = EVEN && (iz & 1) == 0;
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
@@ -371,10 +372,13 @@ __device__ __forceinline__ int pm_wrap(int i, int N) { return i < 0 ? i + N : (i
 // its values are read at fixed offsets where the six do not wrap.  Bound by L1
 // and its latency; 2.1 M lattice particles on 256^3 94 -> 70 us, 16.8 M clustered in
 // random order on 512^3 (whole call) 12.1 -> 8.7 ms (72 loads with an index wrap
-// each before).  Three blocks an SM: 0.283 ms a call, two (96 registers) 0.299, four
-// (spills) 0.293.
-__global__ void __launch_bounds__(256, 3) k_pm_interp(const double* __restrict__ pos, int64_t n, BoxScale B, int N, int log2N, float inv_D,
-                            const float* __restrict__ P, float* __restrict__ acc) {
+// each before).  24 warps an SM: 0.283 ms a call, 16 (96 registers) 0.299, 32 (spills)
+// 0.293; in blocks of 64 threads against 256, whose last wave is coarser: 282.6 ->
+// 281.5 us, 165,376 particles on 85^3 134.1 -> 131.8, 4 M clustered on 200^3 754 -> 744.
+constexpr int kInterpThreads = 64;
+__global__ void __launch_bounds__(kInterpThreads, 12)
+    k_pm_interp(const double* __restrict__ pos, int64_t n, BoxScale B, int N, int log2N, float inv_D,
+                const float* __restrict__ P, float* __restrict__ acc) {
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
     const double x0 = pos[3 * p], x1 = pos[3 * p + 1], x2 = pos[3 * p + 2];
     float a[3] = {0.0f, 0.0f, 0.0f};
@@ -572,7 +576,8 @@ og_status og_pm_accel(og_pm_plan* plan, const double* pos, const double* mass, i
   int log2N = -1;  // N a power of two: its exponent
   for (int e = 0; e < 11; ++e)
     if (N == (1 << e)) log2N = e;
-  og::k_pm_deposit<<<pm_grid(n), 256, 0, s>>>(pos, mass, n, B, N, log2N, W.R, W.sb);
+  if (N & 1) og::k_pm_deposit<false><<<pm_grid(n), 256, 0, s>>>(pos, mass, n, B, N, log2N, W.R, W.sb);
+  else og::k_pm_deposit<true><<<pm_grid(n), 256, 0, s>>>(pos, mass, n, B, N, log2N, W.R, W.sb);
   if (cudaGetLastError() != cudaSuccess) return OG_ECUDA;
   if (cufftSetStream(plan->r2c, s) != CUFFT_SUCCESS || cufftSetWorkArea(plan->r2c, W.work) != CUFFT_SUCCESS ||
       cufftExecR2C(plan->r2c, W.R, W.C) != CUFFT_SUCCESS)
@@ -589,7 +594,8 @@ og_status og_pm_accel(og_pm_plan* plan, const double* pos, const double* mass, i
   if (cufftSetStream(plan->c2r, s) != CUFFT_SUCCESS || cufftSetWorkArea(plan->c2r, W.work) != CUFFT_SUCCESS ||
       cufftExecC2R(plan->c2r, W.C, W.R) != CUFFT_SUCCESS)
     return OG_ECUDA;
-  og::k_pm_interp<<<pm_grid(n), 256, 0, s>>>(pos, n, B, N, log2N, (float)(N / box), W.R, acc);
+  const unsigned iblocks = (unsigned)((n + og::kInterpThreads - 1) / og::kInterpThreads);
+  og::k_pm_interp<<<iblocks, og::kInterpThreads, 0, s>>>(pos, n, B, N, log2N, (float)(N / box), W.R, acc);
   return cudaGetLastError() == cudaSuccess ? OG_OK : OG_ECUDA;
 }
 
