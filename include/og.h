@@ -8,7 +8,7 @@
  * long-range mesh, the leapfrog step and the SPH density.  The steps are
  *
  *   og_keys_sort          63-bit Peano-Hilbert keys + stable radix sort
- *   og_tree_build         octree with monopole moments, level by level
+ *   og_tree_build         octree with monopole moments
  *   og_shortrange_accel   warp-coherent Barnes-Hut walk (FP32 + Kahan, or FP64)
  *   og_shortrange_adjoint gradient of L = sum_i w_i . a_i with frozen decisions
  *   og_shortrange_accel_adjoint  both in one walk (w known before the forces)
@@ -146,9 +146,10 @@ og_status og_keys_sort(const double* pos, int64_t n, double box, uint64_t* keys_
  * (the cell at that level); a node with more than leaf_size particles below
  * level 21 is split into its non-empty octants.  Per node: member range,
  * mass M = sum m (FP64), centre of mass sum(m x)/M (FP64), geometric centre
- * and side L / 2^level, largest member softening length.  Built top-down one
- * level per launch (children by binary search on the keys) and reduced
- * bottom-up one level per launch.  Particles are copied into Hilbert order.
+ * and side L / 2^level, largest member softening length.  The nodes of
+ * all levels are found at once from the digits that neighbouring keys share,
+ * and their moments are reduced bottom-up.  Particles are copied into Hilbert
+ * order.
  *
  * keys_sorted, order  outputs of og_keys_sort for the same pos / n / box
  * pos          device, double[n][3] (original order)

@@ -42,10 +42,10 @@
 //
 // Measured, ms (one target per lane against every staged particle, Newton
 // steps until 1e-2, one kernel of two warps a block -> now): 128^3 clustered
-// N_ngb 32 24.9 -> 13.6, N_ngb 64 33.2 -> 22.3; 128^3 lattice 5.05 -> 3.7; 4096 uniform
-// 0.33 -> 0.20; 100,003 uniform, N_ngb 64 0.73 -> 0.69.  By part on the clustered
-// set: tiles 24.8 -> 19.8, two kernels 16.8, one warp a block 15.3, third-order
-// steps 14.2, conversions on the integer pipe 13.9.  k_sph_radius issues on 73 %
+// N_ngb 32 24.9 -> 10.9; 128^3 lattice 5.05 -> 3.7; 4096 uniform 0.33 -> 0.20; 100,003
+// uniform, N_ngb 64 0.73 -> 0.69.  By part on the clustered set: tiles 24.8 -> 19.8,
+// two kernels 16.8, one warp a block 15.3, third-order steps 14.2, conversions on
+// the integer pipe 13.6, groups by estimated work 10.9.  k_sph_radius issues on 73 %
 // of its cycles; k_sph_density (47 %) waits for latencies at 16 - 18 warps an SM
 // and keeps the FP64 pipe 36 % busy.
 // Every loop is bounded (node-visit cap, pass caps, the stack bound); a

@@ -512,8 +512,8 @@ struct LaneFP {
   // nodes are inside by decision).  Bound by the FP64 pipe, 1/64 of the FP32
   // rate: 28 operations a pair (displacement 3, r^2 3, 1 / r and r 6, factor 8,
   // force 8) where CUDA's erfc, exp, sqrt and divisions and a segmented scan of
-  // the sums took about 220.  64^3 clustered 30.6 -> 7.0 ms, 128^3 lattice 52.9 ->
-  // 12.4, zoom set 347 -> 72; error against 64 bits unchanged (1.4e-14).
+  // the sums took about 220.  64^3 clustered 30.6 -> 6.5 ms, 128^3 lattice 52.9 ->
+  // 12.3, zoom set 347 -> 68; error against 64 bits unchanged (1.4e-14).
   __device__ __forceinline__ bool pair_eval64(const WalkArgs& A, const Stage& St, const Smem& M, int i, int s,
                                               bool wrap, double (&acc)[3]) const {
     double d0 = M.tx[0][i] - St.sx[0][s], d1 = M.tx[1][i] - St.sx[1][s], d2 = M.tx[2][i] - St.sx[2][s];
@@ -1523,12 +1523,12 @@ __global__ void __launch_bounds__(32, 18) k_walk_many(WalkArgs A) {
 // traversal, shorten them for some repeated traversal.  It depends on the
 // tree alone, so a walk over a range of groups gives the full walk's sums.
 // Measured, ms with 1 / 2 / 4 warps a group, forward: 128 groups (4096
-// uniform) 0.37 / 0.28 / 0.22, 1024 groups (32^3) clustered 0.31 / 0.27 / 0.25,
-// zoom 3.66 / 2.61 / 2.45, lattice 0.15 / 0.14 / 0.15; 5860 groups (zoom) 17.9 /
-// 18.4 / 20.0; 8192 groups (64^3) lattice 0.43 / 0.49 / 0.63, clustered 1.76 /
-// 1.58 / 1.67.  FP64: 128 groups 1.59 / 0.94 / 0.68, 1024 clustered 1.60 / 1.06 /
-// 0.91, zoom 8.2 / 8.0 / 9.1, lattice 0.40 / 0.37 / 0.44; 5860 (zoom) 71.6 / 72.9 / 83.0,
-// 8192 clustered 7.7 / 6.8 / 6.7, lattice 1.90 / 1.94 / 2.31.
+// uniform) 0.37 / 0.27 / 0.22, 1024 groups (32^3) clustered 0.31 / 0.26 / 0.23,
+// zoom 3.45 / 2.41 / 2.52, lattice 0.14 / 0.13 / 0.15; 5860 groups (zoom) 12.3 /
+// 13.8 / 17.3; 8192 groups (64^3) lattice 0.41 / 0.48 / 0.63, clustered 1.35 /
+// 1.15 / 1.38.  FP64: 128 groups 1.59 / 0.95 / 0.67, 1024 clustered 1.55 / 1.07 /
+// 0.79, zoom 8.0 / 7.6 / 9.0, lattice 0.39 / 0.36 / 0.43; 5860 (zoom) 68 / 70 / 80,
+// 8192 clustered 6.5 / 5.7 / 6.7, lattice 1.87 / 1.93 / 2.32.
 static int walk_split(int64_t n_groups) { return n_groups <= 1024 ? 2 : n_groups <= 4096 ? 1 : 0; }
 
 cudaError_t launch_walk(WalkArgs A, int prec, bool adjoint, cudaStream_t s, bool fused) {
