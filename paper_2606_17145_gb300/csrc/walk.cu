@@ -1505,15 +1505,18 @@ __device__ __forceinline__ void walk_groups(const WalkArgs& A) {
 // share their sources in L1.  Forward, ms, before / after: lattice 128^3 2.55 / 2.48,
 // clustered 128^3 17.1 / 16.5, 256^3 405 / 387, 90^3 (22,782 groups) 3.59 / 3.58;
 // 5860 groups (zoom) 12.4 / 13.1, 128 groups 0.221 / 0.240.  Adjoint 128^3 clustered
-// 22.8 / 24.2: its code fits the instruction cache less well.
+// 22.8 / 24.2: its code fits the instruction cache less well.  The FP64 walk, which
+// shares little in L1 for its arithmetic, runs 16 in blocks of one: a block of
+// two lasts as long as its longer group.  64^3 lattice 1.90 -> 1.81 ms, clustered 58^3
+// 5.3 -> 5.0, 64^3 6.5 -> 6.35; zoom 68.6 -> 69.2 (18 warps: 1.74, 5.0, 6.6 and 66.4).
 constexpr int64_t kManyGroups = 24576;
 
 template <class Lane>
 __global__ void __launch_bounds__(64) k_walk(WalkArgs A) {
   walk_groups<Lane, 2>(A);
 }
-template <class Lane>
-__global__ void __launch_bounds__(32, 18) k_walk_many(WalkArgs A) {
+template <class Lane, int kBlocks>
+__global__ void __launch_bounds__(32, kBlocks) k_walk_one(WalkArgs A) {
   walk_groups<Lane, 1>(A);
 }
 
@@ -1539,8 +1542,8 @@ cudaError_t launch_walk(WalkArgs A, int prec, bool adjoint, cudaStream_t s, bool
   const unsigned pairs = (unsigned)((warps + 1) / 2);
   if (fused) k_walk<LaneFused><<<pairs, 64, 0, s>>>(A);
   else if (adjoint) k_walk<LaneF32<true>><<<pairs, 64, 0, s>>>(A);
-  else if (prec == OG_FP64) k_walk<LaneF64><<<pairs, 64, 0, s>>>(A);
-  else if (A.T.ngroups >= kManyGroups) k_walk_many<LaneF32<false>><<<(unsigned)warps, 32, 0, s>>>(A);
+  else if (prec == OG_FP64) k_walk_one<LaneF64, 16><<<(unsigned)warps, 32, 0, s>>>(A);
+  else if (A.T.ngroups >= kManyGroups) k_walk_one<LaneF32<false>, 18><<<(unsigned)warps, 32, 0, s>>>(A);
   else k_walk<LaneF32<false>><<<pairs, 64, 0, s>>>(A);
   return cudaGetLastError();
 }
