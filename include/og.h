@@ -151,7 +151,8 @@ og_status og_keys_sort(const double* pos, int64_t n, double box, uint64_t* keys_
  * and their moments are reduced bottom-up.  Particles are copied into Hilbert
  * order.
  *
- * keys_sorted, order  outputs of og_keys_sort for the same pos / n / box
+ * keys_sorted, order  outputs of og_keys_sort for the same pos / n / box (keys
+ *              that do not ascend are reported as OG_ETREE)
  * pos          device, double[n][3] (original order)
  * mass         device, double[n] (original order), > 0
  * eps          device, double[n] softening lengths (original order), or NULL

@@ -258,7 +258,11 @@ __global__ void __launch_bounds__(kTopoThreads) k_count(TreeDev T, const uint64_
   if (blockIdx.x == 0 && threadIdx.x == 0) T.sb->magic = kMagicTree;
   if (threadIdx.x < kLevels) s_cnt[threadIdx.x] = 0;
   int lo, hi, deep;
-  node_levels(keys, T.n, leaf_size, blockIdx.x * (int64_t)kTopoThreads, s_far, lo, hi, deep);
+  const int64_t i0 = blockIdx.x * (int64_t)kTopoThreads, i = i0 + threadIdx.x;
+  node_levels(keys, T.n, leaf_size, i0, s_far, lo, hi, deep);
+  // All that follows holds for sorted keys.  Of others the nodes' ranges still
+  // lie inside the particles, but a node may be nobody's child.
+  if (i > 0 && i < T.n && keys[i - 1] > keys[i]) set_status(T.sb, ST_TREELINK);
   for (int l = lo; l <= hi; ++l) atomicAdd(&s_cnt[l], 1);
   __syncthreads();
   if (threadIdx.x < kLevels) T.blk[threadIdx.x * T.nblk + blockIdx.x] = s_cnt[threadIdx.x];
@@ -515,6 +519,12 @@ __global__ void __launch_bounds__(kUpThreads) k_upward(TreeDev T, BoxScale B) {
       for (int c = 0; c < 8; ++c) {
         if (left > 0) ++nch;
         left -= cy[c];
+      }
+      // children past the last node or more than eight: the keys are not sorted,
+      // or not of 63 bits
+      if (left > 0 || D.z + nch > total) {
+        set_status(T.sb, ST_TREELINK);
+        continue;
       }
       double m8[8], s8[3][8], h8[8];
 #pragma unroll
