@@ -233,6 +233,15 @@ inline size_t carve_adj(void* buf, int64_t n, int64_t cap, AdjWs* W) {
 
 __device__ inline void set_status(StatusBlock* sb, uint32_t bits) { atomicOr(&sb->status, bits); }
 
+// The group at place i of the walks' order o.  An entry that is no group (a
+// damaged tree) is reported, and the nearest index that is one is walked instead.
+__device__ __forceinline__ int64_t group_at(const TreeDev& T, int o, int64_t i, StatusBlock* sb) {
+  const int e = T.gorder[o][i];
+  const int g = min(max(e, 0), (int)T.ngroups - 1);
+  if (g != e) set_status(sb, ST_TREELINK);
+  return g;
+}
+
 // Polls of the grid barrier before it gives up (seconds, far above a level).
 constexpr int kBarrierPolls = 1 << 24;
 

@@ -730,9 +730,10 @@ __device__ __forceinline__ float sph_max(float x) {  // over the warp, x >= 0
 // (tree_build.cu).  Against tree order, ms: clustered 64^3 3.20 -> 2.86, 90^3 6.86 ->
 // 5.44, 128^3 13.6 -> 10.9; 10^6 uniform particles 2.65 -> 2.65; 128^3 lattice
 // 3.67 -> 3.70.  (Ordered by count alone: 11.6 ms at 128^3.)
-__device__ __forceinline__ int64_t sph_group(const TreeDev& T, int64_t i) {
+__device__ __forceinline__ int64_t sph_group(const SphArgs& A, int64_t i) {
+  const TreeDev& T = A.T;
   const bool usable = i < T.ngroups && T.sb->status == 0 && T.sb->magic == kMagicTree;
-  return usable ? T.gorder[0][i] : i;
+  return usable ? group_at(T, 0, i, A.wsb) : i;
 }
 
 // FP32 Newton passes on ln h.  Leaves h (box units) in h_out for the finishing
@@ -741,7 +742,7 @@ __global__ void __launch_bounds__(kSphWarps * 32) k_sph_radius(SphArgs A) {
   __shared__ SphWarp s_warp[kSphWarps];
   const TreeDev& T = A.T;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t vw = (int64_t)blockIdx.x * kSphWarps + wib, g = sph_group(T, vw >> A.split);
+  const int64_t vw = (int64_t)blockIdx.x * kSphWarps + wib, g = sph_group(A, vw >> A.split);
   const bool mine = (lane >> (5 - A.split)) == (int)(vw & ((1 << A.split) - 1));
   SphBufs W;
   int nodes_total;
@@ -824,7 +825,7 @@ __global__ void __launch_bounds__(kSphWarps * 32, 18) k_sph_density(SphArgs A) {
   __shared__ int s_list[kSphWarps][kSphList][32];
   const TreeDev& T = A.T;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t vw = (int64_t)blockIdx.x * kSphWarps + wib, g = sph_group(T, vw >> A.split);
+  const int64_t vw = (int64_t)blockIdx.x * kSphWarps + wib, g = sph_group(A, vw >> A.split);
   const bool mine = (lane >> (5 - A.split)) == (int)(vw & ((1 << A.split) - 1));
   SphBufs W;
   int nodes_total;

@@ -1227,7 +1227,7 @@ __device__ __forceinline__ void walk_groups(const WalkArgs& A) {
   const int64_t gi = A.g_begin + (v >> A.split);
   if (gi >= A.g_end) return;
   const bool usable = T.sb->status == 0 && T.sb->magic == kMagicTree;
-  const int64_t g = A.ordered && usable ? T.gorder[Lane::kOrder][gi] : gi;
+  const int64_t g = A.ordered && usable ? group_at(T, Lane::kOrder, gi, A.wsb) : gi;
   const bool mine = (lane >> (5 - A.split)) == (int)(v & ((1 << A.split) - 1));
   if (!usable) {
     // a failed or missing tree: flag it and give every output of this
