@@ -42,6 +42,8 @@ struct StatusBlock {
 };
 static_assert(sizeof(StatusBlock) <= kAlign, "status block fits 256 bytes");
 
+constexpr int kTreeWildMass = 0;  // tree buffers, of pad: some m / L^2 (of a particle or a node) overflows FP32
+
 constexpr uint32_t kMagicTree = 0x0637ee01u;
 constexpr uint32_t kMagicWs = 0x0637ee02u;
 

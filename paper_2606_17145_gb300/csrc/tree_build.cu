@@ -26,6 +26,8 @@
 // 1050 -> 887 us, 100,003-particle SPH 1.15 -> 0.96 ms.  At 2.1 M particles the
 // kernels take 0.063 (permute), 0.020, 0.008, 0.077 (fill), 0.048 (leaves) and
 // 0.084 ms (upward).
+#include <cfloat>
+
 #include "og_internal.cuh"
 
 namespace og {
@@ -209,6 +211,7 @@ __global__ void k_permute(BuildArgs A, BoxScale B) {
       const double hb = h * B.invL;
       h2 = (float)(hb * hb);
     }
+    if (!(mw <= FLT_MAX)) atomicOr(&T.sb->pad[kTreeWildMass], 1);
     T.pA[k] = make_float4(hi[0], hi[1], hi[2], mw);
     T.pB[k] = make_float4(lo[0], lo[1], lo[2], h2);
   }
@@ -449,6 +452,7 @@ __device__ __forceinline__ void write_moments(const TreeDev& T, const BoxScale& 
     T.com64[3 * (int64_t)p + c] = com[c];
     T.cen64[3 * (int64_t)p + c] = cen[c];
   }
+  if (!(mw <= FLT_MAX)) atomicOr(&T.sb->pad[kTreeWildMass], 1);
   T.nA[p] = make_float4(hi[0], hi[1], hi[2], mw);
   T.nB[p] = make_float4(lo[0], lo[1], lo[2], h2);
   T.nC[p] = make_float4(cenb[0], cenb[1], cenb[2], side_b);

@@ -471,7 +471,8 @@ struct LaneFP {
   double a64[3];      // FP64 variant: plain double sums
   int nint;
 
-  __device__ void init(const WalkArgs& A, Smem& M, int64_t kk, bool v, int lane, const GroupInfo& G) {
+  // True if the warp's batches need batch_wild.
+  __device__ bool init(const WalkArgs& A, Smem& M, int64_t kk, bool v, int lane, const GroupInfo& G) {
     k = kk;
     valid = v;
     const int64_t kc = v ? kk : 0;  // never form an out-of-range address
@@ -494,6 +495,7 @@ struct LaneFP {
     sr = fmaf(xr[0], xr[0], fmaf(xr[1], xr[1], xr[2] * xr[2]));
 #pragma unroll
     for (int c = 0; c < 3; ++c) { P[c] = 0.f; S[c] = 0.f; C[c] = 0.f; Pf[c] = 0.f; Sf[c] = 0.f; Cf[c] = 0.f; }
+    bool wild = A.T.sb->pad[kTreeWildMass] != 0;
     if (ADJ) {
       float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
       if (v) {
@@ -501,8 +503,10 @@ struct LaneFP {
         w = make_float4(A.w[3 * (int64_t)i], A.w[3 * (int64_t)i + 1], A.w[3 * (int64_t)i + 2], 0.f);
       }
       M.tW[lane] = w;
+      wild = wild || !(fabsf(w.x) <= kWildWeight && fabsf(w.y) <= kWildWeight && fabsf(w.z) <= kWildWeight);
     }
     nint = 0;
+    return !F64 && __any_sync(0xffffffffu, wild);
   }
 
   // FP64 variant: force of staged slot s on target i, added to acc; false
@@ -672,6 +676,7 @@ struct LaneFP {
   }
 
   // Evaluate the queued entries (see the header comment).
+  template <bool WILD>
   __device__ void evaluate(const WalkArgs& A, const WarpBufs& W, Stage& St, Smem& M, int nq, int lane,
                            const GroupInfo& G, const float4* SGB, int64_t gbase, uint32_t vmask, float Rg) {
     const int total = queue_offsets(A, W, nq, lane);
@@ -721,6 +726,8 @@ struct LaneFP {
         if constexpr (F64) {
 #pragma unroll 1
           for (int hb = 0; hb < pend; hb += 32) batch_list(A, W, St, M, hb, min(pend - hb, 32), lane, vmask, mi);
+        } else if constexpr (WILD) {
+          batch_wild(A, St, M, pend, lane, gbase + lane, mi);
         } else {
           batch_tiles(A, W, St, M, SGB, pend, lane, gbase, vmask, mi);
         }
@@ -875,6 +882,79 @@ struct LaneFP {
     }
     force_f32<ADJ>(A, r2, h2, F, Fr);
     return true;
+  }
+
+  // Adjoint: a source's sums into its accumulators (id: particle, or -2 - node).
+  static __device__ __forceinline__ void add_source(const WalkArgs& A, int id, const float4& g) {
+    double* Gd = id >= 0 ? A.Gp + 3 * (int64_t)id : A.Gn + 3 * (int64_t)(-2 - id);
+    double* Sd = id >= 0 ? A.Sp + id : A.Sn + (-2 - id);
+    atomicAdd(Gd, f2d_exact(g.x));
+    atomicAdd(Gd + 1, f2d_exact(g.y));
+    atomicAdd(Gd + 2, f2d_exact(g.z));
+    atomicAdd(Sd, f2d_exact(g.w));
+  }
+
+  // The tiles add every listed pair, those that are no hits with a factor of
+  // zero, which clears the term only while its operands are finite: dL/da up to
+  // kWildWeight (a sum of three products with displacements below 0.87) and
+  // masses that do not overflow FP32.  A warp with others evaluates its batches
+  // here, hit by hit: lane = target, slot after slot.
+  static constexpr float kWildWeight = 1e38f;
+  __device__ void batch_wild(const WalkArgs& A, const Stage& St, Smem& M, int cnt, int lane, int64_t i, bool mi) {
+    const float4 ta = M.tA[lane], tb = M.tB[lane];
+    const int so = M.self[lane];
+#pragma unroll 1
+    for (int s = 0; s < cnt; ++s) {
+      const int e = 4 * (s >> 1) + (s & 1);
+      const float* p0 = &St.s0[0].x + e;
+      const float* p1 = &St.s1[0].x + e;
+      const float* p2 = &St.s2[0].x + e;
+      const float* p3 = &St.s3[0].x + e;
+      float d0 = ta.x + p0[0], d1 = ta.y + p0[2], d2 = ta.z + p1[0];
+      if (mi) {
+        d0 = mi1(d0);
+        d1 = mi1(d1);
+        d2 = mi1(d2);
+      }
+      d0 += tb.x + p2[0];
+      d1 += tb.y + p2[2];
+      d2 += tb.z + p3[0];
+      const float r2 = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
+      const int id = St.id[s];
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (((St.sq[s] >> lane) & 1u) && s != so && r2 <= A.pp_hi &&
+          (r2 < A.pp_lo || id < 0 || pair_inside_exact(A, i, id))) {
+        float F, Fr;
+        force_f32<ADJ>(A, r2, fmaxf(ta.w, p3[2]), F, Fr);
+        ++nint;
+        const float nm = p1[2], sc = nm * F;
+        float(&f)[3] = ADJ ? Pf : P;
+        f[0] = fmaf(sc, d0, f[0]);
+        f[1] = fmaf(sc, d1, f[1]);
+        f[2] = fmaf(sc, d2, f[2]);
+        if constexpr (ADJ) {
+          const float4 w = M.tW[lane];
+          const float dw = fmaf(d0, w.x, fmaf(d1, w.y, d2 * w.z));
+          const float qq = Fr * dw;
+          v[0] = fmaf(F, w.x, qq * d0);
+          v[1] = fmaf(F, w.y, qq * d1);
+          v[2] = fmaf(F, w.z, qq * d2);
+          v[3] = F * dw;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) P[c] = fmaf(nm, v[c], P[c]);
+        }
+      }
+      if constexpr (ADJ) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+        if (lane == 0) add_source(A, id, make_float4(-v[0], -v[1], -v[2], -v[3]));
+      }
+    }
+    M.self[lane] = -1;
+    fold();
+    __syncwarp();
   }
 
   // One FP32 batch: the cnt staged sources, as pairs of adjacent slots.
@@ -1045,13 +1125,7 @@ struct LaneFP {
         const int s = lane + 32 * u;
         const float4 g = M.SG[s];
         if (s < cnt && (g.x != 0.f || g.y != 0.f || g.z != 0.f || g.w != 0.f)) {
-          const int id = St.id[s];
-          double* Gd = id >= 0 ? A.Gp + 3 * (int64_t)id : A.Gn + 3 * (int64_t)(-2 - id);
-          double* Sd = id >= 0 ? A.Sp + id : A.Sn + (-2 - id);
-          atomicAdd(Gd, f2d_exact(g.x));
-          atomicAdd(Gd + 1, f2d_exact(g.y));
-          atomicAdd(Gd + 2, f2d_exact(g.z));
-          atomicAdd(Sd, f2d_exact(g.w));
+          add_source(A, St.id[s], g);
         }
         M.SG[s] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
@@ -1211,21 +1285,28 @@ union WarpScratch {
   typename Lane::Stage stage;
 };
 
-template <class Lane, int kWarpsPerBlock>
-__device__ __forceinline__ void walk_groups(const WalkArgs& A) {
-  __shared__ int2 s_stack[kWarpsPerBlock][kStack];
-  __shared__ int4 s_queue[kWarpsPerBlock][kQueue];
-  __shared__ int s_qoff[kWarpsPerBlock][kQueue + 1];
-  __shared__ unsigned short s_list[kWarpsPerBlock][Lane::kListSize];
-  __shared__ WarpScratch<Lane> s_scr[kWarpsPerBlock];
-  __shared__ typename Lane::Smem s_lane[kWarpsPerBlock];
-  __shared__ float4 s_sgb[kWarpsPerBlock][2 * kSub];
+// Shared memory of a warp.
+template <class Lane>
+struct WalkShared {
+  int2 stack[kStack];
+  int4 queue[kQueue];
+  int qoff[kQueue + 1];
+  unsigned short list[Lane::kListSize];
+  WarpScratch<Lane> scr;
+  typename Lane::Smem lane;
+  float4 sgb[2 * kSub];
+};
+
+// The walk of this warp's group.  Without WILD it returns true, having done
+// nothing, if the group needs the variant with it (batch_wild).
+template <class Lane, int kWarpsPerBlock, bool WILD>
+__device__ __forceinline__ bool walk_groups(const WalkArgs& A, WalkShared<Lane>& S) {
   const TreeDev& T = A.T;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   // 2^split warps serve a group, each its part of the targets
   const int64_t v = (int64_t)blockIdx.x * kWarpsPerBlock + wib;
   const int64_t gi = A.g_begin + (v >> A.split);
-  if (gi >= A.g_end) return;
+  if (gi >= A.g_end) return false;
   const bool usable = T.sb->status == 0 && T.sb->magic == kMagicTree;
   const int64_t g = A.ordered && usable ? group_at(T, Lane::kOrder, gi, A.wsb) : gi;
   const bool mine = (lane >> (5 - A.split)) == (int)(v & ((1 << A.split) - 1));
@@ -1252,16 +1333,16 @@ __device__ __forceinline__ void walk_groups(const WalkArgs& A) {
       }
       if (A.counts) A.counts[io] = -1;
     }
-    return;
+    return false;
   }
   WarpBufs W;
-  W.stack = s_stack[wib];
-  W.queue = s_queue[wib];
-  W.qoff = s_qoff[wib];
-  W.list = s_list[wib];
-  MixedScratch& X = s_scr[wib].mix;
-  typename Lane::Stage& St = s_scr[wib].stage;
-  typename Lane::Smem& M = s_lane[wib];
+  W.stack = S.stack;
+  W.queue = S.queue;
+  W.qoff = S.qoff;
+  W.list = S.list;
+  MixedScratch& X = S.scr.mix;
+  typename Lane::Stage& St = S.scr.stage;
+  typename Lane::Smem& M = S.lane;
   int nodes_total = 0;
 #pragma unroll 1
   for (int l = 0; l < kLevels; ++l) nodes_total += T.sb->level_cnt[l];
@@ -1271,14 +1352,14 @@ __device__ __forceinline__ void walk_groups(const WalkArgs& A) {
   const int64_t k = gbase + lane;
   const bool valid = mine && k < T.n;
   const uint32_t vmask = __ballot_sync(0xffffffffu, valid);
-  if (vmask == 0u) return;  // a part beyond the last particle
+  if (vmask == 0u) return false;  // a part beyond the last particle
   const uint32_t lt = (1u << lane) - 1u;
 
   // boxes of this warp's targets and of the 4 sub-groups of 8 targets (box
   // units, padded outward by more than the FP32 rounding of a position in
   // [0, 1))
   GroupInfo G;
-  float4* SGB = s_sgb[wib];
+  float4* SGB = S.sgb;
   {
     const float4 pa = T.pA[valid ? k : 0], pb = T.pB[valid ? k : 0];
     float lo[3] = {pa.x + pb.x, pa.y + pb.y, pa.z + pb.z};
@@ -1308,7 +1389,7 @@ __device__ __forceinline__ void walk_groups(const WalkArgs& A) {
   const float Rg = sqrtf(fmaf(G.ex, G.ex, fmaf(G.ey, G.ey, G.ez * G.ez))) * 1.0001f + 1e-6f;
 
   Lane L;
-  L.init(A, M, k, valid, lane, G);
+  if (L.init(A, M, k, valid, lane, G) && !WILD) return true;
 
   if (lane == 0) W.stack[0] = make_int2((int)(1u << 28), (int)vmask);  // the root: node 0, one node
   int sp = 1, nq = 0;
@@ -1486,7 +1567,7 @@ __device__ __forceinline__ void walk_groups(const WalkArgs& A) {
       }
       __syncwarp();
     } else if (nq > 0) {
-      L.evaluate(A, W, St, M, nq, lane, G, SGB, gbase, vmask, Rg);
+      L.template evaluate<WILD>(A, W, St, M, nq, lane, G, SGB, gbase, vmask, Rg);
       nq = 0;
       __syncwarp();
     } else {
@@ -1498,6 +1579,21 @@ __device__ __forceinline__ void walk_groups(const WalkArgs& A) {
     const unsigned cnt = __reduce_add_sync(0xffffffffu, (unsigned)(valid ? L.nint : 0));
     if (lane == 0 && cnt) atomicAdd(A.total, (unsigned long long)cnt);
   }
+  return false;
+}
+
+// Not inlined, so that the walk of all other groups keeps its registers.
+template <class Lane, int kWarpsPerBlock>
+__device__ __noinline__ void walk_wild(const WalkArgs& A, WalkShared<Lane>& S) {
+  walk_groups<Lane, kWarpsPerBlock, true>(A, S);
+}
+template <class Lane, int kWarpsPerBlock>
+__device__ __forceinline__ void walk_block(const WalkArgs& A) {
+  __shared__ WalkShared<Lane> s_walk[kWarpsPerBlock];
+  WalkShared<Lane>& S = s_walk[threadIdx.x >> 5];
+  const bool wild = walk_groups<Lane, kWarpsPerBlock, false>(A, S);
+  if constexpr (!std::is_same<Lane, LaneF64>::value)
+    if (wild) walk_wild<Lane, kWarpsPerBlock>(A, S);
 }
 
 // Forward walks of many groups run 18 to 20 warps an SM, in blocks of one (96
@@ -1513,11 +1609,11 @@ constexpr int64_t kManyGroups = 24576;
 
 template <class Lane>
 __global__ void __launch_bounds__(64) k_walk(WalkArgs A) {
-  walk_groups<Lane, 2>(A);
+  walk_block<Lane, 2>(A);
 }
 template <class Lane, int kBlocks>
 __global__ void __launch_bounds__(32, kBlocks) k_walk_one(WalkArgs A) {
-  walk_groups<Lane, 1>(A);
+  walk_block<Lane, 1>(A);
 }
 
 // Warps per group (log2).  A walk of fewer groups than the chip holds warps
