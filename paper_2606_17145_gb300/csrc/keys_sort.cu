@@ -475,15 +475,11 @@ namespace {
 
 constexpr int64_t kNoAllocMaxN = int64_t(1) << 20;
 constexpr size_t noalloc_round(size_t x) { return (x + og::kAlign - 1) / og::kAlign * og::kAlign; }
-// The most tiles of any n up to that: at the last n of either tile size.
-constexpr int64_t kNoAllocTiles = og::sort_tiles(og::kSortFew) > og::sort_tiles(kNoAllocMaxN)
-                                      ? og::sort_tiles(og::kSortFew) : og::sort_tiles(kNoAllocMaxN);
-static_assert(og::kSortFew <= kNoAllocMaxN, "either tile size is reached");
 // Same carving as og::carve_sort: status block, histograms, alternate keys,
 // alternate indices, two passes' tile counts.
 constexpr size_t kNoAllocBytes =
     og::kSortZeroBytes + noalloc_round(sizeof(uint64_t) * kNoAllocMaxN) + noalloc_round(sizeof(int32_t) * kNoAllocMaxN) +
-    2 * noalloc_round(sizeof(uint32_t) * 256 * kNoAllocTiles);
+    2 * noalloc_round(sizeof(uint32_t) * 256 * og::sort_tiles_room(kNoAllocMaxN));
 
 // Held by every GPU that loads the library, until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_sort_ws[kNoAllocBytes];

@@ -179,6 +179,11 @@ __host__ __device__ constexpr int sort_items(int64_t n) { return n <= kSortFew ?
 __host__ __device__ constexpr int64_t sort_tiles(int64_t n) {
   return (n + kSortThreads * sort_items(n) - 1) / (kSortThreads * sort_items(n));
 }
+// Tiles that a workspace for n keys holds: the most of any count up to n, so that
+// it serves fewer keys as well (past kSortFew the tiles grow by four).
+__host__ __device__ constexpr int64_t sort_tiles_room(int64_t n) {
+  return n > kSortFew && sort_tiles(kSortFew) > sort_tiles(n) ? sort_tiles(kSortFew) : sort_tiles(n);
+}
 constexpr size_t kSortZeroBytes = kAlign + sizeof(uint32_t) * 8 * 256;  // status block and histograms
 
 inline size_t carve_sort(void* buf, int64_t n, SortWs* W) {
@@ -195,7 +200,7 @@ inline size_t carve_sort(void* buf, int64_t n, SortWs* W) {
   w.hist = static_cast<uint32_t*>(take(sizeof(uint32_t) * 8 * 256));
   w.keys_alt = static_cast<uint64_t*>(take(sizeof(uint64_t) * n));
   w.vals_alt = static_cast<int32_t*>(take(sizeof(int32_t) * n));
-  for (int i = 0; i < 2; ++i) w.tile_state[i] = static_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * w.ntiles));
+  for (int i = 0; i < 2; ++i) w.tile_state[i] = static_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * sort_tiles_room(n)));
   if (W) *W = w;
   return off;
 }

@@ -106,3 +106,13 @@ def test_sph_and_integrator_host_argument_checks(L):
     assert L.og_kick(None, p, None, 10, 0.1, None) == N.OG_EINVAL
     assert L.og_kick(p, p, None, 0, 0.1, None) == N.OG_EINVAL
     assert L.og_drift(p, p, 10, float("nan"), None) == N.OG_EINVAL
+
+
+def test_workspace_sizes_never_decrease(L):
+    """A buffer sized for n particles serves every smaller count."""
+    around = [1, 1000, 16384, 1 << 18, 1 << 20, 1 << 24]
+    around += [512 * 1024, 1024 * 32, 4096 * 32, 256 * 1024, 290_000]
+    ns = sorted({max(1, a + d) for a in around for d in (-4097, -1025, -513, -33, -1, 0, 1, 33, 513, 1025, 4097, 30_000)})
+    for size in (L.og_keys_sort_ws_bytes, lambda n: L.og_tree_bytes(n, None)):
+        sizes = [size(n) for n in ns]
+        assert all(a <= b for a, b in zip(sizes, sizes[1:]))

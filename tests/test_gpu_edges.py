@@ -69,6 +69,18 @@ def test_sort_tile_sizes(orc, n):
     assert np.array_equal(keys.cpu().numpy().view(np.uint64), ks) and np.array_equal(order.cpu().numpy(), o)
 
 
+@pytest.mark.parametrize("room,n", [((1 << 18) + 1, 1 << 18), (290_000, 235_000), ((1 << 18) + 1, 16384)])
+def test_sort_in_a_larger_workspace(orc, room, n):
+    """A workspace sized for more keys, in tiles of the other size, serves fewer."""
+    dev = device()
+    m = og()
+    ws = m._workspace(m.lib().og_keys_sort_ws_bytes(room), dev)
+    pos = np.random.default_rng(n).random((n, 3))
+    keys, order = m.keys_sort(torch.tensor(pos, dtype=torch.float64, device=dev), 1.0, ws=ws)
+    ks, o = orc.sort(orc.keys(pos, 1.0)[0])
+    assert np.array_equal(keys.cpu().numpy().view(np.uint64), ks) and np.array_equal(order.cpu().numpy(), o)
+
+
 @pytest.mark.parametrize("axis", ["random", "ones"])
 def test_keys_by_table_and_by_bits(axis):
     """Keys of more than 16,384 particles are looked up level by level, fewer
