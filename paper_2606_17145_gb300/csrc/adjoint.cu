@@ -16,69 +16,79 @@
 
 namespace og {
 
-// One cooperative launch, level by level from the root with a grid barrier
-// between levels (block 0 alone while they are small): 22 launches, most of them
-// for empty or tiny levels, took 135 us on 2.1 M particles and 90 us on a few
-// thousand.
 constexpr int kDownThreads = 512;
+__device__ __forceinline__ void push_down(const TreeDev& T, const AdjWs& W, int p, double invL) {
+  const float4 NC = T.nC[p];
+  const double C[3] = {(double)NC.x, (double)NC.y, (double)NC.z};
+  double G[3], X[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    G[c] = W.Gn[3 * (int64_t)p + c];
+    X[c] = T.com64[3 * (int64_t)p + c] * invL;
+  }
+  double B = W.Sn[p] - (G[0] * (C[0] - X[0]) + G[1] * (C[1] - X[1]) + G[2] * (C[2] - X[2]));
+  const int q = T.nParent[p];
+  if (q >= 0) {
+    const float4 QC = T.nC[q];
+    const double Cq[3] = {(double)QC.x, (double)QC.y, (double)QC.z};
+    double CGq[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) CGq[c] = __ldcg(&W.CG[3 * (int64_t)q + c]);
+    B += __ldcg(&W.Bn[q]) - (CGq[0] * (C[0] - Cq[0]) + CGq[1] * (C[1] - Cq[1]) + CGq[2] * (C[2] - Cq[2]));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) G[c] += CGq[c];
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) W.CG[3 * (int64_t)p + c] = G[c];
+  W.Bn[p] = B;
+}
+
+// One launch, level by level from the root, in parts (next_part) of nodes of one
+// level; the first part is the levels from the root on that have at most
+// kDownThreads nodes each.  22 launches, most of them for empty or
+// tiny levels, took 135 us on 2.1 M particles and 90 us on a few thousand.
 __global__ void __launch_bounds__(kDownThreads) k_adj_down(TreeDev T, AdjWs W, double invL) {
   if (T.sb->status != 0) return;  // tree not usable (flagged at build time)
   int total = 0, lone = -1;
   for (int l = 0; l < kLevels; ++l) {
     total += T.sb->level_cnt[l];
-    // levels 0 .. lone have at most kDownThreads nodes each
     if (lone == l - 1 && T.sb->level_cnt[l] <= kDownThreads) lone = l;
   }
   if (total > T.cap) return;
-  int base = 0;
-  unsigned long long phase = 0;
-#pragma unroll 1
-  for (int lev = 0; lev < kLevels; ++lev) {
-    const int cnt = T.sb->level_cnt[lev];
-    if (cnt == 0) break;  // nor any below
-    const bool single = lev <= lone;
-    if (lev > 0) {
-      if (single) {
-        __threadfence_block();
-        __syncthreads();
-      } else {
-        ++phase;
-        if (!grid_barrier(&W.sb->work, phase * gridDim.x)) {
-          if (threadIdx.x == 0) set_status(W.sb, ST_WALKCAP);
-          return;
-        }
-      }
+  int lev = lone, c_l = 0, base = 0;
+  for (int l = 0; l <= lone; ++l) base += T.sb->level_cnt[l];  // nodes of the levels up to lev
+  int first = 0, next = 1, parts = 1;  // the level's first part, the next level's, their number
+  int ready = 0;
+  for (bool any = false;; any = true) {
+    const int part = next_part(W.sb, any);
+    while (part >= next) {
+      if (++lev == kLevels) return;
+      c_l = T.sb->level_cnt[lev];
+      base += c_l;
+      parts = level_parts(c_l, kDownThreads);
+      first = next;
+      next += parts;
     }
-    const int stride = single ? kDownThreads : gridDim.x * kDownThreads;
-    if (!single || blockIdx.x == 0) {
-      for (int s = (single ? 0 : blockIdx.x * kDownThreads) + threadIdx.x; s < cnt; s += stride) {
-        const int p = base + s;
-        const float4 NC = T.nC[p];
-        const double C[3] = {(double)NC.x, (double)NC.y, (double)NC.z};
-        double G[3], X[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          G[c] = W.Gn[3 * (int64_t)p + c];
-          X[c] = T.com64[3 * (int64_t)p + c] * invL;
-        }
-        double B = W.Sn[p] - (G[0] * (C[0] - X[0]) + G[1] * (C[1] - X[1]) + G[2] * (C[2] - X[2]));
-        const int q = T.nParent[p];
-        if (q >= 0) {
-          const float4 QC = T.nC[q];
-          const double Cq[3] = {(double)QC.x, (double)QC.y, (double)QC.z};
-          double CGq[3];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) CGq[c] = __ldcg(&W.CG[3 * (int64_t)q + c]);
-          B += __ldcg(&W.Bn[q]) - (CGq[0] * (C[0] - Cq[0]) + CGq[1] * (C[1] - Cq[1]) + CGq[2] * (C[2] - Cq[2]));
-#pragma unroll
-          for (int c = 0; c < 3; ++c) G[c] += CGq[c];
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) W.CG[3 * (int64_t)p + c] = G[c];
-        W.Bn[p] = B;
+    if (first > ready) {
+      if (!wait_parts(W.sb, first)) {
+        if (threadIdx.x == 0) set_status(W.sb, ST_WALKCAP);
+        return;
       }
+      ready = first;
     }
-    base += cnt;
+    if (lev > lone) {
+      for (int s = (part - first) * kDownThreads + threadIdx.x; s < c_l; s += parts * kDownThreads)
+        push_down(T, W, base - c_l + s, invL);
+      continue;
+    }
+    int p = threadIdx.x;
+    for (int l = 0; l <= lone; ++l) {
+      const int c = T.sb->level_cnt[l];
+      if ((int)threadIdx.x < c) push_down(T, W, p, invL);
+      p += c;
+      __threadfence_block();
+      __syncthreads();
+    }
   }
 }
 
@@ -109,16 +119,10 @@ __global__ void k_adj_particles(TreeDev T, AdjWs W, double L, double* __restrict
 cudaError_t launch_adjoint_push(const TreeDev& T, const AdjWs& W, double L, double* dpos, double* dmass,
                                 cudaStream_t s) {
   // the node counts live on the device: the grid is sized for the particles
-  TreeDev Tv = T;
-  AdjWs Wv = W;
-  double invL = 1.0 / L;
-  void* args[] = {&Tv, &Wv, &invL};
   int64_t grid = (T.n / 4 + kDownThreads - 1) / kDownThreads;
   if (grid > grid_cap(2)) grid = grid_cap(2);
   if (grid < 1) grid = 1;
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_adj_down, dim3((unsigned)grid), dim3(kDownThreads),
-                                                    args, 0, s);
-  if (e != cudaSuccess) return e;
+  k_adj_down<<<(unsigned)grid, kDownThreads, 0, s>>>(T, W, 1.0 / L);
   int64_t pg = (T.n + 255) / 256;
   if (pg > grid_cap(32)) pg = grid_cap(32);
   k_adj_particles<<<(unsigned)pg, 256, 0, s>>>(T, W, L, dpos, dmass);

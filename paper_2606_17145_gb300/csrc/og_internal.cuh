@@ -36,8 +36,8 @@ struct StatusBlock {
   uint32_t status;
   uint32_t magic;
   int32_t level_cnt[24];              // nodes per level (tree buffers)
-  unsigned long long counter;         // interaction count / misc
-  unsigned long long work;            // dynamic work counter
+  unsigned long long counter;         // finished parts of a launch (next_part)
+  unsigned long long work;            // taken parts
   int32_t pad[20];
 };
 static_assert(sizeof(StatusBlock) <= kAlign, "status block fits 256 bytes");
@@ -249,19 +249,46 @@ __device__ __forceinline__ int64_t group_at(const TreeDev& T, int o, int64_t i, 
   return g;
 }
 
-// Polls of the grid barrier before it gives up (seconds, far above a level).
-constexpr int kBarrierPolls = 1 << 24;
+// A launch whose parts wait for one another (the levels of the tree, one after
+// the other) without a cooperative launch, which a context that holds part of
+// the SMs may refuse.  Blocks take the parts' numbers in order from the status
+// block and count the finished ones.  A part waits only for parts of smaller
+// numbers; those were taken before it, so by running blocks, and the smallest
+// unfinished one waits for none: every wait ends, however few blocks run at a time.
+constexpr int kPartPolls = 1 << 24;  // seconds, far above a part
 
-// Barrier over the grid of a cooperative launch; false if it gave up.  Every
-// block passes the same number of blocks * phase.
-__device__ inline bool grid_barrier(unsigned long long* count, unsigned long long target) {
-  __shared__ int s_ok;
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// The next part of this block, after it has finished the one before (any).
+// Every thread of the block calls it, and wait_parts.
+__device__ __forceinline__ int next_part(StatusBlock* sb, bool any) {
+  __shared__ int s_part;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(count, 1ull);
+    if (any) {
+      __threadfence();
+      atomicAdd(&sb->counter, 1ull);
+    }
+    s_part = (int)atomicAdd(&sb->work, 1ull);
+  }
+  __syncthreads();
+  return s_part;
+}
+// Parts of a level of c_l nodes, one a block at most; part i takes the nodes from
+// i * threads on in strides of all parts' threads.
+__device__ __forceinline__ int level_parts(int c_l, int threads) {
+  return min((c_l + threads - 1) / threads, (int)gridDim.x);
+}
+// Until n parts are finished; false if that took too long.
+__device__ __forceinline__ bool wait_parts(const StatusBlock* sb, int n) {
+  __shared__ int s_ok;
+  if (threadIdx.x == 0) {
     int ok = 0;
-    for (int i = 0; i < kBarrierPolls && !ok; ++i) ok = *(volatile unsigned long long*)count >= target;
+    for (int i = 0; i < kPartPolls && !ok; ++i) ok = ld_acquire(&sb->counter) >= (unsigned long long)n;
     __threadfence();
     s_ok = ok;
   }

@@ -15,8 +15,8 @@
 // gives every node its index, and a second pass writes them.
 //
 // Moments: all leaves in one launch, then the split nodes from the deepest
-// level up in one cooperative launch with a grid barrier per level (one block
-// alone where the levels are small).  One thread serves one node and sums its
+// level up in one launch whose blocks wait for the level below (one block alone
+// where the levels are small).  One thread serves one node and sums its
 // children (or a leaf's particles) in FP64 in index order, so the result does
 // not depend on scheduling.
 //
@@ -482,91 +482,99 @@ __global__ void __launch_bounds__(256) k_leaves(TreeDev T, BoxScale B) {
   }
 }
 
-// The split nodes, from the deepest level up.
+// A split node's moments from its children's.
 constexpr int kUpThreads = 512;
-__global__ void __launch_bounds__(kUpThreads) k_upward(TreeDev T, BoxScale B) {
-  int cnt[kLevels];
-  int total = 0;
+__device__ __forceinline__ void node_moments(const TreeDev& T, const BoxScale& B, int p, int l, int total) {
+  int4 D = T.nD[p];
+  if (meta_leaf(D.w)) return;
+  // the children's counts first (independent loads), which give their
+  // number, then their sums: two memory latencies a level instead of one
+  // a child (4096 particles: 28 -> 23 us)
+  int nch = 0, left = D.y;
+  int cy[8];
 #pragma unroll
+  for (int c = 0; c < 8; ++c) cy[c] = D.z + c < total ? T.nD[D.z + c].y : 0;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    if (left > 0) ++nch;
+    left -= cy[c];
+  }
+  // children past the last node or more than eight: the keys are not sorted,
+  // or not of 63 bits
+  if (left > 0 || D.z + nch > total) {
+    set_status(T.sb, ST_TREELINK);
+    return;
+  }
+  double m8[8], s8[3][8], h8[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int64_t q = D.z + (c < nch ? c : 0);
+    m8[c] = __ldcg(&T.mass64[q]);
+    s8[0][c] = __ldcg(&T.S64[3 * q]);
+    s8[1][c] = __ldcg(&T.S64[3 * q + 1]);
+    s8[2][c] = __ldcg(&T.S64[3 * q + 2]);
+    h8[c] = __ldcg(&T.hmax64[q]);
+  }
+  double M = 0.0, S0 = 0.0, S1 = 0.0, S2 = 0.0;
+  long long Hb = 0;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    if (c < nch) {
+      M += m8[c];
+      S0 += s8[0][c];
+      S1 += s8[1][c];
+      S2 += s8[2][c];
+      Hb = max(Hb, __double_as_longlong(h8[c]));
+      T.nParent[D.z + c] = p;
+    }
+  }
+  D.w = make_meta(nch, l, 0);
+  T.nD[p] = D;
+  write_moments(T, B, p, D, M, S0, S1, S2, __longlong_as_double(Hb));
+}
+
+// The split nodes, from the deepest level up, in parts (next_part) of
+// nodes of one level.  The last part is the levels from the root on that have at
+// most kUpThreads nodes each.
+__global__ void __launch_bounds__(kUpThreads) k_upward(TreeDev T, BoxScale B) {
+  int total = 0, lone = -1;
   for (int l = 0; l < kLevels; ++l) {
-    cnt[l] = T.sb->level_cnt[l];
-    total += cnt[l];
+    const int c = T.sb->level_cnt[l];
+    total += c;
+    if (lone == l - 1 && c <= kUpThreads) lone = l;
   }
   if (total > T.cap) return;  // flagged by k_fill
-  // levels 0 .. lone have at most kUpThreads nodes each: block 0 does them
-  int lone = -1;
-#pragma unroll
-  for (int l = 0; l < kLevels; ++l)
-    if (lone == l - 1 && cnt[l] <= kUpThreads) lone = l;
-  int base = total;
-  unsigned long long phase = 0;
-#pragma unroll 1
-  for (int l = kLevels - 1; l >= 0; --l) {
-    const int c_l = T.sb->level_cnt[l];
-    base -= c_l;
-    if (c_l == 0) continue;
-    const bool single = l <= lone;
-    if (single && blockIdx.x != 0) return;
-    const int stride = single ? kUpThreads : gridDim.x * kUpThreads;
-    for (int s = (single ? 0 : blockIdx.x * kUpThreads) + threadIdx.x; s < c_l; s += stride) {
-      const int p = base + s;
-      int4 D = T.nD[p];
-      if (meta_leaf(D.w)) continue;
-      // the children's counts first (independent loads), which give their
-      // number, then their sums: two memory latencies a level instead of one
-      // a child (4096 particles: 28 -> 23 us)
-      int nch = 0, left = D.y;
-      int cy[8];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) cy[c] = D.z + c < total ? T.nD[D.z + c].y : 0;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        if (left > 0) ++nch;
-        left -= cy[c];
-      }
-      // children past the last node or more than eight: the keys are not sorted,
-      // or not of 63 bits
-      if (left > 0 || D.z + nch > total) {
-        set_status(T.sb, ST_TREELINK);
-        continue;
-      }
-      double m8[8], s8[3][8], h8[8];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const int64_t q = D.z + (c < nch ? c : 0);
-        m8[c] = __ldcg(&T.mass64[q]);
-        s8[0][c] = __ldcg(&T.S64[3 * q]);
-        s8[1][c] = __ldcg(&T.S64[3 * q + 1]);
-        s8[2][c] = __ldcg(&T.S64[3 * q + 2]);
-        h8[c] = __ldcg(&T.hmax64[q]);
-      }
-      double M = 0.0, S0 = 0.0, S1 = 0.0, S2 = 0.0;
-      long long Hb = 0;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        if (c < nch) {
-          M += m8[c];
-          S0 += s8[0][c];
-          S1 += s8[1][c];
-          S2 += s8[2][c];
-          Hb = max(Hb, __double_as_longlong(h8[c]));
-          T.nParent[D.z + c] = p;
-        }
-      }
-      D.w = make_meta(nch, l, 0);
-      T.nD[p] = D;
-      write_moments(T, B, p, D, M, S0, S1, S2, __longlong_as_double(Hb));
+  int l = kLevels - 1, c_l = T.sb->level_cnt[l], base = total - c_l, parts = level_parts(c_l, kUpThreads);
+  int first = 0;  // the level's first part: as many belong to the levels below
+  int ready = 0;
+  for (bool any = false;; any = true) {
+    const int part = next_part(T.sb, any);
+    while (l > lone && part - first >= parts) {
+      first += parts;
+      c_l = T.sb->level_cnt[--l];
+      base -= c_l;
+      parts = level_parts(c_l, kUpThreads);
     }
-    if (l == 0) break;
-    if (single) {
-      __threadfence_block();
-      __syncthreads();
-    } else {
-      ++phase;
-      if (!grid_barrier(&T.sb->work, phase * gridDim.x)) {
+    if (l <= lone && part > first) return;
+    if (first > ready) {
+      if (!wait_parts(T.sb, first)) {
         if (threadIdx.x == 0) set_status(T.sb, ST_WALKCAP);
         return;
       }
+      ready = first;
+    }
+    if (l > lone) {
+      for (int s = (part - first) * kUpThreads + threadIdx.x; s < c_l; s += parts * kUpThreads)
+        node_moments(T, B, base + s, l, total);
+      continue;
+    }
+    for (;;) {
+      if ((int)threadIdx.x < c_l) node_moments(T, B, base + threadIdx.x, l, total);
+      if (l == 0) return;
+      __threadfence_block();
+      __syncthreads();
+      c_l = T.sb->level_cnt[--l];
+      base -= c_l;
     }
   }
 }
@@ -586,15 +594,11 @@ cudaError_t launch_tree_build(const BuildArgs& A, cudaStream_t s) {
   if (lgrid > grid_cap(8)) lgrid = grid_cap(8);
   if (lgrid < 1) lgrid = 1;
   k_leaves<<<(unsigned)lgrid, 256, 0, s>>>(T, B);
-  TreeDev Tv = T;
-  BoxScale Bv = B;
-  void* args[] = {&Tv, &Bv};
   int64_t ugrid = (T.n / 8 + kUpThreads - 1) / kUpThreads;
   if (ugrid > grid_cap(1)) ugrid = grid_cap(1);
   if (ugrid < 1) ugrid = 1;
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_upward, dim3((unsigned)ugrid), dim3(kUpThreads), args,
-                                                    0, s);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  k_upward<<<(unsigned)ugrid, kUpThreads, 0, s>>>(T, B);
+  return cudaGetLastError();
 }
 
 __global__ void k_copy_nodes(TreeDev T, int64_t m, int32_t* level, int32_t* first, int32_t* count, int32_t* parent,
