@@ -43,24 +43,31 @@ __device__ __forceinline__ void push_down(const TreeDev& T, const AdjWs& W, int 
   W.Bn[p] = B;
 }
 
-// One launch, level by level from the root, in parts (next_part) of nodes of one
+// One launch, level by level from the root, in parts (take_part) of nodes of one
 // level; the first part is the levels from the root on that have at most
 // kDownThreads nodes each.  22 launches, most of them for empty or
 // tiny levels, took 135 us on 2.1 M particles and 90 us on a few thousand.
 __global__ void __launch_bounds__(kDownThreads) k_adj_down(TreeDev T, AdjWs W, double invL) {
   if (T.sb->status != 0) return;  // tree not usable (flagged at build time)
-  int total = 0, lone = -1;
+  int part = take_part(W.sb);  // on its way while the levels are read
+  int cnt[kLevels];
+#pragma unroll
+  for (int l = 0; l < kLevels; ++l) cnt[l] = T.sb->level_cnt[l];
+  int total = 0, lone = -1, base = 0;  // base: nodes of the levels up to lev
+#pragma unroll
   for (int l = 0; l < kLevels; ++l) {
-    total += T.sb->level_cnt[l];
-    if (lone == l - 1 && T.sb->level_cnt[l] <= kDownThreads) lone = l;
+    total += cnt[l];
+    if (lone == l - 1 && cnt[l] <= kDownThreads) {
+      lone = l;
+      base = total;
+    }
   }
   if (total > T.cap) return;
-  int lev = lone, c_l = 0, base = 0;
-  for (int l = 0; l <= lone; ++l) base += T.sb->level_cnt[l];  // nodes of the levels up to lev
+  int lev = lone, c_l = 0;
   int first = 0, next = 1, parts = 1;  // the level's first part, the next level's, their number
   int ready = 0;
-  for (bool any = false;; any = true) {
-    const int part = next_part(W.sb, any);
+  for (;; finish_part(W.sb), part = take_part(W.sb)) {
+    part = share_part(part);
     while (part >= next) {
       if (++lev == kLevels) return;
       c_l = T.sb->level_cnt[lev];
@@ -79,6 +86,7 @@ __global__ void __launch_bounds__(kDownThreads) k_adj_down(TreeDev T, AdjWs W, d
     if (lev > lone) {
       for (int s = (part - first) * kDownThreads + threadIdx.x; s < c_l; s += parts * kDownThreads)
         push_down(T, W, base - c_l + s, invL);
+      if (base == total) return;  // the last level: nobody waits for it, and no block needs two of its parts
       continue;
     }
     int p = threadIdx.x;
@@ -89,6 +97,7 @@ __global__ void __launch_bounds__(kDownThreads) k_adj_down(TreeDev T, AdjWs W, d
       __threadfence_block();
       __syncthreads();
     }
+    if (base == total) return;
   }
 }
 

@@ -36,7 +36,7 @@ struct StatusBlock {
   uint32_t status;
   uint32_t magic;
   int32_t level_cnt[24];              // nodes per level (tree buffers)
-  unsigned long long counter;         // finished parts of a launch (next_part)
+  unsigned long long counter;         // finished parts of a launch (take_part)
   unsigned long long work;            // taken parts
   int32_t pad[20];
 };
@@ -263,27 +263,30 @@ __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long lon
   return v;
 }
 
-// The next part of this block, after it has finished the one before (any).
-// Every thread of the block calls it, and wait_parts.
-__device__ __forceinline__ int next_part(StatusBlock* sb, bool any) {
+// The next part of this block (thread 0's number), and every thread's copy of it.
+__device__ __forceinline__ int take_part(StatusBlock* sb) {
+  return threadIdx.x == 0 ? (int)atomicAdd(&sb->work, 1ull) : 0;
+}
+__device__ __forceinline__ int share_part(int part) {
   __shared__ int s_part;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    if (any) {
-      __threadfence();
-      atomicAdd(&sb->counter, 1ull);
-    }
-    s_part = (int)atomicAdd(&sb->work, 1ull);
-  }
+  if (threadIdx.x == 0) s_part = part;
   __syncthreads();
   return s_part;
+}
+// The block's part is finished.
+__device__ __forceinline__ void finish_part(StatusBlock* sb) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&sb->counter, 1ull);
+  }
 }
 // Parts of a level of c_l nodes, one a block at most; part i takes the nodes from
 // i * threads on in strides of all parts' threads.
 __device__ __forceinline__ int level_parts(int c_l, int threads) {
   return min((c_l + threads - 1) / threads, (int)gridDim.x);
 }
-// Until n parts are finished; false if that took too long.
+// Until n parts are finished; false if that took too long.  Every thread calls it.
 __device__ __forceinline__ bool wait_parts(const StatusBlock* sb, int n) {
   __shared__ int s_ok;
   if (threadIdx.x == 0) {

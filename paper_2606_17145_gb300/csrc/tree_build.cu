@@ -533,22 +533,26 @@ __device__ __forceinline__ void node_moments(const TreeDev& T, const BoxScale& B
   write_moments(T, B, p, D, M, S0, S1, S2, __longlong_as_double(Hb));
 }
 
-// The split nodes, from the deepest level up, in parts (next_part) of
+// The split nodes, from the deepest level up, in parts (take_part) of
 // nodes of one level.  The last part is the levels from the root on that have at
 // most kUpThreads nodes each.
 __global__ void __launch_bounds__(kUpThreads) k_upward(TreeDev T, BoxScale B) {
+  int part = take_part(T.sb);  // on its way while the levels are read
+  int cnt[kLevels];
+#pragma unroll
+  for (int l = 0; l < kLevels; ++l) cnt[l] = T.sb->level_cnt[l];
   int total = 0, lone = -1;
+#pragma unroll
   for (int l = 0; l < kLevels; ++l) {
-    const int c = T.sb->level_cnt[l];
-    total += c;
-    if (lone == l - 1 && c <= kUpThreads) lone = l;
+    total += cnt[l];
+    if (lone == l - 1 && cnt[l] <= kUpThreads) lone = l;
   }
   if (total > T.cap) return;  // flagged by k_fill
   int l = kLevels - 1, c_l = T.sb->level_cnt[l], base = total - c_l, parts = level_parts(c_l, kUpThreads);
   int first = 0;  // the level's first part: as many belong to the levels below
   int ready = 0;
-  for (bool any = false;; any = true) {
-    const int part = next_part(T.sb, any);
+  for (;; finish_part(T.sb), part = take_part(T.sb)) {
+    part = share_part(part);
     while (l > lone && part - first >= parts) {
       first += parts;
       c_l = T.sb->level_cnt[--l];
