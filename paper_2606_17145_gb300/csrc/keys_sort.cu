@@ -213,8 +213,18 @@ __global__ void __launch_bounds__(kKeyThreads) k_keys(const double* __restrict__
 }
 
 // A tile's published state for one digit: 0 nothing yet, 1 + count its own
-// count, kStateSum | sum the keys of the digit in all tiles up to it.
+// count, kStateSum | sum the keys of the digit in all tiles up to it.  One
+// word that other blocks poll while it is written, hence relaxed accesses of
+// device scope; nothing else is read on the strength of it.
 constexpr uint32_t kStateSum = 1u << 31;
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 // Polls of one state before a look-back gives up (seconds, far above any
 // tile's run time; the tiles looked at are always running).
 constexpr int kStatePolls = 1 << 22;
@@ -290,7 +300,7 @@ __global__ void __launch_bounds__(kSortThreads, ITEMS == 16 ? 3 : 6)
     }
     own = ((unsigned long long)cnt << 32) | all;
     if (d == 255) cnt -= (uint32_t)(kTile - tile_n);  // less the padding
-    __stcg(&state[tile * 256 + d], tile == 0 ? (kStateSum | cnt) : cnt + 1u);
+    st_relaxed(&state[tile * 256 + d], tile == 0 ? (kStateSum | cnt) : cnt + 1u);
     if (pass < 7) W.tile_state[(pass + 1) & 1][tile * 256 + d] = 0u;  // the next pass's
     x = own;
 #pragma unroll
@@ -331,7 +341,7 @@ __global__ void __launch_bounds__(kSortThreads, ITEMS == 16 ? 3 : 6)
         // several predecessors at a time: their loads are independent
         uint32_t st[kStateAhead];
 #pragma unroll
-        for (int u = 0; u < kStateAhead; ++u) st[u] = t - u >= 0 ? __ldcg(state + (t - u) * 256 + d) : kStateSum;
+        for (int u = 0; u < kStateAhead; ++u) st[u] = t - u >= 0 ? ld_relaxed(state + (t - u) * 256 + d) : kStateSum;
         bool done = false;
         int used = 0;
 #pragma unroll
@@ -348,7 +358,7 @@ __global__ void __launch_bounds__(kSortThreads, ITEMS == 16 ? 3 : 6)
           break;
         }
       }
-      __stcg(&state[tile * 256 + d], kStateSum | (sum + cnt));
+      st_relaxed(&state[tile * 256 + d], kStateSum | (sum + cnt));
     }
     S.base[d] = gbase + sum - tstart;
   }
