@@ -33,8 +33,8 @@ __device__ __forceinline__ void push_down(const TreeDev& T, const AdjWs& W, int 
     const double Cq[3] = {(double)QC.x, (double)QC.y, (double)QC.z};
     double CGq[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) CGq[c] = __ldcg(&W.CG[3 * (int64_t)q + c]);
-    B += __ldcg(&W.Bn[q]) - (CGq[0] * (C[0] - Cq[0]) + CGq[1] * (C[1] - Cq[1]) + CGq[2] * (C[2] - Cq[2]));
+    for (int c = 0; c < 3; ++c) CGq[c] = W.CG[3 * (int64_t)q + c];
+    B += W.Bn[q] - (CGq[0] * (C[0] - Cq[0]) + CGq[1] * (C[1] - Cq[1]) + CGq[2] * (C[2] - Cq[2]));
 #pragma unroll
     for (int c = 0; c < 3; ++c) G[c] += CGq[c];
   }
