@@ -24,8 +24,8 @@
 // all) cost 180 us on 4096 particles, most of it for empty levels.  Whole force
 // passes, build alone changed: 4096 particles 500 -> 294 us, 64^3 leapfrog step
 // 1050 -> 887 us, 100,003-particle SPH 1.15 -> 0.96 ms.  At 2.1 M particles the
-// kernels take 0.063 (permute), 0.020, 0.008, 0.077 (fill), 0.048 (leaves) and
-// 0.084 ms (upward).
+// kernels take 0.065 (permute), 0.024 (count), 0.005 (scan), 0.032 (fill), 0.049
+// (leaves) and 0.073 ms (upward).
 #include <cfloat>
 
 #include "og_internal.cuh"
@@ -49,7 +49,8 @@ namespace og {
 // the FP64 walk, where the pairs are nearly all of the work, the count alone
 // tells more (clustered 64^3 7.6 / 6.5 / 6.8 ms, 7.7 with the volume).  Whole
 // octaves: zoom 13.7 ms; other powers of the volume from 0.2 to 0.3: zoom
-// 14.0 - 12.3, 90^3 3.50 - 3.69.  The orders cost the build 4 us at 2.1 M.
+// 14.0 - 12.3, 90^3 3.50 - 3.69.  (Every tile adding up all tiles' counts again
+// made k_scan 0.32 ms of a 60 M-particle build; with their prefix sums 0.08.)
 
 // Counts the particles per cell (consecutive particles of a cell together) and
 // leaves each group's box volume in T.gorder.  Every lane of the warp calls it.
@@ -114,50 +115,62 @@ __device__ __forceinline__ void group_buckets(const TreeDev& T, int64_t block) {
   }
 }
 
+// The buckets [32 q, 32 q + 32) of order o: their counts in the tiles before each
+// tile, and in all (1024 threads: a warp's lanes are the buckets, its rows a
+// 32nd of the tiles).
+__device__ __forceinline__ void bucket_columns(const TreeDev& T, int o, int q) {
+  __shared__ int s_sum[32][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int* col = T.gtile[o] + 32 * q + lane;
+  const int64_t rows = (T.ntiles + 31) / 32;
+  const int64_t t0 = min(w * rows, T.ntiles), t1 = min(t0 + rows, T.ntiles);
+  int sum = 0;
+#pragma unroll 8
+  for (int64_t t = t0; t < t1; ++t) sum += col[t * kBuckets];
+  s_sum[w][lane] = sum;
+  __syncthreads();
+  int at = 0;
+  for (int ww = 0; ww < w; ++ww) at += s_sum[ww][lane];
+  for (int64_t t = t0; t < t1; t += 8) {
+    int c[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) c[u] = t + u < t1 ? col[(t + u) * kBuckets] : 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (t + u < t1) col[(t + u) * kBuckets] = at;
+      at += c[u];
+    }
+  }
+  if (w == 31) col[T.ntiles * kBuckets] = at;
+}
+
 // Order o of one tile's groups, kOrderTile threads.
 __device__ __forceinline__ void group_places(const TreeDev& T, int64_t tile, int o) {
   __shared__ int s_at[kOrderTile / 32][kBuckets];
   __shared__ int s_base[kBuckets];
-  __shared__ int s_part[2][kOrderTile / kBuckets][kBuckets];  // all tiles, the tiles before this one
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  {
-    const int b = threadIdx.x % kBuckets, q = threadIdx.x / kBuckets;
-    int all = 0, before = 0;
-    for (int64_t t = q; t < T.ntiles; t += kOrderTile / kBuckets) {
-      const int c = T.gtile[o][t * kBuckets + b];
-      all += c;
-      if (t < tile) before += c;
-    }
-    s_part[0][q][b] = all;
-    s_part[1][q][b] = before;
 #pragma unroll
-    for (int i = lane; i < kBuckets; i += 32) s_at[w][i] = 0;
-  }
-  __syncthreads();
+  for (int i = lane; i < kBuckets; i += 32) s_at[w][i] = 0;
   const int64_t g = tile * kOrderTile + threadIdx.x;
   const int bucket = g < T.ngroups ? T.gbucket[o][g] : -1;
-  const uint32_t peers = __match_any_sync(0xffffffffu, bucket);
-  if (bucket >= 0 && lane == __ffs(peers) - 1) s_at[w][bucket] = __popc(peers);
   if (w == 0) {  // exclusive scan of the buckets' totals, 4 a lane
-    int tot[kBuckets / 32], sum = 0;
-#pragma unroll
-    for (int i = 0; i < kBuckets / 32; ++i) {
-      tot[i] = sum;
-      for (int q = 0; q < kOrderTile / kBuckets; ++q) sum += s_part[0][q][lane * (kBuckets / 32) + i];
-    }
+    const int4 c = reinterpret_cast<const int4*>(T.gtile[o] + T.ntiles * kBuckets)[lane];
+    const int sum = c.x + c.y + c.z + c.w;
     int x = sum;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, x, d);
       if (lane >= d) x += y;
     }
-#pragma unroll
-    for (int i = 0; i < kBuckets / 32; ++i) s_base[lane * (kBuckets / 32) + i] = x - sum + tot[i];
+    x -= sum;
+    reinterpret_cast<int4*>(s_base)[lane] = make_int4(x, x + c.x, x + c.x + c.y, x + c.x + c.y + c.z);
   }
   __syncthreads();
+  const uint32_t peers = __match_any_sync(0xffffffffu, bucket);
+  if (bucket >= 0 && lane == __ffs(peers) - 1) s_at[w][bucket] = __popc(peers);
+  __syncthreads();
   if (threadIdx.x < kBuckets) {
-    int at = s_base[threadIdx.x];
-    for (int q = 0; q < kOrderTile / kBuckets; ++q) at += s_part[1][q][threadIdx.x];
+    int at = s_base[threadIdx.x] + T.gtile[o][tile * kBuckets + threadIdx.x];
     for (int i = 0; i < kOrderTile / 32; ++i) {
       const int c = s_at[i][threadIdx.x];
       s_at[i][threadIdx.x] = at;
@@ -227,32 +240,47 @@ __device__ __forceinline__ int common_digits(uint64_t a, uint64_t b) {
 }
 
 // Levels [lo, hi] of the nodes that start at sorted key i of this block (none
-// if lo > hi); deep: the deepest level whose run around i is split (-1: none).
-// Every thread of the block calls it.
+// if lo > hi): all but the one at hi are split.  Every thread of the block calls
+// it.  LEAF: leaf_size, or 0 for any.
+template <int LEAF>
 __device__ __forceinline__ void node_levels(const uint64_t* __restrict__ keys, int64_t n, int leaf_size, int64_t i0,
-                                            signed char* s_far, int& lo, int& hi, int& deep) {
-  // s_far[j]: digits shared by keys i0 - leaf_size + j and i0 + j
-  for (int j = threadIdx.x; j < kTopoThreads + leaf_size; j += kTopoThreads) {
-    const int64_t a = i0 - leaf_size + j, b = i0 + j;
-    s_far[j] = (signed char)(a >= 0 && b < n ? common_digits(keys[a], keys[b]) : -1);
+                                            short* s_far, int& lo, int& hi) {
+  const int leaf = LEAF ? LEAF : leaf_size;
+  // s_far[j]: digits shared by keys i0 - leaf + j and i0 + j
+  for (int j = threadIdx.x; j < kTopoThreads + leaf; j += kTopoThreads) {
+    const int64_t a = i0 - leaf + j, b = i0 + j;
+    s_far[j] = (short)(a >= 0 && b < n ? common_digits(keys[a], keys[b]) : -1);
   }
   __syncthreads();
   const int64_t i = i0 + threadIdx.x;
   lo = 1;
   hi = 0;
-  deep = -1;
   if (i < n) {
-    for (int j = 0; j <= leaf_size; ++j) deep = max(deep, (int)s_far[threadIdx.x + j]);
+    // two at a time from the even place on; those outside the window, one on
+    // either side at most, are left out of the first and the last pair
+    const uint32_t* f = reinterpret_cast<const uint32_t*>(s_far) + (threadIdx.x >> 1);
+    const int odd = threadIdx.x & 1, last = (odd + leaf) >> 1;
+    uint32_t m = odd ? f[0] | 0x0000ffffu : f[0];
+    if (last > 0) {
+#pragma unroll
+      for (int j = 1; j < last; ++j) m = __vmaxs2(m, f[j]);
+      m = __vmaxs2(m, (odd + leaf) & 1 ? f[last] : f[last] | 0xffff0000u);
+    } else if (((odd + leaf) & 1) == 0) {
+      m |= 0xffff0000u;
+    }
+    const int deep = max((int)(short)(m & 0xffffu), (int)(short)(m >> 16));
     lo = i == 0 ? 0 : common_digits(keys[i - 1], keys[i]) + 1;
     hi = min(deep + 1, kMaxLevel);
   }
-  deep = min(deep, kMaxLevel - 1);
 }
 
-// Nodes of each level that start in this block's keys.  The blocks after those
-// of the keys find the groups' buckets.
+// Nodes of each level that start in this block's keys.  The levels of each key's
+// go to T.leaf_of (until k_leaves fills it), which saves k_fill from finding
+// them again (16.8 M keys, us: k_fill 447 -> 352).  The blocks after those of
+// the keys find the groups' buckets.
+template <int LEAF>
 __global__ void __launch_bounds__(kTopoThreads) k_count(TreeDev T, const uint64_t* __restrict__ keys, int leaf_size) {
-  __shared__ signed char s_far[kTopoThreads + kMaxLeaf];
+  __shared__ __align__(4) short s_far[kTopoThreads + kMaxLeaf + 2];
   __shared__ int s_cnt[kLevels];
   if (blockIdx.x >= T.nblk) {
     group_buckets(T, blockIdx.x - T.nblk);
@@ -260,9 +288,10 @@ __global__ void __launch_bounds__(kTopoThreads) k_count(TreeDev T, const uint64_
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) T.sb->magic = kMagicTree;
   if (threadIdx.x < kLevels) s_cnt[threadIdx.x] = 0;
-  int lo, hi, deep;
+  int lo, hi;
   const int64_t i0 = blockIdx.x * (int64_t)kTopoThreads, i = i0 + threadIdx.x;
-  node_levels(keys, T.n, leaf_size, i0, s_far, lo, hi, deep);
+  node_levels<LEAF>(keys, T.n, leaf_size, i0, s_far, lo, hi);
+  if (i < T.n) T.leaf_of[i] = lo | hi << 8;
   // All that follows holds for sorted keys.  Of others the nodes' ranges still
   // lie inside the particles, but a node may be nobody's child.
   if (i > 0 && i < T.n && keys[i - 1] > keys[i]) set_status(T.sb, ST_TREELINK);
@@ -272,21 +301,28 @@ __global__ void __launch_bounds__(kTopoThreads) k_count(TreeDev T, const uint64_
 }
 
 // One block per level: exclusive scan of its counts over the blocks, in
-// place, and the level's total.  The blocks after those write the walks' orders
-// of the groups, one tile in one order each.
-__global__ void __launch_bounds__(1024) k_scan(TreeDev T) {
+// place, and the level's total.  The blocks after those do the same for the
+// buckets of the groups.
+constexpr int kScanThreads = 1024;
+constexpr int kScanItems = 8;
+constexpr int kScanBlocks = kLevels + 2 * (kBuckets / 32);
+__global__ void __launch_bounds__(kScanThreads) k_scan(TreeDev T) {
   __shared__ int s_w[32];
   if (blockIdx.x >= kLevels) {
-    group_places(T, (blockIdx.x - kLevels) >> 1, (blockIdx.x - kLevels) & 1);
+    bucket_columns(T, (blockIdx.x - kLevels) & 1, (blockIdx.x - kLevels) >> 1);
     return;
   }
   int* row = T.blk + blockIdx.x * T.nblk;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int carry = 0;
-  for (int64_t b0 = 0; b0 < T.nblk; b0 += 1024) {
-    const int64_t i = b0 + threadIdx.x;
-    const int v = i < T.nblk ? row[i] : 0;
-    int x = v;
+  for (int64_t b0 = 0; b0 < T.nblk; b0 += kScanThreads * kScanItems) {
+    const int64_t i = b0 + threadIdx.x * kScanItems;
+    int v[kScanItems], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) v[k] = i + k < T.nblk ? row[i + k] : 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) sum += v[k];
+    int x = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, x, o);
@@ -294,12 +330,19 @@ __global__ void __launch_bounds__(1024) k_scan(TreeDev T) {
     }
     if (lane == 31) s_w[w] = x;
     __syncthreads();
-    int before = 0, all = 0;
-    for (int ww = 0; ww < 32; ++ww) {
-      if (ww < w) before += s_w[ww];
-      all += s_w[ww];
+    int y = s_w[lane];  // the warps' sums, then those up to each warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int z = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= o) y += z;
     }
-    if (i < T.nblk) row[i] = carry + before + x - v;
+    const int before = __shfl_sync(0xffffffffu, y, (w + 31) & 31), all = __shfl_sync(0xffffffffu, y, 31);
+    int at = carry + (w > 0 ? before : 0) + x - sum;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+      if (i + k < T.nblk) row[i + k] = at;
+      at += v[k];
+    }
     carry += all;
     __syncthreads();
   }
@@ -312,100 +355,140 @@ __device__ __forceinline__ int level_base(const StatusBlock* sb, int level) {
   return b;
 }
 
-// Writes the nodes' ranges.  nchild and the parent links follow with the
-// moments, where a node meets its children.
-__global__ void __launch_bounds__(kTopoThreads) k_fill(TreeDev T, const uint64_t* __restrict__ keys, int leaf_size) {
-  __shared__ signed char s_far[kTopoThreads + kMaxLeaf];
-  __shared__ uint32_t s_ends[kLevels][kTopoThreads / 32];  // keys at which a run of the level (and a node) starts
-  __shared__ int s_first[kLevels];                      // index of this block's first node of each level
-  __shared__ int s_warp[kTopoThreads / 32][kLevels];    // nodes of each level in each warp, then in the warps before it
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (threadIdx.x < kLevels) {
-    s_first[threadIdx.x] = level_base(T.sb, threadIdx.x) + T.blk[threadIdx.x * T.nblk + blockIdx.x];
-#pragma unroll
-    for (int ww = 0; ww < kTopoThreads / 32; ++ww) s_warp[ww][threadIdx.x] = 0;
+// First key from `end` on whose prefix is not pre (n if there is none), by a
+// whole warp: probes at distances that double, then 32 at a time between the
+// last one inside the run and the first outside it.
+__device__ __forceinline__ int64_t run_end(const uint64_t* __restrict__ keys, int64_t n, int64_t end, uint64_t pre,
+                                           int shift) {
+  const int lane = threadIdx.x & 31;
+  auto inside = [&](int64_t j) {  // how many of the lanes' probes, from the first on
+    return __ffs(~__ballot_sync(0xffffffffu, j < n && (keys[j] >> shift) == pre)) - 1;
+  };
+  int in = inside(end + ((int64_t)1 << lane) - 1);
+  if (in < 0) in = 32;
+  if (in == 0) return end;
+  // the run ends in [a, b]
+  int64_t a = end + ((int64_t)1 << (in - 1)), b = min(n, end + ((int64_t)1 << in) - 1);
+  while (a < b) {
+    const int64_t step = (b - a + 31) >> 5;
+    const int64_t j = a + lane * step;
+    in = inside(j < b ? j : n);
+    if (in < 0) in = 32;
+    b = min(b, a + in * step);
+    if (in > 0) a += (in - 1) * step + 1;
   }
-  int lo, hi, deep;
+  return a;
+}
+
+// Writes the nodes' ranges.  nchild and the parent links follow with the
+// moments, where a node meets its children.  A warp lists the nodes that start
+// at its 32 keys and takes 32 of them at a time: going through the levels with a
+// lane per key left 3 lanes of 32 at work (16.8 M keys, us: 352 -> 314).  Runs that
+// go on past the block are searched for by whole warps, a level each (314 -> 279,
+// 259 with the levels' counts read once).
+// The blocks after those of the keys write the walks' orders of the groups, one
+// tile in one order each.
+__global__ void __launch_bounds__(kTopoThreads) k_fill(TreeDev T, const uint64_t* __restrict__ keys) {
+  constexpr int kWarps = kTopoThreads / 32;
+  __shared__ uint32_t s_ends[kWarps][kLevels];  // keys at which a run of the level (and a node) starts
+  __shared__ uint32_t s_here[kWarps][kLevels];  // keys at which a node of the level starts (the warp's levels)
+  __shared__ int s_warp[kWarps][kLevels];       // their number, then the index of the warp's first
+  __shared__ uint16_t s_list[kWarps][32];       // nodes: lane of the key | level << 8
+  __shared__ int s_past[kLevels];               // where the level's last run in the block ends
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (blockIdx.x >= T.nblk) {
+    group_places(T, (blockIdx.x - T.nblk) >> 1, (blockIdx.x - T.nblk) & 1);
+    return;
+  }
   const int64_t i0 = blockIdx.x * (int64_t)kTopoThreads, i = i0 + threadIdx.x;
-  node_levels(keys, T.n, leaf_size, i0, s_far, lo, hi, deep);
+  const int levels = i < T.n ? T.leaf_of[i] : 1;  // lowest level 1, highest 0: none
+  const int c_l = lane < kLevels ? T.sb->level_cnt[lane] : 0;
+  // index of this block's first node of level threadIdx.x
+  int first = threadIdx.x < kLevels ? T.blk[threadIdx.x * T.nblk + blockIdx.x] - c_l : 0;
+  const int top = 31 - __clz((int)__ballot_sync(0xffffffffu, c_l > 0));  // the last level there is
+  if (w == 0) {
+    int x = c_l;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    first += x;
+  }
+  const int lo = levels & 255, hi = levels >> 8;
   const bool any = lo <= hi;
   const int wlo = (int)__reduce_min_sync(0xffffffffu, (unsigned)(any ? lo : kLevels));
   const int whi = (int)__reduce_max_sync(0xffffffffu, (unsigned)(any ? hi + 1 : 0)) - 1;
-  for (int l = wlo; l <= whi; ++l) {
-    const uint32_t m = __ballot_sync(0xffffffffu, l >= lo && l <= hi);
-    if (lane == 0) s_warp[w][l] = __popc(m);
-  }
-  for (int l = 1; l < kLevels; ++l) {
-    const uint32_t m = __ballot_sync(0xffffffffu, any && lo <= l);
-    if (lane == 0) s_ends[l][w] = m;
+  if (lane < kLevels) s_warp[w][lane] = 0;
+  __syncwarp();
+  for (int l = 0; l <= top; ++l) {
+    const uint32_t e = __ballot_sync(0xffffffffu, any && lo <= l);
+    if (lane == 0) s_ends[w][l] = e;
+    if (l < wlo || l > whi) continue;
+    const uint32_t h = __ballot_sync(0xffffffffu, l >= lo && l <= hi);
+    if (lane == 0) {
+      s_here[w][l] = h;
+      s_warp[w][l] = __popc(h);
+    }
   }
   __syncthreads();
   if (threadIdx.x < kLevels) {
-    int run = s_first[threadIdx.x];
 #pragma unroll
-    for (int ww = 0; ww < kTopoThreads / 32; ++ww) {
+    for (int ww = 0; ww < kWarps; ++ww) {
       const int c = s_warp[ww][threadIdx.x];
-      s_warp[ww][threadIdx.x] = run;
-      run += c;
+      s_warp[ww][threadIdx.x] = first;
+      first += c;
     }
   }
+  // the runs that go on past the block, a warp a level
+  const int64_t past = min(i0 + kTopoThreads, T.n);
+  for (int l = w + 1; l <= top; l += kWarps) {
+    const bool starts = __any_sync(0xffffffffu, lane < kWarps && s_ends[lane & (kWarps - 1)][l] != 0u);
+    if (!starts) continue;  // none of its nodes starts here
+    const int64_t e = run_end(keys, T.n, past, keys[past - 1] >> (63 - 3 * l), 63 - 3 * l);
+    if (lane == 0) s_past[l] = (int)e;
+  }
+  const int cnt = any ? hi - lo + 1 : 0;
+  int off = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, off, o);
+    if (lane >= o) off += y;
+  }
+  const int nodes = __shfl_sync(0xffffffffu, off, 31);
+  off -= cnt;
   __syncthreads();
-  // deepest level first: a node's run lies inside its parent's, so the end
-  // found for one level is where the search for the next one up begins
-  int64_t end = i + 1;
-  int below = -1;  // index of this key's node one level down
-  for (int l = whi; l >= wlo; --l) {
-    const bool here = l >= lo && l <= hi;
-    const uint32_t m = __ballot_sync(0xffffffffu, here);
-    if (!here) continue;
-    const int64_t p = (int64_t)s_warp[w][l] + __popc(m & ((1u << lane) - 1u));
-    if (l == 0) {
-      end = T.n;
-    } else {
+  for (int b = 0; b < nodes; b += 32) {
+    for (int k = max(b - off, 0); k < min(cnt, b + 32 - off); ++k)
+      s_list[w][off + k - b] = (uint16_t)(lane | (lo + k) << 8);
+    __syncwarp();
+    const int e = b + lane < nodes ? s_list[w][lane] : 0;
+    const int at = e & 31, l = e >> 8;  // key and level of this lane's node
+    const bool leaf = l == __shfl_sync(0xffffffffu, hi, at);
+    __syncwarp();
+    if (b + lane >= nodes) break;
+    const int64_t ki = i0 + 32 * w + at;
+    const uint32_t before = (1u << at) - 1u;
+    const int64_t p = (int64_t)s_warp[w][l] + __popc(s_here[w][l] & before);
+    int64_t end = T.n;
+    if (l > 0) {
       // The run ends at the next key that starts a run of level l.  A node
       // starts there too: the two keys' deepest common node is split, so the
       // first level at which they differ has one.  In this block the starts
-      // are in s_ends; past it the end is searched for.
-      const int shift = 63 - 3 * l;
-      const uint64_t pre = keys[i] >> shift;
-      int64_t step = 1;
+      // are in s_ends.
       int ww = w;
-      uint32_t next = lane < 31 ? s_ends[l][w] & (0xfffffffeu << lane) : 0u;
-      while (next == 0u && ++ww < kTopoThreads / 32) next = s_ends[l][ww];
-      if (next) {
-        end = i0 + 32 * ww + __ffs(next) - 1;
-        step = 0;
-      } else {
-        end = max(end, min(i0 + kTopoThreads, T.n));
-      }
-      while (step > 0 && end < T.n && (keys[end] >> shift) == pre) {
-        const int64_t probe = end + step;
-        if (probe < T.n && (keys[probe] >> shift) == pre) {
-          end = probe + 1;
-          step <<= 1;
-        } else if (step > 1) {
-          // the run ends in (end, probe]
-          int64_t a = end + 1, b = probe < T.n ? probe : T.n;
-          while (a < b) {
-            const int64_t mid = (a + b) >> 1;
-            if ((keys[mid] >> shift) == pre) a = mid + 1;
-            else b = mid;
-          }
-          end = a;
-          break;
-        } else {
-          ++end;
-        }
-      }
+      uint32_t next = at < 31 ? s_ends[w][l] & (0xfffffffeu << at) : 0u;
+      while (next == 0u && ++ww < kWarps) next = s_ends[ww][l];
+      end = next ? i0 + 32 * ww + __ffs(next) - 1 : s_past[l];
     }
     if (p < T.cap) {
-      const bool leaf = l > deep;
-      T.nD[p] = make_int4((int)i, (int)(end - i), leaf ? -1 : below, make_meta(0, l, leaf));
+      // the first child starts at the same key, one level down
+      const int child = leaf ? -1 : s_warp[w][l + 1] + __popc(s_here[w][l + 1] & before);
+      T.nD[p] = make_int4((int)ki, (int)(end - ki), child, make_meta(0, l, leaf));
       if (l == 0) T.nParent[p] = -1;
     } else {
       set_status(T.sb, ST_NOSPACE);
     }
-    below = (int)p;
   }
 }
 
@@ -509,11 +592,11 @@ __device__ __forceinline__ void node_moments(const TreeDev& T, const BoxScale& B
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     const int64_t q = D.z + (c < nch ? c : 0);
-    m8[c] = __ldcg(&T.mass64[q]);
-    s8[0][c] = __ldcg(&T.S64[3 * q]);
-    s8[1][c] = __ldcg(&T.S64[3 * q + 1]);
-    s8[2][c] = __ldcg(&T.S64[3 * q + 2]);
-    h8[c] = __ldcg(&T.hmax64[q]);
+    m8[c] = T.mass64[q];
+    s8[0][c] = T.S64[3 * q];
+    s8[1][c] = T.S64[3 * q + 1];
+    s8[2][c] = T.S64[3 * q + 2];
+    h8[c] = T.hmax64[q];
   }
   double M = 0.0, S0 = 0.0, S1 = 0.0, S2 = 0.0;
   long long Hb = 0;
@@ -537,6 +620,8 @@ __device__ __forceinline__ void node_moments(const TreeDev& T, const BoxScale& B
 // nodes of one level.  The last part is the levels from the root on that have at
 // most kUpThreads nodes each.
 __global__ void __launch_bounds__(kUpThreads) k_upward(TreeDev T, BoxScale B) {
+  __shared__ int s_split[kUpThreads / 32][64];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int part = take_part(T.sb);  // on its way while the levels are read
   int cnt[kLevels];
 #pragma unroll
@@ -568,8 +653,24 @@ __global__ void __launch_bounds__(kUpThreads) k_upward(TreeDev T, BoxScale B) {
       ready = first;
     }
     if (l > lone) {
-      for (int s = (part - first) * kUpThreads + threadIdx.x; s < c_l; s += parts * kUpThreads)
-        node_moments(T, B, base + s, l, total);
+      // a warp collects split nodes until there is one for every lane: taken as
+      // they come, one lane in eight is at work, and FP64 instructions cost the
+      // same for it (16.8 M clustered particles, us: 430 -> 358)
+      int have = 0;
+      for (int s0 = (part - first) * kUpThreads + (threadIdx.x & ~31); s0 < c_l; s0 += parts * kUpThreads) {
+        const int s = s0 + lane;
+        const bool split = s < c_l && !meta_leaf(T.nD[base + s].w);
+        const uint32_t m = __ballot_sync(0xffffffffu, split);
+        if (split) s_split[w][have + __popc(m & ((1u << lane) - 1u))] = base + s;
+        have += __popc(m);
+        __syncwarp();
+        if (have >= 32) {
+          have -= 32;
+          node_moments(T, B, s_split[w][have + lane], l, total);
+          __syncwarp();
+        }
+      }
+      if (lane < have) node_moments(T, B, s_split[w][lane], l, total);
       continue;
     }
     for (;;) {
@@ -590,9 +691,11 @@ cudaError_t launch_tree_build(const BuildArgs& A, cudaStream_t s) {
   const BoxScale B = box_scale(A.L);
   k_permute<<<(unsigned)grid, 256, 0, s>>>(A, B);
   const int64_t gblocks = (4 * T.ngroups + kTopoThreads - 1) / kTopoThreads;
-  k_count<<<(unsigned)(T.nblk + gblocks), kTopoThreads, 0, s>>>(T, A.keys, A.leaf_size);
-  k_scan<<<(unsigned)(kLevels + 2 * T.ntiles), kOrderTile, 0, s>>>(T);
-  k_fill<<<(unsigned)T.nblk, kTopoThreads, 0, s>>>(T, A.keys, A.leaf_size);
+  const unsigned cblocks = (unsigned)(T.nblk + gblocks);
+  if (A.leaf_size == 16) k_count<16><<<cblocks, kTopoThreads, 0, s>>>(T, A.keys, 16);  // the default
+  else k_count<0><<<cblocks, kTopoThreads, 0, s>>>(T, A.keys, A.leaf_size);
+  k_scan<<<kScanBlocks, kScanThreads, 0, s>>>(T);
+  k_fill<<<(unsigned)(T.nblk + 2 * T.ntiles), kTopoThreads, 0, s>>>(T, A.keys);
   // the node counts live on the device: grids are sized for the particles
   int64_t lgrid = (T.n / 2 + 255) / 256;
   if (lgrid > grid_cap(8)) lgrid = grid_cap(8);

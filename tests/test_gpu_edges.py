@@ -99,6 +99,46 @@ def test_keys_by_table_and_by_bits(axis):
     assert torch.equal(keys, parts.sort().values)
 
 
+def _nodes_of(keys, leaf):
+    """The nodes over sorted keys, level by level in key order, by their definition."""
+    n = keys.shape[0]
+    first, count, parent = np.array([0]), np.array([n]), np.array([-1])
+    out, base = [], 0
+    for level in range(22):
+        split = (count > leaf) & (level < 21)
+        out.append([np.full_like(first, level), first, count, parent, split])
+        if not split.any():
+            break
+        pre = keys >> np.uint64(63 - 3 * (level + 1))
+        starts = np.flatnonzero(np.concatenate([[True], pre[1:] != pre[:-1]]))
+        ends = np.concatenate([starts[1:], [n]])
+        own = np.searchsorted(first, starts, "right") - 1  # the node of this level that a run may lie in
+        keep = (own >= 0) & split[own] & (starts < first[own] + count[own])
+        parent = base + own[keep]
+        base += first.shape[0]
+        first, count = starts[keep], (ends - starts)[keep]
+    level, first, count, parent, split = (np.concatenate([o[i] for o in out]) for i in range(5))
+    nchild = np.bincount(parent[1:], minlength=level.shape[0])
+    child = np.full(level.shape[0], -1)
+    child[parent[1:][::-1]] = np.arange(1, level.shape[0])[::-1]
+    return dict(level=level, first=first, count=count, parent=parent, nchild=nchild, child_first=child)
+
+
+@pytest.mark.parametrize("n,leaf,clumps", [(511, 16, 0), (5000, 1, 7), (40_000, 1, 0), (40_000, 32, 5), (70_001, 15, 3),
+                                           (70_001, 16, 3), (512 * 1024 + 17, 16, 0), (4_300_000, 16, 2)])
+def test_nodes_of_many_blocks(n, leaf, clumps):
+    """Node ranges and links over the blocks of the topology passes, runs that
+    span many of them, up to more blocks than one step of their scan takes."""
+    dev = device()
+    m = og()
+    pos, mass, eps = _case(n, n + leaf, clumps)
+    p, mt, e = (torch.tensor(x, dtype=torch.float64, device=dev) for x in (pos, mass, eps))
+    keys, order = m.keys_sort(p, 1.0)
+    got = m.tree_build(keys, order, p, mt, e, 1.0, p=m.params(leaf_size=leaf, node_capacity=4 * n + 1024)).nodes()
+    for k, v in _nodes_of(keys.cpu().numpy().view(np.uint64), leaf).items():
+        assert np.array_equal(got[k].cpu().numpy(), v), k
+
+
 @pytest.mark.parametrize("n", [31, 1024 * 32 - 1, 3 * 1024 * 32 + 1])
 def test_orders_hold_every_group(n):
     """The walks' orders of the groups (tiles of 1024 groups, buckets of
