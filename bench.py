@@ -724,7 +724,7 @@ def main():
                 "frac_measured": dk["frac_fp32_measured"], "frac_xu": dk["frac_xu"],
                 "measured_peaks": peaks, "kernels": kern}
 
-    launches = og.LAUNCHES_PER_CALL
+    launches = og.launches_per_call(n)
     per_step_launches = (launches["keys_sort"] + launches["tree_build"] + launches["accel"] +
                          launches["adjoint"])
 

@@ -22,11 +22,18 @@ from . import _native as N
 
 _lib = None
 
-# Kernels libog.so launches per call (fixed sequences, see csrc/): keys (1) +
-# 8 radix passes; permute + count + scan + fill + leaves + upward; one walk;
-# adjoint walk + push-down + the particle gather; SPH radius + density.
+# Kernels libog.so launches per call (see csrc/): keys + 8 radix passes (for more
+# than 16,384 keys, launches_per_call below); permute + count + scan + fill +
+# leaves + upward; one walk; adjoint walk + push-down + the particle gather; SPH
+# radius + density.
 LAUNCHES_PER_CALL = {"keys_sort": 1 + 8, "tree_build": 6, "accel": 1, "adjoint": 3,
                      "pm": 3, "kick": 1, "drift": 1, "sph": 2}  # pm: deposit, Green, interpolation (plus cuFFT's kernels)
+
+
+def launches_per_call(n: int) -> dict:
+    """Kernels launched per call for n particles."""
+    few = {"keys_sort": 2} if n <= 16384 else {}  # keys, sort by counting
+    return {**LAUNCHES_PER_CALL, **few}
 
 
 def lib():
