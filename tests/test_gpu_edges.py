@@ -294,3 +294,63 @@ def test_pm_mesh_sides(N):
     scale = ref.square().sum(1).mean().sqrt()
     plan.close()
     assert float(d.square().mean().sqrt() / scale) < 5e-6 and float(d.max() / scale) < 5e-5
+
+
+def _fp64_case(rcut, side, seed, n=400):
+    """Particles in a box of the given side whose mean spacing is far below the
+    cut of rcut times r_s, which stays below half the box."""
+    rng = np.random.default_rng(seed)
+    return rng.random((n, 3)) * side, 0.5 + rng.random(n), np.full(n, 0.01 * side), 0.45 * side / rcut
+
+
+@pytest.mark.parametrize("rcut,side", [(6.0, 1.0), (8.0, 1.0), (8.0, 50.0), (4.5, 2.0 ** 60), (4.5, 2.0 ** -60)])
+def test_fp64_walk_beyond_its_table(orc, rcut, side):
+    """The FP64 pair force where the short-range factor's table ends (u = 2.25, a
+    cut of 4.5 r_s) and CUDA's functions take over, and in boxes whose squared
+    distances leave the range of the reciprocal root's FP32 start.  Bound of
+    test_sort_tree_and_walks."""
+    dev = device()
+    m = og()
+    pos, mass, eps, r_s = _fp64_case(rcut, side, int(rcut * 10))
+    p, mt, e = (torch.tensor(x, dtype=torch.float64, device=dev) for x in (pos, mass, eps))
+    keys, order = m.keys_sort(p, side)
+    tree = m.tree_build(keys, order, p, mt, e, side, p=m.params(rcut_factor=rcut))
+    acc, _, c = m.shortrange_accel(tree, r_s, 0.5, prec="fp64", counts=True)
+    ref, cnt = orc.Tree(pos, mass, 2.8 * eps, box=side).walk(r_s, rcut * r_s, 0.5)
+    assert np.array_equal(c.cpu().numpy(), cnt)
+    if rcut > 4.5:  # pairs on both sides of the table's end
+        d = np.abs(pos[:, None] - pos[None])
+        d = np.minimum(d, side - d)
+        u = np.sqrt((d ** 2).sum(2)) / (2 * r_s)
+        assert (np.abs(u - 2.25) < 0.05).sum() > 20 and ((u > 2.3) & (u < rcut / 2)).sum() > 100
+    assert np.abs(acc.cpu().numpy() - ref).max() <= 1e-13 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n,N", [(500, 16), (30_000, 48)])
+def test_stepper_in_a_graph(n, N):
+    """A captured step (the mesh's fork and join become branches of the graph)
+    replayed gives the states of uncaptured steps, whose mesh sums its deposits
+    in any order: a few FP32 rounding errors of the largest force."""
+    dev = device()
+    m = og()
+    rng = np.random.default_rng(n)
+    x0 = torch.tensor(rng.random((n, 3)), dtype=torch.float64, device=dev)
+    mass = torch.full((n,), 1.0 / n, dtype=torch.float64, device=dev)
+    dt, steps = 1e-3, 3
+    S, G = (m.TreePMStepper(x0.clone(), torch.zeros_like(x0), mass, 1e-3, 1.0, 0.7 * n ** (-1 / 3), 0.5, N)
+            for _ in range(2))
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        G.step(dt, check=False)
+    for _ in range(steps):
+        S.step(dt)
+        graph.replay()
+    torch.cuda.synchronize()
+    G.poll()
+    amax = max(float(S.acc_s.abs().max()), float(S.acc_l.abs().max()))
+    assert (G.vel - S.vel).abs().max() <= 1e-5 * amax * dt * steps
+    assert (G.pos - S.pos).abs().max() <= 1e-5 * amax * dt * dt * steps * steps + 1e-15
+    S.close()
+    G.close()
