@@ -20,9 +20,10 @@
 // their published counts (a tile publishes its own counts first and the sum
 // up to itself once it knows it, so a look-back ends at the nearest sum);
 // then it stages the tile in shared memory in digit order and writes
-// contiguous runs.  Tiles are numbered by a counter as blocks start, so every
-// tile that is looked back at is running or done.  Stability of every pass
-// gives the (key, original index) order.
+// contiguous runs.  (The scheme is the one-pass radix sort of Adinets and Merrill,
+// 2022, on the look-back of Merrill and Garland, 2016.)  Tiles are numbered by a
+// counter as blocks start, so every tile that is looked back at is running or
+// done.  Stability of every pass gives the (key, original index) order.
 //
 // Bound by HBM: 220 B a key (32 for the keys, 20 for the first pass, whose
 // values are the indices themselves, 24 for each other pass), against 310 B and 25
@@ -87,7 +88,6 @@ __device__ __forceinline__ uint64_t hilbert63(uint32_t a, uint32_t b, uint32_t c
 
 constexpr int kKeyThreads = 256;
 
-// Key of one position; 0 and the status flag for a non-finite one.
 // The same index three levels at a time.  What the levels above leave behind
 // is one of 24 states: which axis each of the three is exchanged with, which
 // are inverted, and the parity.  e[512 s + (a, b, c)], three bits of each axis, is
@@ -167,6 +167,7 @@ __device__ __forceinline__ uint64_t hilbert63(const uint16_t* __restrict__ table
   return key;
 }
 
+// Key of one position; 0 and the status flag for a non-finite one.
 template <bool TABLE>
 __device__ __forceinline__ uint64_t position_key(const double* __restrict__ pos, int64_t i, const BoxScale& B,
                                                  const uint16_t* table, StatusBlock* sb) {
@@ -215,15 +216,16 @@ __global__ void __launch_bounds__(kKeyThreads) k_keys(const double* __restrict__
 // A tile's published state for one digit: 0 nothing yet, 1 + count its own
 // count, kStateSum | sum the keys of the digit in all tiles up to it.  One
 // word that other blocks poll while it is written, hence relaxed accesses of
-// device scope; nothing else is read on the strength of it.
+// device scope (volatile, so that a tile publishes before it polls); nothing else is
+// read on the strength of it.
 constexpr uint32_t kStateSum = 1u << 31;
 __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
   uint32_t v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
 __device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
-  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v));
 }
 // Polls of one state before a look-back gives up (seconds, far above any
 // tile's run time; the tiles looked at are always running).

@@ -27,7 +27,7 @@
 //                  at the 8 CIC nodes, summed with the deposit's weights.
 //
 // The mesh force is never stored: each particle differentiates the potential
-// at its own 8 nodes (72 loads of an L2-resident mesh instead of three more
+// at its own 8 nodes (56 loads of an L2-resident mesh instead of three more
 // N^3 meshes in HBM).  Positions are FP64 until the CIC fraction, which is
 // rounded to FP32 once, as in the deposit.
 #include <cufft.h>

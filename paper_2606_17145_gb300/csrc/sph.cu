@@ -36,18 +36,18 @@
 //      corrected by the neighbours within 4e-4 h of it (their distances are
 //      kept, up to two; with more, or a larger step, the pass is repeated at
 //      the new h).
-// Two kernels: the passes need 63 registers and 7 KB of shared memory a warp,
-// the finishing pass 112 and 13 KB; in one kernel the passes ran at the
-// finishing pass's 16 warps an SM.
+// Two kernels: the passes need 63 registers and 6.0 KB of shared memory a warp,
+// the finishing pass 95 and 12.1 KB (17 warps an SM); in one kernel, of 126
+// registers, the passes ran at 16 warps an SM.
 //
 // Measured, ms (one target per lane against every staged particle, Newton
 // steps until 1e-2, one kernel of two warps a block -> now): 128^3 clustered
 // N_ngb 32 24.9 -> 10.9; 128^3 lattice 5.05 -> 3.7; 4096 uniform 0.33 -> 0.20; 100,003
 // uniform, N_ngb 64 0.73 -> 0.69.  By part on the clustered set: tiles 24.8 -> 19.8,
 // two kernels 16.8, one warp a block 15.3, third-order steps 14.2, conversions on
-// the integer pipe 13.6, groups by estimated work 10.9.  k_sph_radius issues on 73 %
-// of its cycles; k_sph_density (47 %) waits for latencies at 16 - 18 warps an SM
-// and keeps the FP64 pipe 36 % busy.
+// the integer pipe 13.6, groups by estimated work 10.9.  On a 90^3 clustered set
+// k_sph_radius issues on 74 % of its cycles; k_sph_density (58 %) waits for
+// latencies at 15 of 17 warps an SM and keeps the FP64 pipe 32 % busy.
 // Every loop is bounded (node-visit cap, pass caps, the stack bound); a
 // particle whose h does not converge below half the box gets NaN / -1 and
 // sets a status bit.
@@ -528,8 +528,9 @@ struct SphEval32 {
 // tiles) go to their targets' lists; before a list can overflow all are
 // flushed, i.e. every lane evaluates its target's candidates in float-float and
 // adds w to FP64 sums (sum w, sum m w, which set h and rho to ~1e-12); the
-// derivatives, which scale a step below 3e-6 h, are FP32 sums of the same
-// neighbours.
+// derivatives, which scale the step from here (about 6e-5 of h after the FP32
+// passes, 3e-4 at most), are FP32 sums of the same neighbours: a relative error of
+// 1e-7 in them is 3e-11 of h at the largest step.
 struct SphEval64 {
   const SphArgs* A;
   const SphBufs* W;
@@ -820,7 +821,7 @@ __global__ void __launch_bounds__(kSphWarps * 32) k_sph_radius(SphArgs A) {
 }
 
 // Finishing pass(es): second-order step, density and neighbour count.
-__global__ void __launch_bounds__(kSphWarps * 32, 18) k_sph_density(SphArgs A) {
+__global__ void __launch_bounds__(kSphWarps * 32, 17) k_sph_density(SphArgs A) {
   __shared__ SphWarp s_warp[kSphWarps];
   __shared__ int s_list[kSphWarps][kSphList][32];
   const TreeDev& T = A.T;

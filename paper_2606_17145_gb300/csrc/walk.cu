@@ -896,7 +896,7 @@ struct LaneFP {
 
   // The tiles add every listed pair, those that are no hits with a factor of
   // zero, which clears the term only while its operands are finite: dL/da up to
-  // kWildWeight (a sum of three products with displacements below 0.87) and
+  // kWildWeight (three products with displacements below 1 stay below FLT_MAX) and
   // masses that do not overflow FP32.  A warp with others evaluates its batches
   // here, hit by hit: lane = target, slot after slot.
   static constexpr float kWildWeight = 1e38f;
@@ -1596,15 +1596,16 @@ __device__ __forceinline__ void walk_block(const WalkArgs& A) {
     if (wild) walk_wild<Lane, kWarpsPerBlock>(A, S);
 }
 
-// Forward walks of many groups run 18 to 20 warps an SM, in blocks of one (96
-// registers); the others 16, in blocks of two, whose groups are neighbours and
-// share their sources in L1.  Forward, ms, before / after: lattice 128^3 2.55 / 2.48,
-// clustered 128^3 17.1 / 16.5, 256^3 405 / 387, 90^3 (22,782 groups) 3.59 / 3.58;
-// 5860 groups (zoom) 12.4 / 13.1, 128 groups 0.221 / 0.240.  Adjoint 128^3 clustered
-// 22.8 / 24.2: its code fits the instruction cache less well.  The FP64 walk, which
-// shares little in L1 for its arithmetic, runs 16 in blocks of one: a block of
-// two lasts as long as its longer group.  64^3 lattice 1.90 -> 1.81 ms, clustered 58^3
-// 5.3 -> 5.0, 64^3 6.5 -> 6.35; zoom 68.6 -> 69.2 (18 warps: 1.74, 5.0, 6.6 and 66.4).
+// Forward walks of many groups run 18 warps an SM, in blocks of one (96
+// registers); the others 16, in blocks of two (118 to 128 registers), whose groups
+// are neighbours and share their sources in L1.  Forward, ms, blocks of two / one:
+// lattice 128^3 2.55 / 2.36, clustered 128^3 17.1 / 15.7, 256^3 405 / 368, 90^3 (22,782
+// groups) 3.61 / 3.43; 5860 groups (zoom) 12.7 / 12.4, 128 groups 0.217 / 0.233.  Adjoint
+// 128^3 clustered 22.8 / 24.2: its code fits the instruction cache less well.  The
+// FP64 walk, which shares little in L1 for its arithmetic, runs 15 in blocks of
+// one (shared memory, 14 KB a warp and 1 KB a block): of two groups in a block one
+// waits for the other.  16 in blocks of two / 15 in blocks of one: 64^3 lattice
+// 1.90 / 1.81 ms, clustered 58^3 5.3 / 5.0, 64^3 6.5 / 6.35; zoom 68.6 / 69.2.
 constexpr int64_t kManyGroups = 24576;
 
 template <class Lane>
@@ -1622,12 +1623,13 @@ __global__ void __launch_bounds__(32, kBlocks) k_walk_one(WalkArgs A) {
 // traversal, shorten them for some repeated traversal.  It depends on the
 // tree alone, so a walk over a range of groups gives the full walk's sums.
 // Measured, ms with 1 / 2 / 4 warps a group, forward: 128 groups (4096
-// uniform) 0.37 / 0.27 / 0.22, 1024 groups (32^3) clustered 0.31 / 0.26 / 0.23,
-// zoom 3.45 / 2.41 / 2.52, lattice 0.14 / 0.13 / 0.15; 5860 groups (zoom) 12.3 /
-// 13.8 / 17.3; 8192 groups (64^3) lattice 0.41 / 0.48 / 0.63, clustered 1.35 /
-// 1.15 / 1.38.  FP64: 128 groups 1.59 / 0.95 / 0.67, 1024 clustered 1.55 / 1.07 /
-// 0.79, zoom 8.0 / 7.6 / 9.0, lattice 0.39 / 0.36 / 0.43; 5860 (zoom) 68 / 70 / 80,
-// 8192 clustered 6.5 / 5.7 / 6.7, lattice 1.87 / 1.93 / 2.32.
+// uniform) 0.37 / 0.27 / 0.22, 1024 groups (32^3) clustered 0.30 / 0.26 / 0.23,
+// zoom 3.38 / 2.37 / 2.48, lattice 0.15 / 0.13 / 0.15; 5860 groups (zoom) 12.4 /
+// 13.8 / 17.2; 8192 groups (64^3) lattice 0.41 / 0.48 / 0.62, clustered 1.35 /
+// 1.16 / 1.37.  FP64: 128 groups 1.58 / 0.94 / 0.67, 1024 clustered 1.50 / 1.04 /
+// 0.80, zoom 7.5 / 7.1 / 8.7, lattice 0.38 / 0.36 / 0.42; 5860 (zoom) 67.5 / 69.5 /
+// 80.6, 8192 clustered 6.4 / 5.8 / 6.4, lattice 1.81 / 1.90 / 2.27.  Between 1024 and
+// 5860 groups nothing was measured.
 static int walk_split(int64_t n_groups) { return n_groups <= 1024 ? 2 : n_groups <= 4096 ? 1 : 0; }
 
 cudaError_t launch_walk(WalkArgs A, int prec, bool adjoint, cudaStream_t s, bool fused) {
@@ -1638,7 +1640,7 @@ cudaError_t launch_walk(WalkArgs A, int prec, bool adjoint, cudaStream_t s, bool
   const unsigned pairs = (unsigned)((warps + 1) / 2);
   if (fused) k_walk<LaneFused><<<pairs, 64, 0, s>>>(A);
   else if (adjoint) k_walk<LaneF32<true>><<<pairs, 64, 0, s>>>(A);
-  else if (prec == OG_FP64) k_walk_one<LaneF64, 16><<<(unsigned)warps, 32, 0, s>>>(A);
+  else if (prec == OG_FP64) k_walk_one<LaneF64, 15><<<(unsigned)warps, 32, 0, s>>>(A);
   else if (A.T.ngroups >= kManyGroups) k_walk_one<LaneF32<false>, 18><<<(unsigned)warps, 32, 0, s>>>(A);
   else k_walk<LaneF32<false>><<<pairs, 64, 0, s>>>(A);
   return cudaGetLastError();
