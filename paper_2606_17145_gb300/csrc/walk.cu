@@ -977,11 +977,6 @@ struct LaneFP {
   // 27.3 against 25.3 ms with both directions in one walk).
   __device__ void batch_tiles(const WalkArgs& A, const WarpBufs& W, Stage& St, Smem& M, const float4* SGB,
                               int cnt, int lane, int64_t gbase, uint32_t vmask, bool mi) {
-    // an odd count leaves the last pair's second slot empty: its data must be finite
-    if ((cnt & 1) && lane < 8) {
-      float4* p = lane < 2 ? &St.s0[cnt >> 1] : lane < 4 ? &St.s1[cnt >> 1] : lane < 6 ? &St.s2[cnt >> 1] : &St.s3[cnt >> 1];
-      (&p->x)[2 * (lane & 1) + 1] = 0.f;
-    }
     const uint2 qq = *reinterpret_cast<const uint2*>(St.sq + 2 * lane);
     const bool has0 = 2 * lane < cnt, has1 = 2 * lane + 1 < cnt;
     const uint32_t q0 = has0 ? qq.x : 0u, q1 = has1 ? qq.y : 0u;
@@ -1026,6 +1021,12 @@ struct LaneFP {
       const uint32_t others = ~(1u << (so >> 1));
       if (so & 1) m1 &= others;
       else m0 &= others;
+    }
+    __syncwarp();  // every lane has read its slot pair
+    // an odd count leaves the last pair's second slot empty: its data must be finite
+    if ((cnt & 1) && lane < 8) {
+      float4* p = lane < 2 ? &St.s0[cnt >> 1] : lane < 4 ? &St.s1[cnt >> 1] : lane < 6 ? &St.s2[cnt >> 1] : &St.s3[cnt >> 1];
+      (&p->x)[2 * (lane & 1) + 1] = 0.f;
     }
     __syncwarp();
 #pragma unroll 1
